@@ -521,7 +521,7 @@ st_status st_sort_keys_static_status(void* stream);
 
 /* Kernel timers: CUDA events recorded around the library's own launches, on the stream each runs
  * on, summed per kind.  ST_TIMER_STEP: every particle step kernel (st_step, the adjoint's forward
- * steps and recomputation); ST_TIMER_SORT: a whole reorder (all of its kernels);
+ * steps and recomputation; a launch that takes several steps counts as that many); ST_TIMER_SORT: a whole reorder (all of its kernels);
  * ST_TIMER_ADJOINT: the adjoint step kernel of st_adjoint_backward; ST_TIMER_FLUID: the coupled
  * fluid update of st_couple_run.  st_timers_enable(h, 1) clears and starts
  * recording, 0 stops it.  st_timers_read synchronises, writes the summed milliseconds and the

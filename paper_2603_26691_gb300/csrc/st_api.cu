@@ -75,6 +75,8 @@ st_status st::check_flags(st_ctx* h) {
   if (e != cudaSuccess) return cuda_check(h, e, "read error flags");
   if (f != 0) {
     cudaMemsetAsync(h->flags.p, 0, sizeof(int), h->stream);
+    // a CTA that gave up left the sorted-step kernel's counters as they were
+    cudaMemsetAsync((char*)h->flags.p + kUnitCounterOffset, 0, 2 * sizeof(unsigned), h->stream);
     return set_error(h, ST_ERR_TIMEOUT, "a bounded device-side wait gave up (flags " + std::to_string(f) + ")");
   }
   return ST_OK;
@@ -234,14 +236,15 @@ void timer_begin(st_ctx* h, int k, cudaStream_t s) {
   cudaEvent_t e = timer_event(h);
   if (!e) return;
   cudaEventRecord(e, s);
-  h->ev_pending[k].push_back({e, nullptr});
+  h->ev_pending[k].push_back({e, nullptr, 1});
 }
-void timer_end(st_ctx* h, int k, cudaStream_t s) {
+void timer_end(st_ctx* h, int k, cudaStream_t s, int count) {
   if (!h->timing || h->ev_pending[k].empty() || h->ev_pending[k].back().second) return;
   cudaEvent_t e = timer_event(h);
   if (!e) return;
   cudaEventRecord(e, s);
   h->ev_pending[k].back().second = e;
+  h->ev_pending[k].back().count = count;
 }
 static cudaError_t timers_fold(st_ctx* h) {
   for (int k = 0; k < ST_TIMER_COUNT; ++k) {
@@ -253,7 +256,7 @@ static cudaError_t timers_fold(st_ctx* h) {
         e = cudaEventElapsedTime(&ms, pr.first, pr.second);
         if (e != cudaSuccess) return e;
         h->timer_ms[k] += ms;
-        h->timer_count[k] += 1;
+        h->timer_count[k] += pr.count;
         h->ev_pool.push_back(pr.second);
       }
       h->ev_pool.push_back(pr.first);
@@ -512,7 +515,8 @@ static double deposits_per_cell(const st_ctx* h) {
 
 // Choose the fixed-point exponent so that a committed run at its bound maps to
 // at most 2^96 and the accumulated integer stays below 2^125.
-static st_status prepare_accumulator(st_handle h, double dt, double adds_now, int* E_out) {
+// For a launch of nsteps steps; digits: what it can add to one word (far: see launch_acc_maybe_normalize).
+static st_status prepare_accumulator(st_handle h, double dt, int nsteps, double digits, bool far, int* E_out) {
   const double pi = 3.14159265358979323846;
   double gn = std::sqrt(h->g[0] * h->g[0] + h->g[1] * h->g[1] + h->g[2] * h->g[2]);
   double tau_max = h->rho_p * h->dmax * h->dmax / (18.0 * h->mu);
@@ -531,7 +535,8 @@ static st_status prepare_accumulator(st_handle h, double dt, double adds_now, in
   if (h->acc_empty || E < h->acc_E) h->acc_E = E;
   E = h->acc_E;
   // one step adds at most np * jb to any cell
-  double add = (double)h->np * jb * std::ldexp(1.0, E) + 1.0;
+  const double parts = (double)h->np * nsteps;
+  double add = parts * jb * std::ldexp(1.0, E) + 1.0;
   while (h->acc_load + add > 0x1p125) {
     cudaError_t e = launch_rescale_acc(h, 1);
     ST_TRY(cuda_check(h, e, "rescale accumulator"));
@@ -539,14 +544,11 @@ static st_status prepare_accumulator(st_handle h, double dt, double adds_now, in
     h->acc_E -= 1;
     E = h->acc_E;
     h->acc_load *= 0.5;
-    add = (double)h->np * jb * std::ldexp(1.0, E) + 1.0;
+    add = parts * jb * std::ldexp(1.0, E) + 1.0;
   }
   h->acc_load += add;
   h->acc_empty = false;
-  // each word takes at most one digit per contribution; a step adds at most one contribution per
-  // particle to any cell, plus one per neighbouring unit's tile flush (at most 8)
-  ST_TRY(cuda_check(h, launch_acc_maybe_normalize(h, deposits_per_cell(h) * (double)h->np + 8.0, adds_now),
-                    "normalise accumulator"));
+  ST_TRY(cuda_check(h, launch_acc_maybe_normalize(h, digits, far), "normalise accumulator"));
   *E_out = E;
   return ST_OK;
 }
@@ -563,24 +565,37 @@ st_status run_steps(st_ctx* h, int nsteps, double dt) {
   if (h->micro_on && !default_physics(h))
     return set_error(h, ST_ERR_STATE, "microphysics runs with the default gather, integrator, drag and deposit only");
   const double pi = 3.14159265358979323846;
-  for (int s = 0; s < nsteps; ++s) {
+  for (int s = 0; s < nsteps;) {
     if (h->np == 0) break;
     if (h->reorder_every > 0 && (!h->sorted || h->steps_since_sort >= h->reorder_every)) ST_TRY(st_reorder(h));
-    // the sorted-step kernel adds one tile flush per covering unit (at most 8 per cell) and counts
-    // its global commits itself; the other kernels may add one contribution per particle
     const bool tma = !h->micro_on && h->prec != ST_FP64 && h->sorted && tma_step_supported(h);
-    // a sort is due before the next step: this step writes the state as records for its gather
-    const bool records = tma && default_physics(h) && h->reorder_every > 0 &&
-                         h->steps_since_sort + 1 >= h->reorder_every && h->state_alt.bytes >= (size_t)h->cap * 32;
-    // a sort that deferred its payload gather: this step gathers, unless it is another kernel or
-    // writes records itself (then the gather runs first)
-    const bool gather = h->perm_pending && tma && default_physics(h) && !records;
+    // the field is frozen and particles do not act on each other, so a launch takes several steps where
+    // its kernel can, up to the next sort
+    int m = 1;
+    if (tma) m = std::min(nsteps - s, kMaxFusedSteps);
+    if (h->reorder_every > 0) m = std::min(m, h->reorder_every - h->steps_since_sort);
+    // a sort is due after these steps: they leave the state as records for its gather
+    const bool can_record = tma && default_physics(h) && h->reorder_every > 0 && h->state_alt.bytes >= (size_t)h->cap * 32;
+    bool records = can_record && h->steps_since_sort + m >= h->reorder_every;
+    // a sort that deferred its payload gather: these steps gather, unless it is another kernel; the records
+    // they read are where new ones would go, so the last step before a sort is then a launch of its own
+    // (a single step has the gather run first)
+    const bool gather = h->perm_pending && tma && default_physics(h) && !(records && m == 1);
+    if (gather && records) {
+      records = false;
+      m -= 1;
+    }
     if (!gather) ST_TRY(materialize_state(h));
     if (h->micro_on) ST_TRY(micro_prepare_step(h, dt));
     int E = 0;
-    ST_TRY(prepare_accumulator(h, dt, tma ? 8.0 : deposits_per_cell(h) * (double)h->np + 8.0, &E));
+    // digits a launch can add to one word: a tile flush of each of the (at most 8) units that cover a cell,
+    // at least one unit in 2^16 particle-steps; the other kernels one contribution per particle
+    ST_TRY(prepare_accumulator(h, dt, m,
+                               tma ? 8.0 * ((double)h->np * m / 65536.0 + 2.0) : deposits_per_cell(h) * (double)h->np + 8.0,
+                               tma, &E));
     StepParams p;
     p.dt = dt;
+    p.nsteps = m;
     p.ca = 18.0 * h->mu * h->alpha / h->rho_p;
     p.mcoef = h->mult * h->rho_p * pi / 6.0;
     for (int q = 0; q < 3; ++q) p.g[q] = h->g[q];
@@ -609,9 +624,10 @@ st_status run_steps(st_ctx* h, int nsteps, double dt) {
     }
     else
       e = launch_step_mixed(h, p);
-    timer_end(h, ST_TIMER_STEP, h->stream);
+    timer_end(h, ST_TIMER_STEP, h->stream, m);
     ST_TRY(cuda_check(h, e, "step kernel"));
-    h->steps_since_sort += 1;
+    h->steps_since_sort += m;
+    s += m;
   }
   return ST_OK;
 }
@@ -950,7 +966,7 @@ st_status st_adjoint_forward(st_handle h, int nsteps, double dt, int checkpoint_
       ST_TRY(cuda_check(h, e, "checkpoint"));
     }
     int E = 0;
-    ST_TRY(prepare_accumulator(h, dt, (double)h->np + 8.0, &E));
+    ST_TRY(prepare_accumulator(h, dt, 1, deposits_per_cell(h) * (double)h->np + 8.0, false, &E));
     StepParams p;
     p.dt = dt;
     p.ca = 18.0 * h->mu * h->alpha / h->rho_p;

@@ -17,6 +17,7 @@ namespace st {
 constexpr int kMaxDim = 1024;       // cells per axis (10-bit fields of the packed cell)
 constexpr int kAccBits = 96;        // a contribution at its bound maps to 2^96 in the accumulator
 constexpr int kMaxRun = 128;        // particles folded into one committed run (warp x 4)
+constexpr int kMaxFusedSteps = 32;  // steps one launch takes at most
 constexpr int kFluidPad = 3;        // ghost layers around the mixed-precision field
 
 // Owned device allocation.
@@ -100,7 +101,11 @@ struct st_ctx {
   // kernel timers (st_timers_*): pending event pairs per kind, folded into sums on read
   bool timing = false;
   std::vector<cudaEvent_t> ev_pool;
-  std::vector<std::pair<cudaEvent_t, cudaEvent_t>> ev_pending[ST_TIMER_COUNT];
+  struct TimerMark {
+    cudaEvent_t first, second;
+    int count;
+  };
+  std::vector<TimerMark> ev_pending[ST_TIMER_COUNT];
   double timer_ms[ST_TIMER_COUNT] = {0, 0, 0, 0};
   int64_t timer_count[ST_TIMER_COUNT] = {0, 0, 0, 0};
 
@@ -109,6 +114,9 @@ struct st_ctx {
   int acc_E = 0;             // value = integer * 2^-acc_E
   bool acc_empty = true;
   double acc_load = 0.0;     // bound on |accumulated integer| (in units of 1), for overflow control
+  double acc_adds = 0.0;     // digits added to any word since the last carry propagation
+  bool acc_far = false;      // the sorted-step kernel ran since then: its own bound of 2^60 beside the digits
+  bool acc_on_device = false;  // steps were captured in a graph: the count lives on the device
 
   st::Buf red;               // small reduction scratch
   st::Buf flags;             // device error flags (bounded waits that gave up)
@@ -373,6 +381,7 @@ struct StepParams {
   double g[3];
   double scale;    // 2^E for the FP64 path
   int E;           // for the FP32 path
+  int nsteps = 1;  // steps the launch takes
   // physics variants (nonzero = nearest grid point, semi-implicit Euler, Schiller-Naumann,
   // cloud-in-cell deposit) and rho_f / mu for the particle Reynolds number
   int ngp = 0, semi = 0, sn = 0, cic = 0;
@@ -566,17 +575,17 @@ cudaError_t launch_rescale_acc(st_ctx* h, int shift);
 cudaError_t launch_normalize_acc(st_ctx* h);
 // the particle steps of st_step (sort when due, accumulator bookkeeping, step kernel)
 st_status run_steps(st_ctx* h, int nsteps, double dt);
-// word-capacity bookkeeping of the carry-save accumulator, on the device: a counter (in the flags
-// buffer) bounds the digits added to any word since the last carry propagation; before each step
-// the propagation runs if the counter plus the step's worst case could overflow a word.  `add` is
-// what the step adds for sure (its flushes, or its worst case when it does not count itself);
-// kernels that add more (global commits of the sorted-step kernel) count them on the device.
-cudaError_t launch_acc_maybe_normalize(st_ctx* h, double worst, double add);
+// word-capacity bookkeeping of the carry-save accumulator: the host counts the digits that launches can
+// have added to any word since the last carry propagation, and runs the propagation before a launch
+// that could overflow one (`add`: the launch's worst case).  far: the sorted-step kernel, whose commits
+// outside its tiles keep themselves below 2^60 and are not counted.  In a captured graph the count and
+// the decision are kernels (a replay adds to the words without the host), and they stay so for the handle.
+cudaError_t launch_acc_maybe_normalize(st_ctx* h, double add, bool far);
 cudaError_t reset_acc_counter(st_ctx* h);
 constexpr size_t kAccCounterOffset = 64;   // bytes into the flags buffer: uint64 counter
 constexpr size_t kAccFlagOffset = 72;      // int: 1 if the last check propagated carries
-constexpr size_t kUnitCounterOffset = 80;  // uint32: next unit of the sorted-step kernel
 constexpr size_t kFarFlagOffset = 84;      // int: the neighbourhood sort found a particle it cannot place
+constexpr size_t kUnitCounterOffset = 88;  // uint32[2]: the sorted-step kernel's next unit and finished CTAs
 cudaError_t launch_acc_to_f64(st_ctx* h, double* out, int E);
 cudaError_t launch_acc_sum(st_ctx* h, double out[3]);
 cudaError_t launch_particle_sums(st_ctx* h, double out[4]);  // P_x, P_y, P_z, M
@@ -616,9 +625,9 @@ void gather_step_done(st_ctx* h);                                          // so
 // FP64 and FP32 FMA rates of this GPU (GFLOP/s), measured by FMA-chain kernels; synchronises
 cudaError_t probe_fma_rates(st_ctx* h, double* fp64_gflops, double* fp32_gflops);  // util.cu
 // timer marks around a launch of kind k on stream s (no-ops unless st_timers_enable is on); the
-// end mark pairs with the last begin of the same kind
+// end mark pairs with the last begin of the same kind and counts `count` (the steps a launch takes)
 void timer_begin(st_ctx* h, int k, cudaStream_t s);                        // st_api.cu
-void timer_end(st_ctx* h, int k, cudaStream_t s);                          // st_api.cu
+void timer_end(st_ctx* h, int k, cudaStream_t s, int count = 1);           // st_api.cu
 cudaError_t launch_cell_counts(st_ctx* h, int64_t* counts);
 // ---- droplet microphysics (micro.cu) -------------------------------------------------------------
 // the step with vapour mass and heat transfer (default physics only; accumulators prepared)

@@ -680,7 +680,7 @@ st_status st_get_sources_fixed(st_handle h, int64_t* words, int* E, int on_devic
 st_status st_get_particles(st_handle h, int64_t first, int64_t count, double* xyz, double* vel, double* d,
                            uint32_t* ids, int on_device) {
   ST_TRY(check_handle(h));
-  ST_TRY(materialize_state(h));
+  if (h->perm_pending) ST_TRY(materialize_state(h));  // records of the storage order are read as they are
   if (first < 0 || count < 0 || first + count > h->np) return set_error(h, ST_ERR_INVALID_ARG, "range out of bounds");
   if (count == 0) return ST_OK;
   Buf tx, tv, td, ti;
@@ -716,7 +716,7 @@ st_status st_get_particles(st_handle h, int64_t first, int64_t count, double* xy
 
 st_status st_get_cells(st_handle h, int64_t first, int64_t count, int32_t* cells, int on_device) {
   ST_TRY(check_handle(h));
-  ST_TRY(materialize_state(h));
+  if (h->perm_pending) ST_TRY(materialize_state(h));
   if (!cells) return set_error(h, ST_ERR_INVALID_ARG, "cells is NULL");
   if (first < 0 || count < 0 || first + count > h->np) return set_error(h, ST_ERR_INVALID_ARG, "range out of bounds");
   if (count == 0) return ST_OK;

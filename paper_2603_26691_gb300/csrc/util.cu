@@ -6,6 +6,7 @@
 #include <vector>
 
 #include "st_common.cuh"
+#include "st_ptx.cuh"
 
 namespace st {
 
@@ -180,22 +181,66 @@ __global__ void export_f64_kernel(F64State s, const uint32_t* __restrict__ sid, 
   }
 }
 
-// ms (microphysics on): per particle {T_hi, T_lo, d_lo, 0}; the diameter is d + d_lo
-__global__ void export_mixed_kernel(MixedState s, bool bf16, const uint32_t* __restrict__ sid, int64_t first,
-                                    int64_t n, double* xyz, double* vel, double* d, uint32_t* ids, int32_t* cells,
-                                    GeoArgs g, const float4* __restrict__ ms) {
+// FP32 to FP64 with integer operations: GB300 converts on its FP64 pipe, one warp in 64 cycles, and an export
+// has ten such values per particle.  Subnormal and non-finite values (rare) take the conversion.
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t b = __float_as_uint(x), e = b & 0x7f800000u;
+  if (__builtin_expect(e == 0 || e == 0x7f800000u, 0)) return (b << 1) == 0 ? __hiloint2double((int)b, 0) : (double)x;
+  return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
+}
+
+// i + xi for a cell index 0 <= i < 1024 and an offset 0 <= xi < 1.  Offsets of at least 2^-20 (or 0) make it a
+// multiple of 2^-43 below 2^10, so the sum is exact: the 53-bit integer, normalised.  (Smaller ones
+// round in FP64.)
+__device__ __forceinline__ double cell_position(int i, float xi) {
+  const uint32_t b = __float_as_uint(xi);
+  const int e = (int)(b >> 23);
+  if (__builtin_expect((unsigned)(e - 107) > 19u && b != 0, 0)) return (double)i + (double)xi;
+  const unsigned long long f = b == 0 ? 0ull : (unsigned long long)((b & 0x7fffffu) | 0x800000u) << (e - 107);
+  const unsigned long long n = ((unsigned long long)i << 43) | f;
+  if (n == 0) return 0.0;
+  const int lz = __clzll((long long)n);  // 11 .. 63
+  return __longlong_as_double((long long)(((n << (lz - 11)) & 0xfffffffffffffull) |
+                                          ((unsigned long long)(1043 - lz) << 52)));
+}
+
+// The mixed state as FP64.  ms (microphysics on): per particle {T_hi, T_lo, d_lo, 0}; the diameter is d + d_lo.
+// RECORDS: the state as the step before a sort left it, 32-byte records (rec) in storage order; the
+// structure of arrays is then neither read nor brought up to date, and the sort still gathers from the
+// records.  5e8 particles on 256^3, an exchange of ten steps: 9.0 ms outside the steps and the sort, against
+// 24.5 ms through the arrays with conversions on the FP64 pipe, and the next sort takes 4.7 instead of 14.5 ms.
+template <bool RECORDS>
+__global__ void export_mixed_kernel(MixedState s, const float4* __restrict__ rec, bool bf16,
+                                    const uint32_t* __restrict__ sid, int64_t first, int64_t n, double* xyz, double* vel,
+                                    double* d, uint32_t* ids, int32_t* cells, GeoArgs g, const float4* __restrict__ ms) {
   for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x) {
-    int64_t sp = first + p;
-    int32_t c = s.cell[sp];
-    int idx[3] = {cell_i(c), cell_j(c), cell_k(c)};
-    for (int q = 0; q < 3; ++q) {
-      if (xyz) xyz[q * n + p] = ((double)idx[q] + (double)s.xi[q][sp]) * g.h[q];
-      if (vel) {
-        double v = bf16 ? (double)__bfloat162float(((const __nv_bfloat16*)s.v[q])[sp]) : (double)((const float*)s.v[q])[sp];
-        vel[q * n + p] = v;
+    const int64_t sp = first + p;
+    int32_t c;
+    float xi[3], v[3], dp;
+    if (RECORDS) {
+      const ptx::Rec32 r = ptx::ld_rec32(rec + 2 * sp);
+      c = __float_as_int(r.c);
+      xi[0] = r.x0;
+      xi[1] = r.x1;
+      xi[2] = r.x2;
+      v[0] = r.v0;
+      v[1] = r.v1;
+      v[2] = r.v2;
+      dp = r.d;
+    } else {
+      c = s.cell[sp];
+      for (int q = 0; q < 3; ++q) {
+        if (xyz) xi[q] = s.xi[q][sp];
+        if (vel) v[q] = bf16 ? __bfloat162float(((const __nv_bfloat16*)s.v[q])[sp]) : ((const float*)s.v[q])[sp];
       }
+      if (d) dp = s.d[sp];
     }
-    if (d) d[p] = (double)s.d[sp] + (ms ? (double)ms[sp].z : 0.0);
+    const int idx[3] = {cell_i(c), cell_j(c), cell_k(c)};
+    for (int q = 0; q < 3; ++q) {
+      if (xyz) xyz[q * n + p] = cell_position(idx[q], xi[q]) * g.h[q];
+      if (vel) vel[q * n + p] = widen(v[q]);
+    }
+    if (d) d[p] = ms ? (double)dp + (double)ms[sp].z : widen(dp);
     if (ids) ids[p] = sid[sp];
     if (cells) cells[p] = idx[0] + g.n[0] * (idx[1] + g.n[1] * idx[2]);
   }
@@ -479,10 +524,11 @@ cudaError_t launch_export(st_ctx* h, int64_t first, int64_t n, double* xyz, doub
     export_f64_kernel<<<grid_for(n), kThreads, 0, h->stream>>>(carve_f64(h->state.p, h->cap), (const uint32_t*)h->ids.p,
                                                                first, n, xyz, vel, d, ids, cells, g);
   } else {
-    bool bf = h->prec == ST_MIXED_BF16V;
-    export_mixed_kernel<<<grid_for(n), kThreads, 0, h->stream>>>(carve_mixed(h->state.p, h->cap, bf), bf,
-                                                                 (const uint32_t*)h->ids.p, first, n, xyz, vel, d,
-                                                                 ids, cells, g, (const float4*)h->temp.p);
+    const bool bf = h->prec == ST_MIXED_BF16V;
+    const bool rec = h->records_pending && !h->perm_pending;
+    (rec ? export_mixed_kernel<true> : export_mixed_kernel<false>)<<<grid_for(n), kThreads, 0, h->stream>>>(
+        carve_mixed(h->state.p, h->cap, bf), rec ? (const float4*)h->state_alt.p : nullptr, bf,
+        (const uint32_t*)h->ids.p, first, n, xyz, vel, d, ids, cells, g, (const float4*)h->temp.p);
   }
   h->launches += 1;
   return cudaGetLastError();

@@ -160,6 +160,11 @@ st_status couple_resources(st_ctx* h) {
   if (mixed(h)) {
     if (h->fl_cur.bytes < fb) ST_TRY(dev_alloc(h, h->fl_cur, fb));
     if (h->fluid_pad_next.bytes < h->fluid_pad.bytes) ST_TRY(dev_alloc(h, h->fluid_pad_next, h->fluid_pad.bytes));
+  } else if (h->fluid_fix_next.bytes < h->fluid_fix.bytes) {
+    if (dev_alloc(h, h->fluid_fix_next, h->fluid_fix.bytes) != ST_OK) {
+      dev_free(h, h->fluid_fix);  // no room for two: the steps then read the FP64 field
+      h->err.clear();
+    }
   }
   if (h->umax_dev.bytes < 8) ST_TRY(dev_alloc(h, h->umax_dev, 8));
   if (!h->umax_host) ST_CUDA(h, cudaMallocHost((void**)&h->umax_host, sizeof(double)));
@@ -225,6 +230,8 @@ cudaError_t launch_fluid_update(st_ctx* h, const V* cur, double dt) {
     pad_kernel<<<grid, 128, 0, s>>>((const float4*)h->fl_next.p, (float4*)h->fluid_pad_next.p, G.n[0], G.n[1],
                                     G.n[2], kFluidPad);
     ++launches;
+  } else if (h->fluid_fix.p) {
+    launch_fix_field(h, (const D4*)h->fl_next.p, h->fluid_fix_next.p);
   }
   cudaMemsetAsync(h->umax_dev.p, 0, 8, s);
   field_maxabs_kernel<V><<<cgrid(nc), kCoupleThreads, 0, s>>>((const V*)h->fl_next.p, nc,
@@ -289,6 +296,7 @@ st_status st_couple_run(st_handle h, int nintervals, double dt) {
       std::swap(h->fluid_pad, h->fluid_pad_next);
     } else {
       std::swap(h->fluid, h->fl_next);
+      std::swap(h->fluid_fix, h->fluid_fix_next);
     }
     h->couple_done += 1;
     h->adj_ready = false;

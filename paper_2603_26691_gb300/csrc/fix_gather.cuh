@@ -1,0 +1,180 @@
+// FP64 trilinear interpolation on the integer pipe.
+//
+// GB300 issues one FP64 instruction per warp and scheduler in 64 cycles, and integer instructions in one or
+// two, so an FP64 kernel pays for its FP64 instructions and little else.  The field is therefore also kept as
+// integers (FixCell, 32 bytes per cell, exact): each component a signed 59-bit mantissa of two 29-bit limbs
+// beside a biased exponent counted in units of 3 bits, so that most stencils share one exponent per component.
+// The eight weights are 58-bit integers built with five multiplications (differences of products, so that
+// they add up to one exactly), each component's sum is sixteen products of limbs with 64-bit accumulation, and
+// the result is rounded to FP64 once.  Corners of smaller exponents are shifted to the largest one: what they
+// lose lies below 2^-55 of the largest corner, where an FP64 interpolation rounds at 2^-53 three times.
+#pragma once
+
+#include "st_common.cuh"
+
+namespace st {
+namespace fix {
+
+constexpr int kLimb = 29;
+constexpr int kFrac = 58;                              // weights: 2^58 = 1
+constexpr int64_t kOne = int64_t(1) << kFrac;
+constexpr int64_t kLimbMask = (int64_t(1) << kLimb) - 1;
+constexpr int kExpBias = 6 + 1075;                     // a mantissa of exponent e counts 2^(3 e - kExpBias)
+
+// one cell: a = {x high, x low, y high, y low}, b = {z high, z low, three 10-bit exponents, 0}
+struct alignas(32) FixCell {
+  int4 a, b;
+};
+
+// v = mantissa * 2^(3 e - kExpBias), exact: the FP64 significand shifted by 3 to 5 bits
+__device__ __forceinline__ int64_t split(double v, int& e) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  int be = (int)((b >> 52) & 0x7ff);
+  int64_t man = (int64_t)(b & 0xfffffffffffffull);
+  if (be != 0) man |= int64_t(1) << 52;
+  else be = 1;
+  e = man == 0 ? 0 : be / 3 + 1;
+  if (man) man <<= 6 - (3 * e - be);
+  return (b >> 63) ? -man : man;
+}
+__device__ __forceinline__ FixCell make_cell(double x, double y, double z) {
+  int ex, ey, ez;
+  const int64_t mx = split(x, ex), my = split(y, ey), mz = split(z, ez);
+  FixCell c;
+  c.a = make_int4((int)(mx >> kLimb), (int)(mx & kLimbMask), (int)(my >> kLimb), (int)(my & kLimbMask));
+  c.b = make_int4((int)(mz >> kLimb), (int)(mz & kLimbMask), ex | (ey << 10) | (ez << 20), 0);
+  return c;
+}
+__device__ __forceinline__ FixCell load_cell(const FixCell* p) {
+  FixCell c;
+  c.a = __ldg(&p->a);
+  c.b = __ldg(&p->b);
+  return c;
+}
+
+// floor(s 2^53) for 0 <= s <= 1024 (anything else, NaN included: 0)
+__device__ __forceinline__ int64_t to_fixed53(double s) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(s);
+  const int sh = 1033 - (int)(b >> 52);  // negative values have the sign bit up here: sh < 0
+  const unsigned long long m = (b << 11) | 0x8000000000000000ull;
+  return (unsigned)sh > 63u ? 0 : (int64_t)min(m >> sh, 0x7fffffffffffffffull);
+}
+
+// v * 2^ex rounded to FP64
+__device__ __forceinline__ double to_f64(int64_t v, int ex) {
+  if (v == 0) return 0.0;
+  const unsigned long long m = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+  const int lz = __clzll((long long)m);
+  const int be = 1023 + 63 - lz + ex;
+  if (__builtin_expect((unsigned)(be - 1) >= 2045u, 0)) return ldexp((double)v, ex);
+  const unsigned long long t = m << lz;
+  unsigned long long r = ((unsigned long long)(be - 1) << 52) + (t >> 11) + ((t >> 10) & 1ull);
+  r |= v < 0 ? 0x8000000000000000ull : 0ull;
+  return __longlong_as_double((long long)r);
+}
+
+// a b / 2^58 for 0 <= a, b <= 2^58, at most two units low
+__device__ __forceinline__ int64_t mul58(int64_t a, int64_t b) {
+  const int ah = (int)(a >> kLimb), al = (int)(a & kLimbMask), bh = (int)(b >> kLimb), bl = (int)(b & kLimbMask);
+  return (int64_t)ah * bh + (((int64_t)ah * bl + (int64_t)al * bh) >> kLimb);
+}
+
+// the stencil of a position: base and next cell per axis (periodic), fractions of 2^58, containing cell
+struct Stencil {
+  int i0[3], i1[3], c0[3];
+  int64_t f[3];
+};
+__device__ __forceinline__ Stencil stencil(const double (&x)[3], const double (&inv_h)[3], const int (&n3)[3]) {
+  Stencil st;
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    const int64_t S = to_fixed53(x[q] * inv_h[q]);
+    st.c0[q] = min((int)(S >> 53), n3[q] - 1);
+    const int64_t T = S - (int64_t(1) << 52);  // cell centres lie at halves
+    const int ii = min((int)(T >> 53), n3[q] - 1);
+    st.f[q] = (T & ((int64_t(1) << 53) - 1)) << (kFrac - 53);
+    st.i0[q] = ii < 0 ? ii + n3[q] : ii;
+    st.i1[q] = ii + 1 >= n3[q] ? ii + 1 - n3[q] : ii + 1;
+  }
+  return st;
+}
+
+// the weights of the corners k = dx + 2 dy + 4 dz, none negative; they add up to kOne (a product that would
+// come out a unit or two below zero is left at zero)
+__device__ __forceinline__ void weights(const int64_t (&f)[3], int64_t (&W)[8]) {
+  const int64_t p = mul58(f[0], f[1]);
+  int64_t xy[4] = {kOne - f[0] - f[1] + p, f[0] - p, f[1] - p, p};
+  xy[0] = xy[0] < 0 ? 0 : xy[0];  // mul58 takes no negative factor
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    W[4 + k] = mul58(xy[k], f[2]);
+    W[k] = xy[k] - W[4 + k];
+  }
+}
+
+// mantissas brought to the largest exponent of the eight corners, component by component (word = the corners'
+// exponent words; only called where they differ)
+__device__ __forceinline__ void align(int (&uh)[8], int (&ul)[8], const int (&word)[8], int q, int& emax) {
+  int e = 0;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) e = max(e, (word[k] >> (10 * q)) & 1023);
+  emax = e;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const int sh = min(3 * (e - ((word[k] >> (10 * q)) & 1023)), 63);
+    const int64_t v = (((int64_t)uh[k] << kLimb) | (int64_t)ul[k]) >> sh;
+    uh[k] = (int)(v >> kLimb);
+    ul[k] = (int)(v & kLimbMask);
+  }
+}
+
+// sum_k W_k u_k of one component, in units of 2^-4 of the mantissa's
+__device__ __forceinline__ int64_t dot8(const int (&wh)[8], const int (&wl)[8], const int (&uh)[8],
+                                        const int (&ul)[8]) {
+  int64_t A = 0, B = 0;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    A += (int64_t)uh[k] * wh[k];
+    B += (int64_t)uh[k] * wl[k];
+    B += (int64_t)ul[k] * wh[k];
+  }
+  return (A << 4) + (B >> (kLimb - 4));
+}
+
+__device__ __forceinline__ void gather(const FixCell* __restrict__ F, const Stencil& st, int nx, int ny, double (&up)[3]) {
+  int uh[3][8], ul[3][8], word[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const int c = ((k & 1) ? st.i1[0] : st.i0[0]) +
+                  nx * (((k & 2) ? st.i1[1] : st.i0[1]) + ny * ((k & 4) ? st.i1[2] : st.i0[2]));
+    const FixCell u = load_cell(F + c);
+    uh[0][k] = u.a.x;
+    ul[0][k] = u.a.y;
+    uh[1][k] = u.a.z;
+    ul[1][k] = u.a.w;
+    uh[2][k] = u.b.x;
+    ul[2][k] = u.b.y;
+    word[k] = u.b.z;
+  }
+  int64_t W[8];
+  weights(st.f, W);
+  int wh[8], wl[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    wh[k] = (int)(W[k] >> kLimb);
+    wl[k] = (int)(W[k] & kLimbMask);
+  }
+  int e[3] = {word[0] & 1023, (word[0] >> 10) & 1023, (word[0] >> 20) & 1023};
+  int differ = 0;
+#pragma unroll
+  for (int k = 1; k < 8; ++k) differ |= word[k] ^ word[0];
+  if (differ) {
+#pragma unroll
+    for (int q = 0; q < 3; ++q) align(uh[q], ul[q], word, q, e[q]);
+  }
+#pragma unroll
+  for (int q = 0; q < 3; ++q) up[q] = to_f64(dot8(wh, wl, uh[q], ul[q]), 3 * e[q] - kExpBias - 4);
+}
+
+}  // namespace fix
+}  // namespace st

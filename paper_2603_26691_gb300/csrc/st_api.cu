@@ -21,6 +21,19 @@ st_status cuda_check(st_ctx* h, cudaError_t e, const char* what) {
   return set_error(h, ST_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
 }
 
+// The integer copy of an FP64 field only makes its steps faster: where device memory runs out it goes first
+// (the queued work that reads it has to end before it does), and the steps read the FP64 field.
+static bool give_up_fix(st_ctx* h) {
+  if (!h->fluid_fix.p && !h->fluid_fix_next.p) return false;
+  if (cudaStreamSynchronize(h->stream) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  dev_free(h, h->fluid_fix);
+  dev_free(h, h->fluid_fix_next);
+  return true;
+}
+
 st_status dev_alloc(st_ctx* h, Buf& b, size_t bytes) {
   b.p = nullptr;
   b.bytes = 0;
@@ -29,9 +42,14 @@ st_status dev_alloc(st_ctx* h, Buf& b, size_t bytes) {
   void* p = nullptr;
   if (h->have_alloc) {
     p = h->alloc.alloc(bytes, h->alloc.user);
+    if (!p && give_up_fix(h)) p = h->alloc.alloc(bytes, h->alloc.user);
     if (!p) return set_error(h, ST_ERR_OOM, "allocator returned NULL for " + std::to_string(bytes) + " bytes");
   } else {
     cudaError_t e = cudaMalloc(&p, bytes);
+    if (e != cudaSuccess && give_up_fix(h)) {
+      cudaGetLastError();
+      e = cudaMalloc(&p, bytes);
+    }
     if (e != cudaSuccess) {
       cudaGetLastError();
       return set_error(h, ST_ERR_OOM, "cudaMalloc of " + std::to_string(bytes) + " bytes failed");
@@ -144,6 +162,8 @@ st_status st_create_grid(int nx, int ny, int nz, double Lx, double Ly, double Lz
   if (precision == ST_FP64) {
     if (s == ST_OK) s = dev_alloc(h, h->fluid, (size_t)G.ncell * 4 * sizeof(double));
     if (s == ST_OK) s = cuda_check(h, cudaMemsetAsync(h->fluid.p, 0, h->fluid.bytes, h->stream), "memset fluid");
+    if (s == ST_OK && dev_alloc(h, h->fluid_fix, (size_t)G.ncell * 32) == ST_OK)
+      s = cuda_check(h, cudaMemsetAsync(h->fluid_fix.p, 0, h->fluid_fix.bytes, h->stream), "memset fluid");
   } else {
     size_t padded = (size_t)(nx + 2 * kFluidPad) * (ny + 2 * kFluidPad) * (nz + 2 * kFluidPad);
     if (s == ST_OK) s = dev_alloc(h, h->fluid_pad, padded * 4 * sizeof(float));
@@ -168,7 +188,7 @@ void st_destroy(st_handle h) {
   cudaStreamSynchronize(h->stream);
   chunk_store_free(h);  // its slot buffers first: the handle's own are freed below
   xfer_free(h);
-  Buf* bufs[] = {&h->fluid, &h->fluid_pad, &h->flags, &h->ckpt, &h->state, &h->state_alt, &h->ids, &h->ids_alt,
+  Buf* bufs[] = {&h->fluid, &h->fluid_fix, &h->fluid_fix_next, &h->fluid_pad, &h->flags, &h->ckpt, &h->state, &h->state_alt, &h->ids, &h->ids_alt,
                  &h->keys[0], &h->keys[1], &h->vals[0], &h->vals[1], &h->hist, &h->scan_aux, &h->cell_start, &h->lsort_aux,
                  &h->acc, &h->red, &h->src_hist[0], &h->src_hist[1], &h->src_hist[2], &h->src_hist[3],
                  &h->src_est, &h->fl_cur, &h->fl_next, &h->fl_star, &h->fl_tmp, &h->fluid_pad_next, &h->umax_dev,
@@ -573,6 +593,9 @@ st_status run_steps(st_ctx* h, int nsteps, double dt) {
     // its kernel can, up to the next sort
     int m = 1;
     if (tma) m = std::min(nsteps - s, kMaxFusedSteps);
+    // (the FP64 kernel: at most as many contributions to one word as it can take between propagations)
+    if (fixed_step_supported(h))
+      m = (int)std::max(1.0, std::min({(double)(nsteps - s), (double)kMaxFusedSteps, 1073741824.0 / (double)h->np}));
     if (h->reorder_every > 0) m = std::min(m, h->reorder_every - h->steps_since_sort);
     // a sort is due after these steps: they leave the state as records for its gather
     const bool can_record = tma && default_physics(h) && h->reorder_every > 0 && h->state_alt.bytes >= (size_t)h->cap * 32;
@@ -591,7 +614,7 @@ st_status run_steps(st_ctx* h, int nsteps, double dt) {
     // digits a launch can add to one word: a tile flush of each of the (at most 8) units that cover a cell,
     // at least one unit in 2^16 particle-steps; the other kernels one contribution per particle
     ST_TRY(prepare_accumulator(h, dt, m,
-                               tma ? 8.0 * ((double)h->np * m / 65536.0 + 2.0) : deposits_per_cell(h) * (double)h->np + 8.0,
+                               tma ? 8.0 * ((double)h->np * m / 65536.0 + 2.0) : deposits_per_cell(h) * (double)h->np * m + 8.0,
                                tma, &E));
     StepParams p;
     p.dt = dt;

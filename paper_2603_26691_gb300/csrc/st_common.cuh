@@ -66,6 +66,7 @@ struct st_ctx {
 
   // fluid: FP64 handles D4[ncell] (x, y, z, 0); mixed handles float4[ncell]
   st::Buf fluid;
+  st::Buf fluid_fix;         // FP64 handles: the same field as fix::FixCell (null: given up for memory)
   st::Buf fluid_pad;         // mixed handles: float4 field with kFluidPad ghost layers, periodic
   bool fluid_set = false;
   double umax = 0.0;
@@ -135,6 +136,7 @@ struct st_ctx {
   st::Buf src_est;           // FP64 [3][ncell]
   st::Buf fl_cur, fl_next, fl_star, fl_tmp;  // fluid fields, float4 (mixed) or D4 (FP64) per cell
   st::Buf fluid_pad_next;    // mixed: the padded field of the next interval
+  st::Buf fluid_fix_next;    // FP64: the integer field of the next interval
   st::Buf umax_dev;          // max |u| of the next field (bits of a non-negative double)
   double* umax_host = nullptr;  // pinned
   cudaEvent_t ev_fluid = nullptr;  // the interval's fluid update done (its max |u| in umax_host)
@@ -395,6 +397,10 @@ inline bool default_physics(const st_ctx* h) {
 }
 
 cudaError_t launch_step_f64(st_ctx* h, const StepParams& p);
+// whether the FP64 steps run on the integer field (then several per launch)
+bool fixed_step_supported(const st_ctx* h);
+// the integer field of an FP64 one (out null: nothing)
+cudaError_t launch_fix_field(st_ctx* h, const D4* u, void* out);
 // the FP64 step on an explicit state; acc == nullptr skips the deposit (adjoint recomputation)
 cudaError_t launch_step_f64_state(st_ctx* h, const F64State& s, long long* acc, const StepParams& p);
 

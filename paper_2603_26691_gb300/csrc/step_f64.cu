@@ -6,6 +6,7 @@
 // semi-implicit Euler, Schiller-Naumann drag, cloud-in-cell deposit) are
 // uniform branches on the step's parameters.  GB300's FP64 rate is low, so this kernel is bound by
 // FP64 arithmetic rather than by HBM.
+#include "fix_gather.cuh"
 #include "st_common.cuh"
 
 namespace st {
@@ -184,13 +185,193 @@ __global__ void __launch_bounds__(256) step_f64_kernel(const F64Args a) {
   }
 }
 
+// The default physics (trilinear gather, exponential integrator, Stokes drag, cell deposit), nsteps steps per
+// launch, bound by what is left on the FP64 pipe.  There an FP64 instruction costs 64 issue cycles, so:
+//   * the gather runs on integers (fix_gather.cuh): about 400 issue cycles instead of 45 FP64 instructions;
+//   * what the diameter alone decides (the exponential and the division) is computed once per launch: the
+//     field is frozen, so a launch takes the steps up to the next sort one particle after the other, with
+//     the state in registers;
+//   * positions inside the box, told by their bits, need no wrap;
+//   * the impulses are converted to the accumulator's integers at once and summed as 128-bit integers, over
+//     the steps a particle stays in a cell and then over the warp's lanes of equal cell: exact, so the
+//     sources do not depend on the storage order or on how steps are split over launches.
+// 24 FP64 instructions are left per particle and step (3 per axis for the position and cell, 5 for the
+// motion and the impulse), against 190.  3e7 particles on 128^3, ten steps: 18.6 ms against 84.7 ms.
+struct FixArgs {
+  F64State s;
+  const fix::FixCell* __restrict__ U;
+  long long* __restrict__ acc;  // null: no deposit (the adjoint's recomputation)
+  int64_t n, ncell;
+  int nx, ny, nz, nsteps, E;
+  double L[3], invL[3], inv_h[3];
+  double dt, inv_ca, mcoef, g[3];
+};
+
+// a += round(x 2^E), |x| 2^E < 2^100
+__device__ __forceinline__ void add_fixed(__int128& a, double x, int E) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int ex = (int)((b >> 52) & 0x7ff);
+  unsigned long long man = b & 0xfffffffffffffull;
+  if (ex != 0) man |= 1ull << 52;
+  const int s = (ex == 0 ? 1 : ex) - 1075 + E;
+  unsigned long long lo, hi = 0;
+  if (__builtin_expect(s < 0, 0)) {
+    lo = s > -64 ? (man + ((1ull << -s) >> 1)) >> -s : 0ull;
+  } else {
+    const int k = min(s, 63);
+    lo = man << k;
+    hi = k ? man >> (64 - k) : 0ull;
+  }
+  const __int128 t = (__int128)(((unsigned __int128)hi << 64) | lo);
+  a += (b >> 63) ? -t : t;
+}
+
+// an integer in units of 2^-E to a cell's words: its magnitude's digits with its sign
+__device__ __forceinline__ void commit_fixed(long long* p, __int128 v) {
+  const bool neg = v < 0;
+  const unsigned __int128 m = neg ? -(unsigned __int128)v : (unsigned __int128)v;
+#pragma unroll
+  for (int k = 0; k < kAccWords; ++k) {
+    const long long d = (long long)(uint32_t)(m >> (32 * k));
+    if (d) atomicAdd((unsigned long long*)&p[k], (unsigned long long)(neg ? -d : d));
+  }
+}
+
+__device__ __forceinline__ __int128 shfl_down(__int128 v, int off) {
+  const unsigned long long lo = __shfl_down_sync(0xffffffffu, (unsigned long long)v, off);
+  const unsigned long long hi = __shfl_down_sync(0xffffffffu, (unsigned long long)((unsigned __int128)v >> 64), off);
+  return (__int128)(((unsigned __int128)hi << 64) | lo);
+}
+
+__global__ void __launch_bounds__(256, 2) step_f64_fixed_kernel(const FixArgs a) {
+  const int lane = threadIdx.x & 31;
+  const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  const int64_t nwarp = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  const int n3[3] = {a.nx, a.ny, a.nz};
+  for (int64_t base = warp * 32; base < a.n; base += nwarp * 32) {
+    const int64_t p = base + lane;
+    int key = -1;
+    __int128 J[3] = {0, 0, 0};
+    if (p < a.n) {
+      double x[3], v[3];
+      for (int q = 0; q < 3; ++q) {
+        x[q] = a.s.x[q][p];
+        v[q] = a.s.v[q][p];
+      }
+      const double d = a.s.d[p];
+      const double dd = d * d;
+      const double inv_ra = dd * a.inv_ca;
+      const double ra = 1.0 / inv_ra;
+      // 1 - e^{-a dt} from expm1; e^{-a dt} as its complement (absolute error ~1e-16, which is what
+      // multiplies v - w)
+      const double E1 = -expm1(-ra * a.dt);
+      const double E = 1.0 - E1;
+      const double Q = E1 * inv_ra;
+      const double m = a.mcoef * dd * d;
+      const double mE1 = m * E1;
+      double gi[3], mg[3];
+      for (int q = 0; q < 3; ++q) {
+        gi[q] = a.g[q] * inv_ra;
+        mg[q] = m * (a.g[q] * a.dt);
+      }
+#pragma unroll 1
+      for (int step = 0; step < a.nsteps; ++step) {
+        const fix::Stencil st = fix::stencil(x, a.inv_h, n3);
+        const int k = st.c0[0] + a.nx * (st.c0[1] + a.ny * st.c0[2]);
+        if (k != key) {
+          if (key >= 0 && a.acc) {
+            for (int q = 0; q < 3; ++q) {
+              commit_fixed(a.acc + kAccWords * (q * a.ncell + key), J[q]);
+              J[q] = 0;
+            }
+          }
+          key = k;
+        }
+        double up[3];
+        fix::gather(a.U, st, a.nx, a.ny, up);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          const double wt = up[q] + gi[q];
+          const double dvw = v[q] - wt;
+          const double xn = x[q] + (wt * a.dt + dvw * Q);
+          v[q] = wt + dvw * E;
+          // m [(v - w)(1 - E) + g dt] = -m [(v' - v) - g dt]
+          if (a.acc) add_fixed(J[q], dvw * mE1 + mg[q], a.E);
+          // inside [0, L): the bits of non-negative doubles are ordered like the values
+          x[q] = (unsigned long long)__double_as_longlong(xn) < (unsigned long long)__double_as_longlong(a.L[q])
+                     ? xn
+                     : wrap_pos(xn, a.L[q], a.invL[q]);
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        a.s.x[q][p] = x[q];
+        a.s.v[q][p] = v[q];
+      }
+    }
+    if (!a.acc) continue;
+    // the impulses since each particle's last change of cell: runs of equal cell over the warp
+    const int prev = __shfl_up_sync(0xffffffffu, key, 1);
+    const bool head = (lane == 0) || (prev != key);
+    const unsigned heads = __ballot_sync(0xffffffffu, head);
+    if (heads != 0xffffffffu) {
+      const unsigned above = lane == 31 ? 0u : (heads & ~((2u << lane) - 1u));
+      const int end = above ? (__ffs(above) - 2) : 31;
+#pragma unroll 1
+      for (int off = 1; off < 32; off <<= 1) {
+        const __int128 t0 = shfl_down(J[0], off), t1 = shfl_down(J[1], off), t2 = shfl_down(J[2], off);
+        if (lane + off <= end) {
+          J[0] += t0;
+          J[1] += t1;
+          J[2] += t2;
+        }
+      }
+    }
+    if (head && key >= 0)
+      for (int q = 0; q < 3; ++q) commit_fixed(a.acc + kAccWords * (q * a.ncell + key), J[q]);
+  }
+}
+
 }  // namespace
 
 cudaError_t launch_step_f64(st_ctx* h, const StepParams& p) {
   return launch_step_f64_state(h, carve_f64(h->state.p, h->cap), (long long*)h->acc.p, p);
 }
 
+bool fixed_step_supported(const st_ctx* h) {
+  return h->prec == ST_FP64 && h->fluid_fix.p && !h->micro_on && default_physics(h);
+}
+
+static cudaError_t launch_step_f64_fixed(st_ctx* h, const F64State& s, long long* acc, const StepParams& p) {
+  FixArgs a;
+  a.s = s;
+  a.U = (const fix::FixCell*)h->fluid_fix.p;
+  a.acc = acc;
+  a.n = h->np;
+  a.ncell = h->geo.ncell;
+  a.nx = h->geo.n[0];
+  a.ny = h->geo.n[1];
+  a.nz = h->geo.n[2];
+  a.nsteps = p.nsteps;
+  a.E = p.E;
+  for (int q = 0; q < 3; ++q) {
+    a.L[q] = h->geo.L[q];
+    a.invL[q] = 1.0 / h->geo.L[q];
+    a.inv_h[q] = h->geo.inv_h[q];
+    a.g[q] = p.g[q];
+  }
+  a.dt = p.dt;
+  a.inv_ca = 1.0 / p.ca;
+  a.mcoef = p.mcoef;
+  const int64_t blocks = std::min<int64_t>((h->np + 255) / 256, 152 * 32);
+  step_f64_fixed_kernel<<<(int)std::max<int64_t>(blocks, 1), 256, 0, h->stream>>>(a);
+  h->launches += 1;
+  return cudaGetLastError();
+}
+
 cudaError_t launch_step_f64_state(st_ctx* h, const F64State& s, long long* acc, const StepParams& p) {
+  if (fixed_step_supported(h)) return launch_step_f64_fixed(h, s, acc, p);
+  if (p.nsteps != 1) return cudaErrorInvalidValue;
   F64Args a;
   a.s = s;
   a.U = (const D4*)h->fluid.p;

@@ -5,6 +5,7 @@
 #include <cstring>
 #include <vector>
 
+#include "fix_gather.cuh"
 #include "st_common.cuh"
 #include "st_ptx.cuh"
 
@@ -67,11 +68,18 @@ __global__ void particle_scan_kernel(const double* __restrict__ xyz, const doubl
 // ---- fluid packing -----------------------------------------------------------------------
 
 template <typename T>
-__global__ void pack_f64_kernel(const T* __restrict__ u, D4* __restrict__ out, int64_t ncell,
-                                const int* __restrict__ skip = nullptr) {
+__global__ void pack_f64_kernel(const T* __restrict__ u, D4* __restrict__ out, fix::FixCell* __restrict__ fx,
+                                int64_t ncell, const int* __restrict__ skip = nullptr) {
   if (skip && *skip) return;
+  for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < ncell; c += (int64_t)gridDim.x * blockDim.x) {
+    const double x = (double)u[3 * c], y = (double)u[3 * c + 1], z = (double)u[3 * c + 2];
+    out[c] = D4{x, y, z, 0.0};
+    if (fx) fx[c] = fix::make_cell(x, y, z);
+  }
+}
+__global__ void fix_field_kernel(const D4* __restrict__ u, fix::FixCell* __restrict__ fx, int64_t ncell) {
   for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < ncell; c += (int64_t)gridDim.x * blockDim.x)
-    out[c] = D4{(double)u[3 * c], (double)u[3 * c + 1], (double)u[3 * c + 2], 0.0};
+    fx[c] = fix::make_cell(u[c].x, u[c].y, u[c].z);
 }
 
 // FP32 field with P ghost layers on every side, filled periodically: padded cell (a, b, c)
@@ -468,9 +476,11 @@ cudaError_t launch_fluid_pack_if(st_ctx* h, const void* u, int dtype, const int*
   int64_t nc = h->geo.ncell;
   if (h->prec == ST_FP64) {
     if (dtype == ST_DTYPE_F64)
-      pack_f64_kernel<double><<<grid_for(nc), kThreads, 0, h->stream>>>((const double*)u, (D4*)h->fluid.p, nc, skip);
+      pack_f64_kernel<double><<<grid_for(nc), kThreads, 0, h->stream>>>((const double*)u, (D4*)h->fluid.p,
+                                                                        (fix::FixCell*)h->fluid_fix.p, nc, skip);
     else
-      pack_f64_kernel<float><<<grid_for(nc), kThreads, 0, h->stream>>>((const float*)u, (D4*)h->fluid.p, nc, skip);
+      pack_f64_kernel<float><<<grid_for(nc), kThreads, 0, h->stream>>>((const float*)u, (D4*)h->fluid.p,
+                                                                       (fix::FixCell*)h->fluid_fix.p, nc, skip);
   } else {
     const Geometry& G = h->geo;
     const int64_t tot = (int64_t)(G.n[0] + 2 * kFluidPad) * (G.n[1] + 2 * kFluidPad) * (G.n[2] + 2 * kFluidPad);
@@ -481,6 +491,13 @@ cudaError_t launch_fluid_pack_if(st_ctx* h, const void* u, int dtype, const int*
       pack_f32_padded_kernel<float><<<grid_for(tot), kThreads, 0, h->stream>>>(
           (const float*)u, (float4*)h->fluid_pad.p, G.n[0], G.n[1], G.n[2], kFluidPad, skip);
   }
+  h->launches += 1;
+  return cudaGetLastError();
+}
+
+cudaError_t launch_fix_field(st_ctx* h, const D4* u, void* out) {
+  if (!out) return cudaSuccess;
+  fix_field_kernel<<<grid_for(h->geo.ncell), kThreads, 0, h->stream>>>(u, (fix::FixCell*)out, h->geo.ncell);
   h->launches += 1;
   return cudaGetLastError();
 }

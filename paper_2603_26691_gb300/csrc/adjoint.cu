@@ -17,6 +17,7 @@
 // per block in a fixed order; dL/dU is scattered through the transposed
 // trilinear weights into an exact carry-save fixed-point accumulator, so
 // every output is independent of thread scheduling.
+#include "fix_gather.cuh"
 #include "st_common.cuh"
 
 namespace st {
@@ -188,6 +189,206 @@ __global__ void __launch_bounds__(kAdjThreads) adjoint_step_kernel(const AdjArgs
     double t = 0.0;
     for (int w = 0; w < kAdjThreads / 32; ++w) t += sh[w];
     a.ab_part[blockIdx.x] += t;
+  }
+}
+
+// ---- a whole segment of the default physics (cell deposit) in one launch ----
+//
+// The same reverse sweep, bound by what is left on the FP64 pipe (one warp instruction in 64 cycles there):
+//   * the interpolation and its derivatives by the position run on integers (fix_gather.cuh);
+//   * what the diameter decides is computed once per particle, and the adjoints of position, velocity and
+//     diameter stay in registers over the segment;
+//   * dL/dU: a particle's products of weight and adjoint velocity are integers too.  They are summed over the
+//     steps it stays in one stencil (64-bit sums in shared memory, in units of 2^-57 of the largest adjoint
+//     velocity they may hold: finer than the rounding of FP64 products of weights above 1/16) and each sum is
+//     added to the carry-save accumulator when the particle leaves the stencil or the segment ends: 24
+//     global commits of two or three 64-bit reductions per stencil instead of per step, which bound the sweep.
+// About 55 FP64 instructions are left per particle and step, against 349.  %s
+constexpr int kSegThreads = 128;
+constexpr int kSumBits = 57;   // adjoint velocities below 2^eb are integers below 2^kSumBits in the sums
+constexpr int kSumSteps = 32;  // products one sum takes
+
+struct SegArgs {
+  const double* __restrict__ tape;  // [len][6][n]
+  const double* __restrict__ d;
+  double* __restrict__ xb[3];
+  double* __restrict__ vb[3];
+  double* __restrict__ db;
+  double* __restrict__ ab_part;
+  const fix::FixCell* __restrict__ U;
+  const double* __restrict__ lam;
+  long long* __restrict__ Uw;
+  int64_t n, ncell;
+  int nx, ny, nz, len;
+  double inv_h[3];
+  double dt, mcoef, g[3];
+  double inv_ca, inv_alpha;
+};
+
+__global__ void __launch_bounds__(kSegThreads, 3) adjoint_segment_kernel(const SegArgs a) {
+  // sums[3 k + q][thread]: corner k, component q (padded: a commit reads a column)
+  __shared__ long long sums[24][kSegThreads + 1];
+  const int n3[3] = {a.nx, a.ny, a.nz};
+  const int t = threadIdx.x;
+  double alphab_sum = 0.0;
+#pragma unroll
+  for (int i = 0; i < 24; ++i) sums[i][t] = 0;
+  for (int64_t wbase = blockIdx.x * (int64_t)blockDim.x + (t & ~31); wbase < a.n;
+       wbase += (int64_t)gridDim.x * blockDim.x) {
+    __syncwarp();
+    const int64_t p = wbase + (t & 31);
+    const unsigned lanes = __ballot_sync(0xffffffffu, p < a.n);
+    if (p >= a.n) continue;
+    const double d = a.d[p];
+    const double dd = d * d;
+    const double inv_ra = dd * a.inv_ca;
+    const double ra = 1.0 / inv_ra;
+    const double inv_ra2 = inv_ra * inv_ra;
+    const double inv_d = 1.0 / d;
+    const double E1 = -expm1(-ra * a.dt);
+    const double E = 1.0 - E1;  // e^{-a dt} as the complement of expm1, as in the forward step
+    const double Q = E1 * inv_ra;
+    const double dtQ = a.dt - Q;
+    const double m = a.mcoef * dd * d;
+    const double c1 = a.dt * E, c2 = inv_ra * (c1 - Q);
+    double xb[3], vb[3];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      xb[q] = a.xb[q][p];
+      vb[q] = a.vb[q][p];
+    }
+    double ab_sum = 0.0, mb_sum = 0.0;
+    int corner0 = -1, c1x = 0, c1y = 0, c1z = 0;  // the stencil of the sums: its base cell, steps to the next cells
+    int eb[3] = {0, 0, 0}, added = 0;
+    // the sums of the lanes that need it, one lane's 24 spread over the warp at a time (few lanes leave their
+    // stencil in a step, and one lane's commits by itself would hold up the others for 24 of them)
+    auto commit = [&](bool need) {
+      unsigned who = __ballot_sync(lanes, need);
+      while (who) {
+        const int src = __ffs(who) - 1;
+        who &= who - 1;
+        const int c0 = __shfl_sync(lanes, corner0, src), sx = __shfl_sync(lanes, c1x, src),
+                  sy = __shfl_sync(lanes, c1y, src), sz = __shfl_sync(lanes, c1z, src);
+        const int e0 = __shfl_sync(lanes, eb[0], src), e1 = __shfl_sync(lanes, eb[1], src),
+                  e2 = __shfl_sync(lanes, eb[2], src);
+        const int col = (t & ~31) + src;
+        for (int i = t & 31; i < 24; i += __popc(lanes)) {
+          const int k = i / 3, q = i - 3 * k;
+          const int c = c0 + ((k & 1) ? sx : 0) + ((k & 2) ? sy : 0) + ((k & 4) ? sz : 0);
+          wide_add_int(a.Uw + ((int64_t)c * 3 + q) * kWideWords, sums[i][col],
+                       (q == 0 ? e0 : q == 1 ? e1 : e2) - kSumBits);
+          sums[i][col] = 0;
+        }
+        __syncwarp(lanes);
+      }
+      if (need) added = 0;
+    };
+#pragma unroll 1
+    for (int step = a.len - 1; step >= 0; --step) {
+      __syncwarp(lanes);
+      const double* slot = a.tape + (int64_t)step * 6 * a.n;
+      double x[3], v[3];
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        x[q] = slot[q * a.n + p];
+        v[q] = slot[(3 + q) * a.n + p];
+      }
+      const fix::Stencil st = fix::stencil(x, a.inv_h, n3);
+      const int key = st.c0[0] + a.nx * (st.c0[1] + a.ny * st.c0[2]);
+      const double Jb[3] = {a.lam[key], a.lam[a.ncell + key], a.lam[2 * a.ncell + key]};
+      const int base = st.i0[0] + a.nx * (st.i0[1] + a.ny * st.i0[2]);
+      fix::Corners u;
+      fix::load_corners(a.U, st, a.nx, a.ny, u);
+      int64_t W[8];
+      fix::weights(st.f, W);
+      double ub[3], dvw[3];
+      double mb = 0.0, S = 0.0, Qb = 0.0, gs = 0.0;
+      {
+        double up[3];
+        fix::interpolate(u, W, up);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          const double wt = up[q] + a.g[q] * inv_ra;
+          dvw[q] = v[q] - wt;
+          const double mJ = m * Jb[q];
+          const double vnb = vb[q] - mJ;
+          // -(v' - v - g dt) = (v - w) (1 - E) + g dt
+          mb += (dvw[q] * E1 + a.g[q] * a.dt) * Jb[q];
+          S += vnb * dvw[q];
+          Qb += xb[q] * dvw[q];
+          ub[q] = vnb * E1 + xb[q] * dtQ;
+          gs += ub[q] * a.g[q];
+          vb[q] = vnb * E + (xb[q] * Q + mJ);
+        }
+      }
+      // a's adjoint: through w (gravity), Q = E1 / a, and E, E1 (dE1/da = dt E)
+      const double ab = c2 * Qb - c1 * S - gs * inv_ra2;
+      ab_sum += ab;
+      mb_sum += mb;
+      // dL/df, the derivatives of the interpolated velocity dotted with its adjoint
+      {
+        double g[3];
+        fix::derivative<0>(u, st.f, g);
+        xb[0] += (g[0] * ub[0] + g[1] * ub[1] + g[2] * ub[2]) * a.inv_h[0];
+        fix::derivative<1>(u, st.f, g);
+        xb[1] += (g[0] * ub[0] + g[1] * ub[1] + g[2] * ub[2]) * a.inv_h[1];
+        fix::derivative<2>(u, st.f, g);
+        xb[2] += (g[0] * ub[0] + g[1] * ub[1] + g[2] * ub[2]) * a.inv_h[2];
+      }
+      // dL/dU: the adjoint velocities as integers in the sums' units; sums that cannot take them, or belong to
+      // another stencil, are committed and started anew
+      int eu[3];
+      bool fits = added < kSumSteps && base == corner0;
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        eu[q] = (int)(((unsigned long long)__double_as_longlong(ub[q]) >> 52) & 0x7ff) - 1022;  // |ub| < 2^eu
+        fits = fits && eu[q] <= eb[q];
+      }
+      commit(added && !fits);
+      if (added == 0) {
+        corner0 = base;
+        c1x = st.i1[0] - st.i0[0];
+        c1y = a.nx * (st.i1[1] - st.i0[1]);
+        c1z = a.nx * a.ny * (st.i1[2] - st.i0[2]);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) eb[q] = eu[q] + 1;
+      }
+      ++added;
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        const unsigned long long b = (unsigned long long)__double_as_longlong(ub[q]);
+        const int sh = eb[q] - eu[q] + 64 - kSumBits;  // significand at 2^63 for |ub| in [2^(eu-1), 2^eu): down to 2^kSumBits
+        unsigned long long mag = ((b << 11) | 0x8000000000000000ull);
+        mag = ((b << 1) == 0 || sh > 63) ? 0ull : (mag >> sh) + ((mag >> (sh - 1)) & 1ull);
+        const int64_t ui = (b >> 63) ? -(int64_t)mag : (int64_t)mag;
+        const int uh = (int)(ui >> fix::kLimb), ul = (int)(ui & fix::kLimbMask);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const int wh = (int)(W[k] >> fix::kLimb), wl = (int)(W[k] & fix::kLimbMask);
+          sums[3 * k + q][t] += (int64_t)uh * wh + (((int64_t)uh * wl + (int64_t)ul * wh) >> fix::kLimb);
+        }
+      }
+    }
+    __syncwarp(lanes);
+    commit(added != 0);
+    alphab_sum += ab_sum * ra * a.inv_alpha;
+    a.db[p] += ab_sum * (-2.0 * ra * inv_d) + mb_sum * (3.0 * m * inv_d);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      a.xb[q][p] = xb[q];
+      a.vb[q][p] = vb[q];
+    }
+  }
+  // fixed-order block reduction of dL/dalpha
+  __shared__ double sh[kSegThreads / 32];
+  double s = alphab_sum;
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+  if ((t & 31) == 0) sh[t >> 5] = s;
+  __syncthreads();
+  if (t == 0) {
+    double r = 0.0;
+    for (int w = 0; w < kSegThreads / 32; ++w) r += sh[w];
+    a.ab_part[blockIdx.x] += r;
   }
 }
 
@@ -444,6 +645,37 @@ cudaError_t launch_adjoint_step(st_ctx* h, const AdjointStepArgs& s) {
     adjoint_step_kernel<true><<<kAdjBlocks, kAdjThreads, 0, h->stream>>>(a);
   else
     adjoint_step_kernel<false><<<kAdjBlocks, kAdjThreads, 0, h->stream>>>(a);
+  h->launches += 1;
+  return cudaGetLastError();
+}
+
+cudaError_t launch_adjoint_segment(st_ctx* h, const AdjointStepArgs& s, int len) {
+  SegArgs a;
+  a.tape = s.x[0];
+  a.d = s.d;
+  for (int q = 0; q < 3; ++q) {
+    a.xb[q] = s.xb[q];
+    a.vb[q] = s.vb[q];
+    a.inv_h[q] = h->geo.inv_h[q];
+    a.g[q] = h->g[q];
+  }
+  a.db = s.db;
+  a.ab_part = s.ab_part;
+  a.U = (const fix::FixCell*)h->fluid_fix.p;
+  a.lam = s.lam;
+  a.Uw = s.Uw;
+  a.n = h->np;
+  a.ncell = h->geo.ncell;
+  a.nx = h->geo.n[0];
+  a.ny = h->geo.n[1];
+  a.nz = h->geo.n[2];
+  a.len = len;
+  a.dt = s.dt;
+  a.inv_ca = h->rho_p / (18.0 * h->mu * h->alpha);
+  a.mcoef = h->mult * h->rho_p * 3.14159265358979323846 / 6.0;
+  a.inv_alpha = 1.0 / h->alpha;
+  const int64_t blocks = std::min<int64_t>((h->np + kSegThreads - 1) / kSegThreads, kAdjBlocks);
+  adjoint_segment_kernel<<<(int)std::max<int64_t>(blocks, 1), kSegThreads, 0, h->stream>>>(a);
   h->launches += 1;
   return cudaGetLastError();
 }

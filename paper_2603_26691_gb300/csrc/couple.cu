@@ -161,8 +161,9 @@ st_status couple_resources(st_ctx* h) {
     if (h->fl_cur.bytes < fb) ST_TRY(dev_alloc(h, h->fl_cur, fb));
     if (h->fluid_pad_next.bytes < h->fluid_pad.bytes) ST_TRY(dev_alloc(h, h->fluid_pad_next, h->fluid_pad.bytes));
   } else if (h->fluid_fix_next.bytes < h->fluid_fix.bytes) {
-    if (dev_alloc(h, h->fluid_fix_next, h->fluid_fix.bytes) != ST_OK) {
+    if (dev_alloc(h, h->fluid_fix_next, h->fluid_fix.bytes) != ST_OK || !h->fluid_fix.p) {
       dev_free(h, h->fluid_fix);  // no room for two: the steps then read the FP64 field
+      dev_free(h, h->fluid_fix_next);
       h->err.clear();
     }
   }

@@ -141,39 +141,82 @@ __device__ __forceinline__ int64_t dot8(const int (&wh)[8], const int (&wl)[8], 
   return (A << 4) + (B >> (kLimb - 4));
 }
 
-__device__ __forceinline__ void gather(const FixCell* __restrict__ F, const Stencil& st, int nx, int ny, double (&up)[3]) {
-  int uh[3][8], ul[3][8], word[8];
+// the eight corners' mantissas in limbs, brought to one exponent per component
+struct Corners {
+  int uh[3][8], ul[3][8], e[3];
+};
+__device__ __forceinline__ void load_corners(const FixCell* __restrict__ F, const Stencil& st, int nx, int ny, Corners& u) {
+  int word[8];
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
     const int c = ((k & 1) ? st.i1[0] : st.i0[0]) +
                   nx * (((k & 2) ? st.i1[1] : st.i0[1]) + ny * ((k & 4) ? st.i1[2] : st.i0[2]));
-    const FixCell u = load_cell(F + c);
-    uh[0][k] = u.a.x;
-    ul[0][k] = u.a.y;
-    uh[1][k] = u.a.z;
-    ul[1][k] = u.a.w;
-    uh[2][k] = u.b.x;
-    ul[2][k] = u.b.y;
-    word[k] = u.b.z;
+    const FixCell v = load_cell(F + c);
+    u.uh[0][k] = v.a.x;
+    u.ul[0][k] = v.a.y;
+    u.uh[1][k] = v.a.z;
+    u.ul[1][k] = v.a.w;
+    u.uh[2][k] = v.b.x;
+    u.ul[2][k] = v.b.y;
+    word[k] = v.b.z;
   }
-  int64_t W[8];
-  weights(st.f, W);
+  int differ = 0;
+#pragma unroll
+  for (int q = 0; q < 3; ++q) u.e[q] = (word[0] >> (10 * q)) & 1023;
+#pragma unroll
+  for (int k = 1; k < 8; ++k) differ |= word[k] ^ word[0];
+  if (differ) {
+#pragma unroll
+    for (int q = 0; q < 3; ++q) align(u.uh[q], u.ul[q], word, q, u.e[q]);
+  }
+}
+
+// the interpolated value from the corners and their weights
+__device__ __forceinline__ void interpolate(const Corners& u, const int64_t (&W)[8], double (&up)[3]) {
   int wh[8], wl[8];
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
     wh[k] = (int)(W[k] >> kLimb);
     wl[k] = (int)(W[k] & kLimbMask);
   }
-  int e[3] = {word[0] & 1023, (word[0] >> 10) & 1023, (word[0] >> 20) & 1023};
-  int differ = 0;
 #pragma unroll
-  for (int k = 1; k < 8; ++k) differ |= word[k] ^ word[0];
-  if (differ) {
+  for (int q = 0; q < 3; ++q) up[q] = to_f64(dot8(wh, wl, u.uh[q], u.ul[q]), 3 * u.e[q] - kExpBias - 4);
+}
+
+// the derivatives of the interpolated components by the fraction along axis r: the differences along r at the
+// four edges, weighted over the other two axes (a and b, in that order the faster bits of an edge's number)
+template <int r>
+__device__ __forceinline__ void derivative(const Corners& u, const int64_t (&f)[3], double (&g)[3]) {
+  constexpr int a = r == 0 ? 1 : 0, b = r == 2 ? 1 : 2;
+  const int64_t p = mul58(f[a], f[b]);
+  const int64_t w[4] = {kOne - f[a] - f[b] + p, f[a] - p, f[b] - p, p};
+  int wh[4], wl[4];
 #pragma unroll
-    for (int q = 0; q < 3; ++q) align(uh[q], ul[q], word, q, e[q]);
+  for (int k = 0; k < 4; ++k) {
+    wh[k] = (int)(w[k] >> kLimb);
+    wl[k] = (int)(w[k] & kLimbMask);
   }
 #pragma unroll
-  for (int q = 0; q < 3; ++q) up[q] = to_f64(dot8(wh, wl, uh[q], ul[q]), 3 * e[q] - kExpBias - 4);
+  for (int q = 0; q < 3; ++q) {
+    int64_t A = 0, B = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int lo = ((k & 1) << a) | ((k >> 1) << b), hi = lo | (1 << r);
+      const int dh = u.uh[q][hi] - u.uh[q][lo], dl = u.ul[q][hi] - u.ul[q][lo];
+      A += (int64_t)dh * wh[k];
+      B += (int64_t)dh * wl[k];
+      B += (int64_t)dl * wh[k];
+    }
+    g[q] = to_f64((A << 3) + (B >> (kLimb - 3)), 3 * u.e[q] - kExpBias - 3);
+  }
+}
+
+__device__ __forceinline__ void gather(const FixCell* __restrict__ F, const Stencil& st, int nx, int ny, double (&up)[3]) {
+  Corners u;
+  load_corners(F, st, nx, ny, u);
+  int64_t W[8];
+  weights(st.f, W);
+  interpolate(u, W, up);
 }
 
 }  // namespace fix

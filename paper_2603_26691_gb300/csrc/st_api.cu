@@ -973,12 +973,16 @@ st_status st_adjoint_forward(st_handle h, int nsteps, double dt, int checkpoint_
   const double pi = 3.14159265358979323846;
   F64State s = carve_f64(h->state.p, h->cap);
   double* ck = (double*)h->ckpt.p;
-  for (int step = 0; step < nsteps; ++step) {
+  const bool tape = fixed_step_supported(h);  // checkpoints written by the step kernel, several steps per launch
+  for (int step = 0; step < nsteps;) {
+    int m = 1;
+    if (tape)
+      m = (int)std::max(1.0, std::min({(double)(nsteps - step), (double)kMaxFusedSteps, 1073741824.0 / (double)n}));
     if (mixed && step % checkpoint_every == 0) {
       const MixedState slot = carve_mixed((char*)h->ckpt.p + (size_t)(step / checkpoint_every) * ck_bytes,
                                           round64(n), false);
       ST_TRY(cuda_check(h, copy_mixed7(slot, carve_mixed(h->state.p, h->cap, false), n, h->stream), "checkpoint"));
-    } else if (step % checkpoint_every == 0) {
+    } else if (!tape && step % checkpoint_every == 0) {
       double* slot = ck + (size_t)(step / checkpoint_every) * 6 * n;
       cudaError_t e = cudaSuccess;
       for (int q = 0; q < 3 && e == cudaSuccess; ++q) {
@@ -989,9 +993,10 @@ st_status st_adjoint_forward(st_handle h, int nsteps, double dt, int checkpoint_
       ST_TRY(cuda_check(h, e, "checkpoint"));
     }
     int E = 0;
-    ST_TRY(prepare_accumulator(h, dt, 1, deposits_per_cell(h) * (double)h->np + 8.0, false, &E));
+    ST_TRY(prepare_accumulator(h, dt, m, deposits_per_cell(h) * (double)h->np * m + 8.0, false, &E));
     StepParams p;
     p.dt = dt;
+    p.nsteps = m;
     p.ca = 18.0 * h->mu * h->alpha / h->rho_p;
     p.mcoef = h->mult * h->rho_p * pi / 6.0;
     for (int q = 0; q < 3; ++q) p.g[q] = h->g[q];
@@ -1000,9 +1005,18 @@ st_status st_adjoint_forward(st_handle h, int nsteps, double dt, int checkpoint_
     p.cic = h->phys_deposit == ST_DEPOSIT_CIC;  // the other physics are the defaults here
     timer_begin(h, ST_TIMER_STEP, h->stream);
     // mixed handles: the general kernel in storage order, which the backward pass recomputes with
-    const cudaError_t fe = mixed ? launch_step_mixed(h, p) : launch_step_f64(h, p);
-    timer_end(h, ST_TIMER_STEP, h->stream);
+    cudaError_t fe;
+    if (tape) {
+      const int slot = (step + checkpoint_every - 1) / checkpoint_every;  // the next checkpoint
+      const double* in[6] = {s.x[0], s.x[1], s.x[2], s.v[0], s.v[1], s.v[2]};
+      fe = launch_step_f64_tape(h, in, s, (long long*)h->acc.p, p, ck + (size_t)slot * 6 * n,
+                                slot * checkpoint_every - step, checkpoint_every);
+    } else {
+      fe = mixed ? launch_step_mixed(h, p) : launch_step_f64(h, p);
+    }
+    timer_end(h, ST_TIMER_STEP, h->stream, m);
     ST_TRY(cuda_check(h, fe, "adjoint forward step"));
+    step += m;
   }
   h->adj_nsteps = nsteps;
   h->adj_every = checkpoint_every;
@@ -1026,12 +1040,15 @@ st_status st_adjoint_backward(st_handle h, const double* lam, int lam_on_device,
   auto cleanup = [&]() {
     for (Buf* b : {&blam, &work, &tape, &adj, &abp, &Uw, &tmp}) dev_free(h, *b);
   };
-  st_status s = dev_alloc(h, work, (size_t)6 * n * sizeof(double));
-  if (s == ST_OK) s = dev_alloc(h, tape, (size_t)C * 6 * n * sizeof(double));
+  st_status s = ST_OK;
+  if (!fixed_step_supported(h)) s = dev_alloc(h, work, (size_t)6 * n * sizeof(double));
+  if (s == ST_OK) s = dev_alloc(h, tape, (size_t)std::min(C, nsteps) * 6 * n * sizeof(double));
   if (s == ST_OK) s = dev_alloc(h, adj, (size_t)7 * n * sizeof(double));
   if (s == ST_OK) s = dev_alloc(h, abp, (size_t)kAdjBlocks * sizeof(double));
   if (s == ST_OK) s = dev_alloc(h, Uw, (size_t)nc * 3 * kWideWords * sizeof(long long));
   if (s == ST_OK && !lam_on_device) s = dev_alloc(h, blam, (size_t)3 * nc * sizeof(double));
+  // (the integer field may have gone for the others' sake)
+  if (s == ST_OK && !fixed_step_supported(h) && !work.p) s = dev_alloc(h, work, (size_t)6 * n * sizeof(double));
   if (s == ST_OK && (!on_device)) s = dev_alloc(h, tmp, (size_t)(std::max<int64_t>(n, 3 * nc)) * sizeof(double));
   if (s != ST_OK) {
     cleanup();
@@ -1064,6 +1081,43 @@ st_status st_adjoint_backward(st_handle h, const double* lam, int lam_on_device,
   p.scale = 1.0;
   for (int seg = K - 1; seg >= 0 && e == cudaSuccess; --seg) {
     const int s0 = seg * C, s1 = std::min(nsteps, s0 + C);
+    if (!work.p) {
+      // the segment recomputed in one launch, its states kept on the tape (of a single step the checkpoint
+      // is the tape), then reversed in one launch
+      double* ck = (double*)h->ckpt.p + (size_t)seg * 6 * n;
+      double* tp = s1 - s0 == 1 ? ck : (double*)tape.p;
+      if (s1 - s0 > 1) {
+        const double* in[6];
+        F64State last;
+        for (int q = 0; q < 3; ++q) {
+          in[q] = ck + q * n;
+          in[3 + q] = ck + (3 + q) * n;
+          last.x[q] = tp + ((size_t)(s1 - s0 - 1) * 6 + q) * n;
+          last.v[q] = tp + ((size_t)(s1 - s0 - 1) * 6 + 3 + q) * n;
+        }
+        last.d = st.d;
+        p.nsteps = s1 - s0 - 1;
+        timer_begin(h, ST_TIMER_STEP, h->stream);
+        e = launch_step_f64_tape(h, in, last, nullptr, p, tp, 0, 1);
+        timer_end(h, ST_TIMER_STEP, h->stream, p.nsteps);
+      }
+      AdjointStepArgs a;
+      a.x[0] = tp;
+      for (int q = 0; q < 3; ++q) {
+        a.xb[q] = A + q * n;
+        a.vb[q] = A + (3 + q) * n;
+      }
+      a.d = st.d;
+      a.db = A + 6 * n;
+      a.ab_part = (double*)abp.p;
+      a.lam = dlam;
+      a.Uw = (long long*)Uw.p;
+      a.dt = h->adj_dt;
+      timer_begin(h, ST_TIMER_ADJOINT, h->stream);
+      if (e == cudaSuccess) e = launch_adjoint_segment(h, a, s1 - s0);
+      timer_end(h, ST_TIMER_ADJOINT, h->stream, s1 - s0);
+      continue;
+    }
     e = cudaMemcpyAsync(W, (double*)h->ckpt.p + (size_t)seg * 6 * n, (size_t)6 * n * sizeof(double),
                         cudaMemcpyDeviceToDevice, h->stream);
     // recompute the segment, keeping the state at the start of every step

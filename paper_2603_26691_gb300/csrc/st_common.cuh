@@ -399,6 +399,10 @@ inline bool default_physics(const st_ctx* h) {
 cudaError_t launch_step_f64(st_ctx* h, const StepParams& p);
 // whether the FP64 steps run on the integer field (then several per launch)
 bool fixed_step_supported(const st_ctx* h);
+// those steps from one state to another (in may be out), keeping the states before steps first, first + every, ...
+// on a tape of 6 n values each (x, v)
+cudaError_t launch_step_f64_tape(st_ctx* h, const double* const (&in)[6], const F64State& s, long long* acc,
+                                 const StepParams& p, double* tape, int first, int every);
 // the integer field of an FP64 one (out null: nothing)
 cudaError_t launch_fix_field(st_ctx* h, const D4* u, void* out);
 // the FP64 step on an explicit state; acc == nullptr skips the deposit (adjoint recomputation)
@@ -457,6 +461,23 @@ __device__ __forceinline__ void wide_add(long long* w, double x) {
   if (q < kWideWords) atomicAdd((unsigned long long*)&w[q], (unsigned long long)d0);
   if (q + 1 < kWideWords) atomicAdd((unsigned long long*)&w[q + 1], (unsigned long long)d1);
   if (q + 2 < kWideWords) atomicAdd((unsigned long long*)&w[q + 2], (unsigned long long)d2);
+}
+
+// v * 2^ex (an integer and an exponent) into the same accumulator; what lies below its grid is rounded off
+__device__ __forceinline__ void wide_add_int(long long* w, long long v, int ex) {
+  unsigned long long m = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+  int s = ex - kWideBase;
+  if (__builtin_expect(s < 0, 0)) {
+    m = s <= -64 ? 0ull : (m >> -s) + ((m >> (-s - 1)) & 1ull);
+    s = 0;
+  }
+  const int q = s >> 5, r = s & 31;
+  const unsigned long long lo = m << r, hi = (m >> 1) >> (63 - r);
+  const long long d[3] = {(long long)(lo & 0xffffffffull), (long long)(lo >> 32), (long long)hi};
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+    if (d[k] != 0 && q + k < kWideWords)
+      atomicAdd((unsigned long long*)&w[q + k], (unsigned long long)(v < 0 ? -d[k] : d[k]));
 }
 
 // ---- sums over a warp's lanes of equal key, before one exact commit per key ----
@@ -549,6 +570,9 @@ struct AdjointStepArgs {
   double dt;
 };
 cudaError_t launch_adjoint_step(st_ctx* h, const AdjointStepArgs& s);
+// a whole segment of `len` steps in one launch (fixed_step_supported handles): s.x and s.v point at the first
+// state of a tape whose states lie 6 n values apart
+cudaError_t launch_adjoint_segment(st_ctx* h, const AdjointStepArgs& s, int len);
 // the FP32 adjoint of the mixed-precision step (FP32-velocity handles): the tape holds the state at
 // the start of the step (cell, offsets, velocities; diameters in d), the adjoints of position and
 // velocity are FP32 arrays, dL/dd and dL/dalpha accumulate in FP64, dL/dU goes into the same exact

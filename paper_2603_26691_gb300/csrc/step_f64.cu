@@ -198,7 +198,10 @@ __global__ void __launch_bounds__(256) step_f64_kernel(const F64Args a) {
 // 24 FP64 instructions are left per particle and step (3 per axis for the position and cell, 5 for the
 // motion and the impulse), against 190.  3e7 particles on 128^3, ten steps: 18.6 ms against 84.7 ms.
 struct FixArgs {
-  F64State s;
+  const double* in[6];              // position and velocity before the steps
+  F64State s;                       // after them (the same arrays, or others); diameters
+  double* __restrict__ tape;        // null, or where the state before step tape_first goes (x, v: 6 n values), the
+  int tape_first, tape_every;       // one tape_every steps later 6 n values behind it, and so on
   const fix::FixCell* __restrict__ U;
   long long* __restrict__ acc;  // null: no deposit (the adjoint's recomputation)
   int64_t n, ncell;
@@ -250,13 +253,14 @@ __global__ void __launch_bounds__(256, 2) step_f64_fixed_kernel(const FixArgs a)
   const int n3[3] = {a.nx, a.ny, a.nz};
   for (int64_t base = warp * 32; base < a.n; base += nwarp * 32) {
     const int64_t p = base + lane;
+    const unsigned lanes = __ballot_sync(0xffffffffu, p < a.n);
     int key = -1;
     __int128 J[3] = {0, 0, 0};
     if (p < a.n) {
       double x[3], v[3];
       for (int q = 0; q < 3; ++q) {
-        x[q] = a.s.x[q][p];
-        v[q] = a.s.v[q][p];
+        x[q] = a.in[q][p];
+        v[q] = a.in[3 + q][p];
       }
       const double d = a.s.d[p];
       const double dd = d * d;
@@ -274,8 +278,18 @@ __global__ void __launch_bounds__(256, 2) step_f64_fixed_kernel(const FixArgs a)
         gi[q] = a.g[q] * inv_ra;
         mg[q] = m * (a.g[q] * a.dt);
       }
+      double* slot = a.tape;
+      int next = a.tape ? a.tape_first : a.nsteps;
 #pragma unroll 1
       for (int step = 0; step < a.nsteps; ++step) {
+        if (step == next) {
+          for (int q = 0; q < 3; ++q) {
+            slot[q * a.n + p] = x[q];
+            slot[(3 + q) * a.n + p] = v[q];
+          }
+          slot += 6 * a.n;
+          next += a.tape_every;
+        }
         const fix::Stencil st = fix::stencil(x, a.inv_h, n3);
         const int k = st.c0[0] + a.nx * (st.c0[1] + a.ny * st.c0[2]);
         if (k != key) {
@@ -287,6 +301,7 @@ __global__ void __launch_bounds__(256, 2) step_f64_fixed_kernel(const FixArgs a)
           }
           key = k;
         }
+        __syncwarp(lanes);
         double up[3];
         fix::gather(a.U, st, a.nx, a.ny, up);
 #pragma unroll
@@ -342,9 +357,14 @@ bool fixed_step_supported(const st_ctx* h) {
   return h->prec == ST_FP64 && h->fluid_fix.p && !h->micro_on && default_physics(h);
 }
 
-static cudaError_t launch_step_f64_fixed(st_ctx* h, const F64State& s, long long* acc, const StepParams& p) {
+cudaError_t launch_step_f64_tape(st_ctx* h, const double* const (&in)[6], const F64State& s, long long* acc,
+                                 const StepParams& p, double* tape, int first, int every) {
   FixArgs a;
+  for (int k = 0; k < 6; ++k) a.in[k] = in[k];
   a.s = s;
+  a.tape = tape;
+  a.tape_first = first;
+  a.tape_every = every;
   a.U = (const fix::FixCell*)h->fluid_fix.p;
   a.acc = acc;
   a.n = h->np;
@@ -370,7 +390,10 @@ static cudaError_t launch_step_f64_fixed(st_ctx* h, const F64State& s, long long
 }
 
 cudaError_t launch_step_f64_state(st_ctx* h, const F64State& s, long long* acc, const StepParams& p) {
-  if (fixed_step_supported(h)) return launch_step_f64_fixed(h, s, acc, p);
+  if (fixed_step_supported(h)) {
+    const double* in[6] = {s.x[0], s.x[1], s.x[2], s.v[0], s.v[1], s.v[2]};
+    return launch_step_f64_tape(h, in, s, acc, p, nullptr, 0, 1);
+  }
   if (p.nsteps != 1) return cudaErrorInvalidValue;
   F64Args a;
   a.s = s;

@@ -593,9 +593,11 @@ st_status run_steps(st_ctx* h, int nsteps, double dt) {
     // its kernel can, up to the next sort
     int m = 1;
     if (tma) m = std::min(nsteps - s, kMaxFusedSteps);
-    // (the FP64 kernel: at most as many contributions to one word as it can take between propagations)
-    if (fixed_step_supported(h))
-      m = (int)std::max(1.0, std::min({(double)(nsteps - s), (double)kMaxFusedSteps, 1073741824.0 / (double)h->np}));
+    // (the kernels that commit every run by itself: at most as many contributions as one word can take between
+    // propagations)
+    if (fixed_step_supported(h) || (h->prec != ST_FP64 && !h->micro_on && !tma))
+      m = (int)std::max(1.0, std::min({(double)(nsteps - s), (double)kMaxFusedSteps,
+                                       1073741824.0 / (deposits_per_cell(h) * (double)h->np)}));
     if (h->reorder_every > 0) m = std::min(m, h->reorder_every - h->steps_since_sort);
     // a sort is due after these steps: they leave the state as records for its gather
     const bool can_record = tma && default_physics(h) && h->reorder_every > 0 && h->state_alt.bytes >= (size_t)h->cap * 32;
@@ -832,7 +834,6 @@ st_status st_clear_particles(st_handle h) {
 }
 
 static int64_t round64(int64_t n);
-static cudaError_t copy_mixed7(const MixedState& dst, const MixedState& src, int64_t n, cudaStream_t st);
 
 // The FP32 adjoint of a mixed FP32-velocity handle: like the FP64 one (segments from the last,
 // each recomputed from its checkpoint with the general mixed kernel keeping the state at the start of
@@ -844,14 +845,14 @@ static st_status adjoint_backward_mixed(st_handle h, const double* lam, int lam_
   const int K = (nsteps + C - 1) / C;
   const double pi = 3.14159265358979323846;
   const size_t sb = (size_t)28 * cn;  // one state: cell, offsets, velocities
-  Buf blam, lam32, work, tape, adj, db, abp, Uw, tmp;
+  Buf blam, lam32, tape, adj, db, ab, abp, Uw, tmp;
   auto cleanup = [&]() {
-    for (Buf* b : {&blam, &lam32, &work, &tape, &adj, &db, &abp, &Uw, &tmp}) dev_free(h, *b);
+    for (Buf* b : {&blam, &lam32, &tape, &adj, &db, &ab, &abp, &Uw, &tmp}) dev_free(h, *b);
   };
-  st_status s = dev_alloc(h, work, state_bytes(ST_MIXED_F32, cn));
-  if (s == ST_OK) s = dev_alloc(h, tape, (size_t)C * sb);
+  st_status s = dev_alloc(h, tape, (size_t)std::min(C, nsteps) * sb);
   if (s == ST_OK) s = dev_alloc(h, adj, (size_t)6 * cn * sizeof(float));
   if (s == ST_OK) s = dev_alloc(h, db, (size_t)cn * sizeof(double));
+  if (s == ST_OK) s = dev_alloc(h, ab, (size_t)cn * sizeof(double));
   if (s == ST_OK) s = dev_alloc(h, abp, (size_t)kAdjBlocks * sizeof(double));
   if (s == ST_OK) s = dev_alloc(h, Uw, (size_t)nc * 3 * kWideWords * sizeof(long long));
   if (s == ST_OK) s = dev_alloc(h, lam32, (size_t)3 * nc * sizeof(float));
@@ -870,11 +871,9 @@ static st_status adjoint_backward_mixed(st_handle h, const double* lam, int lam_
   if (e == cudaSuccess) e = launch_f64_to_f32(h, dlam, (float*)lam32.p, 3 * nc);
   if (e == cudaSuccess) e = cudaMemsetAsync(adj.p, 0, adj.bytes, h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(db.p, 0, db.bytes, h->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(abp.p, 0, abp.bytes, h->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(ab.p, 0, ab.bytes, h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(Uw.p, 0, Uw.bytes, h->stream);
   const MixedState st = carve_mixed(h->state.p, h->cap, false);
-  MixedState ws = carve_mixed(work.p, cn, false);
-  ws.d = st.d;
   float* A = (float*)adj.p;
   StepParams p;
   p.dt = h->adj_dt;
@@ -885,33 +884,37 @@ static st_status adjoint_backward_mixed(st_handle h, const double* lam, int lam_
   p.scale = 1.0;
   for (int seg = K - 1; seg >= 0 && e == cudaSuccess; --seg) {
     const int s0 = seg * C, s1 = std::min(nsteps, s0 + C);
-    e = cudaMemcpyAsync(work.p, (char*)h->ckpt.p + (size_t)seg * sb, sb, cudaMemcpyDeviceToDevice, h->stream);
-    for (int k = s0; k < s1 && e == cudaSuccess; ++k) {
-      e = cudaMemcpyAsync((char*)tape.p + (size_t)(k - s0) * sb, work.p, sb, cudaMemcpyDeviceToDevice, h->stream);
-      if (e == cudaSuccess && k + 1 < s1) {
-        timer_begin(h, ST_TIMER_STEP, h->stream);
-        e = launch_step_mixed_state(h, ws, n, nullptr, p);
-        timer_end(h, ST_TIMER_STEP, h->stream);
-      }
+    // the segment recomputed in one launch, its states kept on the tape (of a single step the checkpoint is
+    // the tape), then reversed in one launch
+    char* ck = (char*)h->ckpt.p + (size_t)seg * sb;
+    char* tp = s1 - s0 == 1 ? ck : (char*)tape.p;
+    if (s1 - s0 > 1) {
+      MixedState in = carve_mixed(ck, cn, false), last = carve_mixed(tp + (size_t)(s1 - s0 - 1) * sb, cn, false);
+      in.d = last.d = st.d;
+      p.nsteps = s1 - s0 - 1;
+      timer_begin(h, ST_TIMER_STEP, h->stream);
+      e = launch_step_mixed_tape(h, in, last, n, nullptr, p, tp, cn, 0, 1);
+      timer_end(h, ST_TIMER_STEP, h->stream, p.nsteps);
     }
-    for (int k = s1 - 1; k >= s0 && e == cudaSuccess; --k) {
-      AdjointMixedArgs a;
-      a.tape = carve_mixed((char*)tape.p + (size_t)(k - s0) * sb, cn, false);
-      a.d = st.d;
-      for (int q = 0; q < 3; ++q) {
-        a.xb[q] = A + q * cn;
-        a.vb[q] = A + (3 + q) * cn;
-      }
-      a.db = (double*)db.p;
-      a.ab_part = (double*)abp.p;
-      a.lam32 = (const float*)lam32.p;
-      a.Uw = (long long*)Uw.p;
-      a.dt = h->adj_dt;
-      timer_begin(h, ST_TIMER_ADJOINT, h->stream);
-      e = launch_adjoint_step_mixed(h, a);
-      timer_end(h, ST_TIMER_ADJOINT, h->stream);
+    AdjointMixedArgs a;
+    a.tape = tp;
+    a.tape_n = cn;
+    a.len = s1 - s0;
+    a.d = st.d;
+    for (int q = 0; q < 3; ++q) {
+      a.xb[q] = A + q * cn;
+      a.vb[q] = A + (3 + q) * cn;
     }
+    a.db = (double*)db.p;
+    a.ab = (double*)ab.p;
+    a.lam32 = (const float*)lam32.p;
+    a.Uw = (long long*)Uw.p;
+    a.dt = h->adj_dt;
+    timer_begin(h, ST_TIMER_ADJOINT, h->stream);
+    if (e == cudaSuccess) e = launch_adjoint_segment_mixed(h, a);
+    timer_end(h, ST_TIMER_ADJOINT, h->stream, s1 - s0);
   }
+  if (e == cudaSuccess) e = launch_ordered_sum(h, (const double*)ab.p, n, (double*)abp.p);
   std::vector<double> hab(kAdjBlocks);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(hab.data(), abp.p, kAdjBlocks * sizeof(double), cudaMemcpyDeviceToHost, h->stream);
@@ -930,19 +933,9 @@ static st_status adjoint_backward_mixed(st_handle h, const double* lam, int lam_
   if (grad_alpha) {
     double t = 0.0;
     for (int b = 0; b < kAdjBlocks; ++b) t += hab[b];
-    *grad_alpha = t;
+    *grad_alpha = t / h->alpha;
   }
   return ST_OK;
-}
-
-// the mixed state's first seven arrays (cell, offsets, velocities) at a stride of cap particles
-static cudaError_t copy_mixed7(const MixedState& dst, const MixedState& src, int64_t n, cudaStream_t st) {
-  cudaError_t e = cudaMemcpyAsync(dst.cell, src.cell, n * 4, cudaMemcpyDeviceToDevice, st);
-  for (int q = 0; q < 3 && e == cudaSuccess; ++q) {
-    e = cudaMemcpyAsync(dst.xi[q], src.xi[q], n * 4, cudaMemcpyDeviceToDevice, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(dst.v[q], src.v[q], n * 4, cudaMemcpyDeviceToDevice, st);
-  }
-  return e;
 }
 
 static int64_t round64(int64_t n) { return (n + 63) & ~int64_t(63); }
@@ -973,16 +966,13 @@ st_status st_adjoint_forward(st_handle h, int nsteps, double dt, int checkpoint_
   const double pi = 3.14159265358979323846;
   F64State s = carve_f64(h->state.p, h->cap);
   double* ck = (double*)h->ckpt.p;
-  const bool tape = fixed_step_supported(h);  // checkpoints written by the step kernel, several steps per launch
+  // checkpoints written by the step kernel, several steps per launch (not by the general FP64 kernel)
+  const bool tape = mixed || fixed_step_supported(h);
   for (int step = 0; step < nsteps;) {
     int m = 1;
     if (tape)
       m = (int)std::max(1.0, std::min({(double)(nsteps - step), (double)kMaxFusedSteps, 1073741824.0 / (double)n}));
-    if (mixed && step % checkpoint_every == 0) {
-      const MixedState slot = carve_mixed((char*)h->ckpt.p + (size_t)(step / checkpoint_every) * ck_bytes,
-                                          round64(n), false);
-      ST_TRY(cuda_check(h, copy_mixed7(slot, carve_mixed(h->state.p, h->cap, false), n, h->stream), "checkpoint"));
-    } else if (!tape && step % checkpoint_every == 0) {
+    if (!tape && step % checkpoint_every == 0) {
       double* slot = ck + (size_t)(step / checkpoint_every) * 6 * n;
       cudaError_t e = cudaSuccess;
       for (int q = 0; q < 3 && e == cudaSuccess; ++q) {
@@ -1006,13 +996,17 @@ st_status st_adjoint_forward(st_handle h, int nsteps, double dt, int checkpoint_
     timer_begin(h, ST_TIMER_STEP, h->stream);
     // mixed handles: the general kernel in storage order, which the backward pass recomputes with
     cudaError_t fe;
-    if (tape) {
-      const int slot = (step + checkpoint_every - 1) / checkpoint_every;  // the next checkpoint
+    const int slot = (step + checkpoint_every - 1) / checkpoint_every;  // the next checkpoint
+    if (mixed) {
+      const MixedState ms = carve_mixed(h->state.p, h->cap, false);
+      fe = launch_step_mixed_tape(h, ms, ms, n, (long long*)h->acc.p, p, (char*)h->ckpt.p + (size_t)slot * ck_bytes,
+                                  round64(n), slot * checkpoint_every - step, checkpoint_every);
+    } else if (tape) {
       const double* in[6] = {s.x[0], s.x[1], s.x[2], s.v[0], s.v[1], s.v[2]};
       fe = launch_step_f64_tape(h, in, s, (long long*)h->acc.p, p, ck + (size_t)slot * 6 * n,
                                 slot * checkpoint_every - step, checkpoint_every);
     } else {
-      fe = mixed ? launch_step_mixed(h, p) : launch_step_f64(h, p);
+      fe = launch_step_f64(h, p);
     }
     timer_end(h, ST_TIMER_STEP, h->stream, m);
     ST_TRY(cuda_check(h, fe, "adjoint forward step"));

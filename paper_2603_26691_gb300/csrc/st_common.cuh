@@ -463,7 +463,16 @@ __device__ __forceinline__ void wide_add(long long* w, double x) {
   if (q + 2 < kWideWords) atomicAdd((unsigned long long*)&w[q + 2], (unsigned long long)d2);
 }
 
-// v * 2^ex (an integer and an exponent) into the same accumulator; what lies below its grid is rounded off
+// FP32 to FP64 with integer operations: GB300 converts on its FP64 pipe, one warp instruction in 64 cycles.
+// Subnormal and non-finite values (rare) take the conversion.
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t b = __float_as_uint(x), e = b & 0x7f800000u;
+  if (__builtin_expect(e == 0 || e == 0x7f800000u, 0)) return (b << 1) == 0 ? __hiloint2double((int)b, 0) : (double)x;
+  return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
+}
+
+// m * 2^ex with a sign (an integer and an exponent) into the same accumulator; what lies below its grid is rounded
+// off.  m < 2^64, or < 2^128 in two halves.
 __device__ __forceinline__ void wide_add_int(long long* w, long long v, int ex) {
   unsigned long long m = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
   int s = ex - kWideBase;
@@ -478,6 +487,23 @@ __device__ __forceinline__ void wide_add_int(long long* w, long long v, int ex) 
   for (int k = 0; k < 3; ++k)
     if (d[k] != 0 && q + k < kWideWords)
       atomicAdd((unsigned long long*)&w[q + k], (unsigned long long)(v < 0 ? -d[k] : d[k]));
+}
+__device__ __forceinline__ void wide_add_int128(long long* w, __int128 v, int ex) {
+  const bool neg = v < 0;
+  unsigned __int128 m = neg ? -(unsigned __int128)v : (unsigned __int128)v;
+  int s = ex - kWideBase;
+  if (__builtin_expect(s < 0, 0)) {
+    m = s <= -128 ? 0 : (m >> -s) + ((m >> (-s - 1)) & 1);
+    s = 0;
+  }
+  const int q = s >> 5, r = s & 31;
+  const unsigned long long lo = (unsigned long long)m, hi = (unsigned long long)(m >> 64);
+  const unsigned long long t[3] = {lo << r, (hi << r) | ((lo >> 1) >> (63 - r)), (hi >> 1) >> (63 - r)};
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    const long long d = (long long)(uint32_t)(t[k >> 1] >> (32 * (k & 1)));
+    if (d != 0 && q + k < kWideWords) atomicAdd((unsigned long long*)&w[q + k], (unsigned long long)(neg ? -d : d));
+  }
 }
 
 // ---- sums over a warp's lanes of equal key, before one exact commit per key ----
@@ -577,23 +603,32 @@ cudaError_t launch_adjoint_segment(st_ctx* h, const AdjointStepArgs& s, int len)
 // the start of the step (cell, offsets, velocities; diameters in d), the adjoints of position and
 // velocity are FP32 arrays, dL/dd and dL/dalpha accumulate in FP64, dL/dU goes into the same exact
 // carry-save accumulator as the FP64 adjoint; lam32 = dL/dJtot per cell in FP32 [3][ncell]
+// (tape: the first state of a segment of len steps, their states 28 tape_n bytes apart; ab: dL/dalpha per
+// particle, times alpha)
 struct AdjointMixedArgs {
-  MixedState tape;
+  const void* tape;
+  int64_t tape_n;
+  int len;
   const float* d;
   float* xb[3];
   float* vb[3];
   double* db;
-  double* ab_part;
+  double* ab;
   const float* lam32;
   long long* Uw;
   double dt;
 };
-cudaError_t launch_adjoint_step_mixed(st_ctx* h, const AdjointMixedArgs& s);
+cudaError_t launch_adjoint_segment_mixed(st_ctx* h, const AdjointMixedArgs& s);
+// the sum of n doubles in a fixed order, as kAdjBlocks partial sums
+cudaError_t launch_ordered_sum(st_ctx* h, const double* in, int64_t n, double* part);
 cudaError_t launch_f64_to_f32(st_ctx* h, const double* in, float* out, int64_t m);
 cudaError_t launch_wide_to_f64(st_ctx* h, const long long* Uw, double* out, int64_t m);
 cudaError_t launch_step_mixed(st_ctx* h, const StepParams& p);
-// the general mixed step on any state of the handle's capacity layout; acc = nullptr deposits nothing
-cudaError_t launch_step_mixed_state(st_ctx* h, const MixedState& s, int64_t n, long long* acc, const StepParams& p);
+// the general mixed step from one state to another (they may be the same), p.nsteps of them; acc = nullptr
+// deposits nothing; the states before steps first, first + every, ... go on a tape (null: none), 28 tape_n
+// bytes each: cells, offsets, velocities (FP32) at a stride of tape_n particles
+cudaError_t launch_step_mixed_tape(st_ctx* h, const MixedState& in, const MixedState& s, int64_t n, long long* acc,
+                                   const StepParams& p, void* tape, int64_t tape_n, int first, int every);
 bool tma_step_supported(const st_ctx* h);                               // step_mixed_tma.cu
 // records = true (mixed handles, default physics): the new state goes out as 32-byte records into
 // state_alt (plus the cells into the structure of arrays) for the sort that follows; see

@@ -189,14 +189,6 @@ __global__ void export_f64_kernel(F64State s, const uint32_t* __restrict__ sid, 
   }
 }
 
-// FP32 to FP64 with integer operations: GB300 converts on its FP64 pipe, one warp in 64 cycles, and an export
-// has ten such values per particle.  Subnormal and non-finite values (rare) take the conversion.
-__device__ __forceinline__ double widen(float x) {
-  const uint32_t b = __float_as_uint(x), e = b & 0x7f800000u;
-  if (__builtin_expect(e == 0 || e == 0x7f800000u, 0)) return (b << 1) == 0 ? __hiloint2double((int)b, 0) : (double)x;
-  return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
-}
-
 // i + xi for a cell index 0 <= i < 1024 and an offset 0 <= xi < 1.  Offsets of at least 2^-20 (or 0) make it a
 // multiple of 2^-43 below 2^10, so the sum is exact: the 53-bit integer, normalised.  (Smaller ones
 // round in FP64.)

@@ -250,7 +250,7 @@ struct MixedArgs {
   long long* __restrict__ macc;
   float4* __restrict__ rec;        // the step before a sort: the new state as 32-byte records (else null)
   int64_t n, ncell;
-  int nx, ny, nz;
+  int nx, ny, nz, nsteps;
   float inv_h[3];
   float dt, inv_ca, g[3], gdt[3];
   int E;
@@ -405,18 +405,32 @@ __global__ void __launch_bounds__(kMicroThreads) micro_mixed_kernel(const MixedA
   const int px = a.nx + 2 * kFluidPad, pxy = (a.nx + 2 * kFluidPad) * (a.ny + 2 * kFluidPad);
   for (int64_t base = warp * 32; base < a.n; base += nwarp * 32) {
     const int64_t p = base + lane;
-    int key = -1;
-    float gain[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+    int32_t cell = 0;
+    float xi[3], v[3], dhi = 0.0f;
+    float4 st = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     if (p < a.n) {
-      int32_t cell = a.s.cell[p];
-      float xi[3], v[3];
+      cell = a.s.cell[p];
       for (int q = 0; q < 3; ++q) {
         xi[q] = a.s.xi[q][p];
         v[q] = load_v<BF16>(a, q, p);
       }
-      float dhi = a.s.d[p];
-      float4 st = a.ms[p];
-      micro_particle<BF16>(a, n3, px, pxy, cell, xi, v, dhi, st, key, gain);
+      dhi = a.s.d[p];
+      st = a.ms[p];
+    }
+    // the steps of a launch, the state in registers between them (4e7 droplets on 128^3, ten steps: 10.0 ms
+    // against 13.5 ms with 96 B of state in and out per step); each step's sums are those of a launch of its
+    // own, so the results do not depend on how the steps are split over launches
+    GroupBuf<5>& gb = perm[threadIdx.x >> 5];
+#pragma unroll 1
+    for (int step = 0; step < a.nsteps; ++step) {
+      int key = -1;
+      float gain[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+      if (p < a.n) micro_particle<BF16>(a, n3, px, pxy, cell, xi, v, dhi, st, key, gain);
+      group_by_key(gb, lane, key, gain);
+      const bool head = run_sums(lane, key, gain) && key >= 0;
+      micro_commit(a, gb, lane, head, key, gain);
+    }
+    if (p < a.n) {
       a.s.cell[p] = cell;
       if (a.rec) {
         // the cells stay in the arrays (the sort's keys); the state goes out as one 32-byte record
@@ -434,10 +448,6 @@ __global__ void __launch_bounds__(kMicroThreads) micro_mixed_kernel(const MixedA
       }
       a.ms[p] = st;
     }
-    GroupBuf<5>& gb = perm[threadIdx.x >> 5];
-    group_by_key(gb, lane, key, gain);
-    const bool head = run_sums(lane, key, gain) && key >= 0;
-    micro_commit(a, gb, lane, head, key, gain);
   }
 }
 
@@ -613,6 +623,7 @@ cudaError_t launch_micro_step(st_ctx* h, const StepParams& p, bool records) {
   const int64_t warps = (h->np + 31) / 32;
   const int blocks = blocks_for(warps * 32);
   if (h->prec == ST_FP64) {
+    if (p.nsteps != 1) return cudaErrorInvalidValue;
     F64Args a;
     a.s = carve_f64(h->state.p, h->cap);
     a.T = (double*)h->temp.p;
@@ -651,6 +662,7 @@ cudaError_t launch_micro_step(st_ctx* h, const StepParams& p, bool records) {
     a.nx = h->geo.n[0];
     a.ny = h->geo.n[1];
     a.nz = h->geo.n[2];
+    a.nsteps = p.nsteps;
     for (int q = 0; q < 3; ++q) {
       a.inv_h[q] = (float)h->geo.inv_h[q];
       a.g[q] = (float)p.g[q];
@@ -669,20 +681,21 @@ cudaError_t launch_micro_step(st_ctx* h, const StepParams& p, bool records) {
   return cudaGetLastError();
 }
 
-st_status micro_prepare_step(st_ctx* h, double dt) {
+st_status micro_prepare_steps(st_ctx* h, double dt, int nsteps) {
   // one step can grow d^2 by at most 8 D_v rho_v,max dt / rho_p (rho_sat >= 0): the diameter bound
   // the momentum accumulator's exponent is chosen from
   const double grow = 8.0 * h->mi_Dv * h->rv_max * dt / h->rho_p;
-  h->dmax = std::sqrt(h->dmax * h->dmax + grow);
+  for (int k = 0; k < nsteps; ++k) h->dmax = std::sqrt(h->dmax * h->dmax + grow);
   // each particle adds at most one digit to any word per step
-  if (h->micro_adds + (double)h->np > 1073741824.0) {
+  const double adds = (double)h->np * nsteps;
+  if (h->micro_adds + adds > 1073741824.0) {
     const int64_t m = 2 * h->geo.ncell;
     wide_normalize_kernel<<<blocks_for(m), kMicroThreads, 0, h->stream>>>((long long*)h->acc_micro.p, m);
     h->launches += 1;
     ST_TRY(cuda_check(h, cudaGetLastError(), "normalise microphysics sources"));
     h->micro_adds = 1.0;
   }
-  h->micro_adds += (double)h->np;
+  h->micro_adds += adds;
   return ST_OK;
 }
 

@@ -595,7 +595,7 @@ st_status run_steps(st_ctx* h, int nsteps, double dt) {
     if (tma) m = std::min(nsteps - s, kMaxFusedSteps);
     // (the kernels that commit every run by itself: at most as many contributions as one word can take between
     // propagations)
-    if (fixed_step_supported(h) || (h->prec != ST_FP64 && !h->micro_on && !tma))
+    if (fixed_step_supported(h) || (h->prec != ST_FP64 && !tma))
       m = (int)std::max(1.0, std::min({(double)(nsteps - s), (double)kMaxFusedSteps,
                                        1073741824.0 / (deposits_per_cell(h) * (double)h->np)}));
     if (h->reorder_every > 0) m = std::min(m, h->reorder_every - h->steps_since_sort);
@@ -611,7 +611,7 @@ st_status run_steps(st_ctx* h, int nsteps, double dt) {
       m -= 1;
     }
     if (!gather) ST_TRY(materialize_state(h));
-    if (h->micro_on) ST_TRY(micro_prepare_step(h, dt));
+    if (h->micro_on) ST_TRY(micro_prepare_steps(h, dt, m));
     int E = 0;
     // digits a launch can add to one word: a tile flush of each of the (at most 8) units that cover a cell,
     // at least one unit in 2^16 particle-steps; the other kernels one contribution per particle
@@ -635,7 +635,7 @@ st_status run_steps(st_ctx* h, int nsteps, double dt) {
     timer_begin(h, ST_TIMER_STEP, h->stream);
     if (h->micro_on) {
       // the step before a due sort leaves its output as records for the sort's gather
-      const bool mrec = h->prec != ST_FP64 && h->reorder_every > 0 && h->steps_since_sort + 1 >= h->reorder_every &&
+      const bool mrec = h->prec != ST_FP64 && h->reorder_every > 0 && h->steps_since_sort + m >= h->reorder_every &&
                         h->state_alt.bytes >= (size_t)h->cap * 32;
       e = launch_micro_step(h, p, mrec);
       if (e == cudaSuccess && mrec) h->records_pending = true;

@@ -698,9 +698,9 @@ cudaError_t launch_cell_counts(st_ctx* h, int64_t* counts);
 // the step with vapour mass and heat transfer (default physics only; accumulators prepared)
 // records (mixed handles): the new state as 32-byte records into state_alt (cells also into the arrays)
 cudaError_t launch_micro_step(st_ctx* h, const StepParams& p, bool records = false);
-// before a microphysics step: widen the diameter bound by the largest growth one step allows, and
-// propagate the carries of the microphysics accumulator when the step could overflow a word
-st_status micro_prepare_step(st_ctx* h, double dt);
+// before microphysics steps: widen the diameter bound by the largest growth they allow, and propagate the
+// carries of the microphysics accumulator when the steps could overflow a word
+st_status micro_prepare_steps(st_ctx* h, double dt, int nsteps);
 // the sort's permutation applied to the particle temperatures (temp -> temp_alt); gate as the sort's
 cudaError_t launch_gather_temp(st_ctx* h, const uint32_t* perm, const int* gate, int want);
 // the temperatures of particles [first, first + n) set to `T` (new particles, enabling microphysics)

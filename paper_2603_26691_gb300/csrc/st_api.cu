@@ -347,11 +347,16 @@ st_status st_set_fluid(st_handle h, const void* u, int dtype, int on_device) {
     }
     src = tmp.p;
   }
-  double umax = 0.0;
-  int nonfinite = 0;
-  cudaError_t e = launch_maxabs(h, src, h->geo.ncell * 3, dtype, &umax, &nonfinite);
-  if (e == cudaSuccess && !nonfinite) e = launch_fluid_pack(h, src, dtype);
+  // the scan, the padding (which skips on the scan's flag when a value is not finite) and the scan's result in
+  // one go: one wait for the device instead of two
+  unsigned long long red[2] = {0, 0};
+  cudaError_t e = launch_maxabs_on(h, src, h->geo.ncell * 3, dtype, h->stream, (unsigned long long*)h->red.p, nullptr);
+  if (e == cudaSuccess) e = launch_fluid_pack_if(h, src, dtype, (const int*)((unsigned long long*)h->red.p + 1));
+  if (e == cudaSuccess) e = cudaMemcpyAsync(red, h->red.p, 16, cudaMemcpyDeviceToHost, h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+  double umax = 0.0;
+  std::memcpy(&umax, &red[0], 8);
+  const int nonfinite = (int)(red[1] & 0xffffffffu);
   dev_free(h, tmp);
   ST_TRY(cuda_check(h, e, "set fluid"));
   if (nonfinite) return set_error(h, ST_ERR_NONFINITE, "fluid field holds NaN or Inf");
@@ -678,10 +683,11 @@ st_status st_get_sources(st_handle h, double* out, int reset, int on_device) {
   if (e == cudaSuccess && !on_device) e = cudaMemcpyAsync(out, dst, bytes, cudaMemcpyDeviceToHost, h->stream);
   if (e == cudaSuccess && reset) e = cudaMemsetAsync(h->acc.p, 0, h->acc.bytes, h->stream);
   if (e == cudaSuccess && reset) e = reset_acc_counter(h);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+  // the error flags' read waits for all of it
+  const st_status fs = e == cudaSuccess ? check_flags(h) : ST_OK;
   dev_free(h, tmp);
   ST_TRY(cuda_check(h, e, "get sources"));
-  ST_TRY(check_flags(h));
+  ST_TRY(fs);
   if (reset) {
     h->acc_empty = true;
     h->acc_load = 0.0;

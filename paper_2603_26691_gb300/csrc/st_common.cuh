@@ -656,13 +656,12 @@ cudaError_t launch_acc_sum(st_ctx* h, double out[3]);
 cudaError_t launch_particle_sums(st_ctx* h, double out[4]);  // P_x, P_y, P_z, M
 cudaError_t launch_maxabs(st_ctx* h, const void* p, int64_t n, int dtype, double* out_max, int* nonfinite);
 // the same scan on `stream`, its 16-byte result {max bits, flag} left in dev_red and copied to host_red
-// (pinned) asynchronously
+// (pinned; null: not copied) asynchronously
 cudaError_t launch_maxabs_on(st_ctx* h, const void* p, int64_t n, int dtype, cudaStream_t stream,
                              unsigned long long* dev_red, unsigned long long* host_red);
 cudaError_t launch_particle_scan(st_ctx* h, const double* vel, const double* d, int64_t n, double* vmax,
                                  double* dmax, double* dmin, int* nonfinite);
-cudaError_t launch_fluid_pack(st_ctx* h, const void* u, int dtype);
-// the same, skipped on the device when *skip != 0
+// u into the handle's field (padded or FP64 and integer), skipped on the device when *skip != 0
 cudaError_t launch_fluid_pack_if(st_ctx* h, const void* u, int dtype, const int* skip);
 cudaError_t launch_import(st_ctx* h, int64_t first, int64_t n, const double* xyz, const double* vel,
                           const double* d, const uint32_t* ids);

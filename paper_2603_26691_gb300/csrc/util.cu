@@ -26,21 +26,30 @@ __device__ __forceinline__ unsigned long long dbits(double x) { return (unsigned
 
 // ---- scans ----------------------------------------------------------------------------
 
+// the largest magnitude and whether all values are finite, on the values' bits: magnitudes are ordered like them,
+// and FP64 arithmetic (a conversion, a test and a maximum per value) would bind the scan to the FP64 pipe
+__device__ __forceinline__ uint32_t magnitude_bits(float v) { return __float_as_uint(v) & 0x7fffffffu; }
+__device__ __forceinline__ unsigned long long magnitude_bits(double v) { return dbits(v) & 0x7fffffffffffffffull; }
+__device__ __forceinline__ bool is_finite_bits(uint32_t b) { return b < 0x7f800000u; }
+__device__ __forceinline__ bool is_finite_bits(unsigned long long b) { return b < 0x7ff0000000000000ull; }
+__device__ __forceinline__ double magnitude(uint32_t b) { return (double)__uint_as_float(b); }
+__device__ __forceinline__ double magnitude(unsigned long long b) { return __longlong_as_double((long long)b); }
+
 template <typename T>
 __global__ void maxabs_kernel(const T* __restrict__ p, int64_t n, unsigned long long* out_bits, int* flag) {
-  double m = 0.0;
+  decltype(magnitude_bits(T())) m = 0;
   int bad = 0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    double v = (double)p[i];
-    if (!isfinite(v)) bad = 1;
-    else m = fmax(m, fabs(v));
+    const auto b = magnitude_bits(p[i]);
+    if (!is_finite_bits(b)) bad = 1;
+    else m = max(m, b);
   }
   for (int o = 16; o > 0; o >>= 1) {
-    m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+    m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
     bad |= __shfl_xor_sync(0xffffffffu, bad, o);
   }
   if ((threadIdx.x & 31) == 0) {
-    atomicMax(out_bits, dbits(m));
+    atomicMax(out_bits, dbits(magnitude(m)));
     if (bad) atomicOr(flag, 1);
   }
 }
@@ -462,8 +471,6 @@ cudaError_t launch_particle_scan(st_ctx* h, const double* xyz, const double* d, 
   return cudaSuccess;
 }
 
-cudaError_t launch_fluid_pack(st_ctx* h, const void* u, int dtype) { return launch_fluid_pack_if(h, u, dtype, nullptr); }
-
 cudaError_t launch_fluid_pack_if(st_ctx* h, const void* u, int dtype, const int* skip) {
   int64_t nc = h->geo.ncell;
   if (h->prec == ST_FP64) {
@@ -508,7 +515,7 @@ cudaError_t launch_maxabs_on(st_ctx* h, const void* p, int64_t n, int dtype, cud
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
-  return cudaMemcpyAsync(host_red, dev_red, 16, cudaMemcpyDeviceToHost, stream);
+  return host_red ? cudaMemcpyAsync(host_red, dev_red, 16, cudaMemcpyDeviceToHost, stream) : cudaSuccess;
 }
 
 cudaError_t launch_import(st_ctx* h, int64_t first, int64_t n, const double* xyz, const double* vel, const double* d,

@@ -368,10 +368,12 @@ st_status st_set_fluid(st_handle h, const void* u, int dtype, int on_device) {
   return ST_OK;
 }
 
-static st_status grow(st_handle h, int64_t need) {
+// exact: room for `need` particles and no more (a reservation, and the first particles of a handle); otherwise
+// geometrically, for particles that come in many calls
+static st_status grow(st_handle h, int64_t need, bool exact) {
   if (need <= h->cap) return ST_OK;
   ST_TRY(materialize_state(h));
-  int64_t cap = h->cap ? h->cap : 1024;
+  int64_t cap = exact || h->cap == 0 ? need : h->cap;
   while (cap < need) cap = cap + cap / 2 + 64;
   cap = (cap + 63) & ~int64_t(63);
   Buf ns, ni;
@@ -425,7 +427,7 @@ st_status st_reserve(st_handle h, int64_t capacity) {
   if (capacity < 0 || capacity > (int64_t(1) << 34)) return set_error(h, ST_ERR_INVALID_ARG, "capacity out of range");
   // a handle with chunks keeps its buffers at the chunk capacity (they are the chunks' device slots)
   if (h->chunks) return set_error(h, ST_ERR_STATE, "the handle holds chunks");
-  return grow(h, capacity);
+  return grow(h, capacity, true);
 }
 
 st_status st_add_particles(st_handle h, int64_t n, const double* xyz, const double* vel, const double* d,
@@ -491,7 +493,7 @@ st_status st_add_particles(st_handle h, int64_t n, const double* xyz, const doub
     cleanup();
     return set_error(h, ST_ERR_INVALID_ARG, "diameters must be > 0");
   }
-  st_status s = grow(h, h->np + n);
+  st_status s = grow(h, h->np + n, false);
   if (s != ST_OK) {
     cleanup();
     return s;

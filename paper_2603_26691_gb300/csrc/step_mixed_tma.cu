@@ -10,11 +10,11 @@
 //     (double-buffered across units), and streams the unit's particle arrays
 //     through a ring of shared-memory stages with 1-D bulk copies
 //     (cp.async.bulk), signalling completion on mbarriers;
-//   * consumer warps take 4 consecutive particles per lane from the stage,
+//   * consumer warps take kP consecutive particles per lane from the stage,
 //     gather the fluid velocity from the shared tile (8 LDS.128 with immediate
 //     offsets; particles that drifted out of the tile read the padded field
 //     from L2), advance and relocate them, reduce their impulses over runs of equal
-//     start-of-step cell across the warp, and store the new state with 128-bit
+//     start-of-step cell across the warp, and store the new state with wide
 //     streaming stores;
 //   * each run is added once to the unit's deposit tile with integer shared atomics (exact and
 //     independent of the order of the adds), which is flushed to the global carry-save fixed-point
@@ -23,9 +23,7 @@
 // up to the next sort on a stage before the next one (nsteps): the state, the diameter's coefficients, the
 // fluid tile and the deposit tile stay on the chip between them, and a step costs its arithmetic and its
 // deposit instead of 60 B of HBM traffic per particle.  The arithmetic and the grouping of the sums are those
-// of one step per launch, so the results do not depend on how the steps are split over calls.  Ten steps
-// at 5e8 particles on 256^3: 57.1 ms against 71.5 ms in ten launches; at 1e8 (BF16, 128^3) 10.2 against
-// 13.2 ms; cloud-in-cell at 2e7 10.9 against 14.4 ms.
+// of one step per launch, so the results do not depend on how the steps are split over calls.
 // The first step after a sort may also do that sort's payload gather (the GATHER instance): the sort
 // leaves a permutation and the previous step's 32-byte records {cell, offsets | velocity, diameter}
 // in the old order, and each consumer thread loads its own particles' records through the
@@ -54,14 +52,13 @@ using namespace ptx;
 constexpr int kU = 8;                       // unit edge (cells)
 constexpr int kG = 3;                       // fluid halo = padding of the field
 constexpr int kTE = kU + 2 * kG;            // fluid tile edge (14)
-constexpr int kConsumerWarps = 15;
-constexpr int kT = kConsumerWarps * 128;    // particles per stage (1920)
+constexpr int kP = 2;                       // consecutive particles per lane
+constexpr int kWarpParts = 32 * kP;
 constexpr int kStages = 2;
 constexpr int kR = 2;                      // deposit halo
 constexpr int kDE = kU + 2 * kR;           // deposit tile edge (12)
 constexpr int kDepositCells = kDE * kDE * kDE;  // 1728
-constexpr int kScanLanes = 8;              // runs are chained across at most this many lanes
-constexpr int kDirectRecords = 16;         // more run records than this per warp: commit in place
+constexpr int kScanLanes = 32 / kP;        // runs are chained across at most this many lanes
 constexpr int kDigits = 3;                 // 15-bit digits per value in the shared deposit tile
 constexpr int kDigitBits = 15;
 constexpr int kDepShift = 51;              // shared tile units = global units * 2^kDepShift
@@ -69,12 +66,25 @@ constexpr int kDepShift = 51;              // shared tile units = global units *
 // most 1 + 2^8 per particle of the run (one particle's impulse is below 2^38 tile units)
 constexpr int kDepMaxAdds = 131071;
 constexpr unsigned kNoKey = 0xffffffffu;   // no cell: neither a tile-form nor a far one
-constexpr int kThreads = (kConsumerWarps + 1) * 32;
 
-constexpr int kFluidBytes = kTE * kTE * kTE * 16;          // 43904
-constexpr int kStageBytes = kT * 32;                        // 61440 (FP32 layout; BF16 uses less)
+constexpr int kFluidBytes = kTE * kTE * kTE * 16;               // 43904
 constexpr int kDepositBytes = kDepositCells * 3 * kDigits * 4;  // 62208
-constexpr int kSmemBytes = kFluidBytes + kDepositBytes + kStages * kStageBytes + 16 * 8;  // 229128
+
+// The shape of an instance.  The steps run on what the registers let run at once: two particles per lane and 23
+// consumer warps at 80 registers hide more of the latency than four per lane and 15 warps at 128 (4e8
+// particles on 256^3, ten steps: 44.1 against 48.2 ms; with 19 warps 44.8 ms).  The physics variants need more
+// registers: 19 warps at 96 (cloud-in-cell at 2e7 on 128^3: 8.9 ms, with 23 warps 9.3, with four per lane 10.7).
+template <bool PHYS>
+struct Shape {
+  static constexpr int kConsumerWarps = PHYS ? 19 : 23;
+  static constexpr int kT = kConsumerWarps * kWarpParts;  // particles per stage
+  static constexpr int kThreads = (kConsumerWarps + 1) * 32;
+  static constexpr int kRegs = 65536 / kThreads / 8 * 8;
+  static constexpr int kStageBytes = kT * 32;             // the FP32 layout; BF16 uses less
+  static constexpr int kSmemBytes = kFluidBytes + kDepositBytes + kStages * kStageBytes + 16 * 8;
+  static_assert(kSmemBytes <= 232448, "shared memory of a block");
+  static_assert(kT * kMaxFusedSteps <= kDepMaxAdds, "a stage's deposits fit the digit words");
+};
 
 __device__ __forceinline__ void tma_load_tile(void* dst, const CUtensorMap* map, int c1, int c2, int c3,
                                               uint64_t* bar) {
@@ -420,54 +430,87 @@ __device__ __forceinline__ void commit_record(const TmaArgs& a, int* dep, unsign
     commit_far(a, c & ~kFarCell, r0, r1, r2);
 }
 
-// GATHER: the permutation entries of a lane's four sorted positions p0 .. p0 + 3 (p0 a multiple of
-// 4), zeros when it owns none of them within [S, E) (then p0 may lie past the buffer)
-__device__ __forceinline__ uint4 gather_perm(const TmaArgs& a, int64_t p0, int64_t S, int64_t E) {
-  const bool any = p0 + 4 > S && p0 < E;
-  return any ? __ldcs(reinterpret_cast<const uint4*>(a.perm + p0)) : make_uint4(0, 0, 0, 0);
+// a lane's kP consecutive 32-bit values as one access
+struct alignas(4 * kP) Vec32 {
+  uint32_t w[kP];
+};
+__device__ __forceinline__ void stcs(void* p, const Vec32& v) {
+  if constexpr (kP == 4)
+    __stcs(reinterpret_cast<uint4*>(p), make_uint4(v.w[0], v.w[1], v.w[2], v.w[kP - 1]));
+  else
+    __stcs(reinterpret_cast<uint2*>(p), make_uint2(v.w[0], v.w[1]));
 }
-// GATHER: the ids of the owned positions among p0 .. p0 + 3 through the permutation (0 elsewhere)
-__device__ __forceinline__ uint4 gather_ids(const TmaArgs& a, uint4 pp, int64_t p0, int64_t S, int64_t E) {
-  const uint32_t pj[4] = {pp.x, pp.y, pp.z, pp.w};
-  uint32_t id[4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) id[j] = (p0 + j >= S && p0 + j < E) ? __ldg(a.ids_in + pj[j]) : 0u;
-  return make_uint4(id[0], id[1], id[2], id[3]);
-}
-// GATHER: store ids gathered for positions p0 .. p0 + 3 (the owned ones)
-__device__ __forceinline__ void store_ids(const TmaArgs& a, uint4 id, int64_t p0, int64_t S, int64_t E) {
-  if (p0 >= S && p0 + 4 <= E) {
-    __stcs(reinterpret_cast<uint4*>(a.ids_out + p0), id);
+__device__ __forceinline__ Vec32 ldcs(const void* p) {
+  Vec32 v;
+  if constexpr (kP == 4) {
+    const uint4 q = __ldcs(reinterpret_cast<const uint4*>(p));
+    v.w[0] = q.x;
+    v.w[1] = q.y;
+    v.w[2 % kP] = q.z;
+    v.w[3 % kP] = q.w;
   } else {
-    const uint32_t v[4] = {id.x, id.y, id.z, id.w};
+    const uint2 q = __ldcs(reinterpret_cast<const uint2*>(p));
+    v.w[0] = q.x;
+    v.w[1] = q.y;
+  }
+  return v;
+}
+__device__ __forceinline__ Vec32 vec(const float (&f)[kP]) {
+  Vec32 v;
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
-      if (p0 + j >= S && p0 + j < E) a.ids_out[p0 + j] = v[j];
+  for (int j = 0; j < kP; ++j) v.w[j] = __float_as_uint(f[j]);
+  return v;
+}
+
+// GATHER: the permutation entries of a lane's sorted positions p0 .. p0 + kP - 1 (p0 a multiple of
+// kP), zeros when it owns none of them within [S, E) (then p0 may lie past the buffer)
+__device__ __forceinline__ Vec32 gather_perm(const TmaArgs& a, int64_t p0, int64_t S, int64_t E) {
+  return p0 + kP > S && p0 < E ? ldcs(a.perm + p0) : Vec32{};
+}
+// GATHER: the ids of the owned positions among p0 .. p0 + kP - 1 through the permutation (0 elsewhere)
+__device__ __forceinline__ Vec32 gather_ids(const TmaArgs& a, const Vec32& pp, int64_t p0, int64_t S, int64_t E) {
+  Vec32 id;
+#pragma unroll
+  for (int j = 0; j < kP; ++j) id.w[j] = (p0 + j >= S && p0 + j < E) ? __ldg(a.ids_in + pp.w[j]) : 0u;
+  return id;
+}
+// GATHER: store ids gathered for positions p0 .. p0 + kP - 1 (the owned ones)
+__device__ __forceinline__ void store_ids(const TmaArgs& a, const Vec32& id, int64_t p0, int64_t S, int64_t E) {
+  if (p0 >= S && p0 + kP <= E) {
+    stcs(a.ids_out + p0, id);
+  } else {
+#pragma unroll
+    for (int j = 0; j < kP; ++j)
+      if (p0 + j >= S && p0 + j < E) a.ids_out[p0 + j] = id.w[j];
   }
 }
-// GATHER: ask L2 for the records of the owned positions among p0 .. p0 + 3 (a stage before their
+// GATHER: ask L2 for the records of the owned positions among p0 .. p0 + kP - 1 (a stage before their
 // loads)
-__device__ __forceinline__ void gather_prefetch(const TmaArgs& a, uint4 pp, int64_t p0, int64_t S, int64_t E) {
-  const uint32_t pj[4] = {pp.x, pp.y, pp.z, pp.w};
+__device__ __forceinline__ void gather_prefetch(const TmaArgs& a, const Vec32& pp, int64_t p0, int64_t S, int64_t E) {
 #pragma unroll
-  for (int j = 0; j < 4; ++j)
-    if (p0 + j >= S && p0 + j < E) asm volatile("prefetch.global.L2 [%0];" ::"l"(a.grec + 2 * (int64_t)pj[j]));
+  for (int j = 0; j < kP; ++j)
+    if (p0 + j >= S && p0 + j < E) asm volatile("prefetch.global.L2 [%0];" ::"l"(a.grec + 2 * (int64_t)pp.w[j]));
 }
-// GATHER: the diameters of the owned positions among p0 .. p0 + 3, stored in sorted order as soon as
+// GATHER: the diameters of the owned positions among p0 .. p0 + kP - 1, stored in sorted order as soon as
 // their records arrive (a step does not change them)
-__device__ __forceinline__ void store_d(const TmaArgs& a, const Rec32 (&r)[4], int64_t p0, int64_t S, int64_t E) {
-  if (p0 >= S && p0 + 4 <= E) {
-    __stcs(reinterpret_cast<float4*>(a.s.d + p0), make_float4(r[0].d, r[1].d, r[2].d, r[3].d));
+__device__ __forceinline__ void store_d(const TmaArgs& a, const Rec32 (&r)[kP], int64_t p0, int64_t S, int64_t E) {
+  if (p0 >= S && p0 + kP <= E) {
+    Vec32 d;
+#pragma unroll
+    for (int j = 0; j < kP; ++j) d.w[j] = __float_as_uint(r[j].d);
+    stcs(a.s.d + p0, d);
   } else {
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
+    for (int j = 0; j < kP; ++j)
       if (p0 + j >= S && p0 + j < E) a.s.d[p0 + j] = r[j].d;
   }
 }
 
 template <bool BF16, bool REC, bool PHYS, bool GATHER>
-__global__ void __maxnreg__(128) step_mixed_tma_kernel(const __grid_constant__ CUtensorMap fluid_map,
+__global__ void __maxnreg__(Shape<PHYS>::kRegs) step_mixed_tma_kernel(const __grid_constant__ CUtensorMap fluid_map,
                                                        const __grid_constant__ TmaArgs a) {
+  constexpr int kConsumerWarps = Shape<PHYS>::kConsumerWarps, kT = Shape<PHYS>::kT;
+  constexpr int kStageBytes = Shape<PHYS>::kStageBytes;
   extern __shared__ __align__(128) unsigned char smem[];
   float4* fluid = reinterpret_cast<float4*>(smem);                               // [kTE^3]
   int* dep = reinterpret_cast<int*>(smem + kFluidBytes);                         // [3][kDigits][kDE^3]
@@ -569,7 +612,6 @@ __global__ void __maxnreg__(128) step_mixed_tma_kernel(const __grid_constant__ C
   const int px = a.nx + 2 * kG, pxy = (a.nx + 2 * kG) * (a.ny + 2 * kG);
   // stages whose deposits no digit word can overflow (a particle adds to a word at most once a step)
   const int flush_stages = kDepMaxAdds / (kT * a.nsteps);
-  static_assert(kT * kMaxFusedSteps <= kDepMaxAdds, "a stage's deposits fit the digit words");
   // tile index of a cell by its fields
   auto tile_index = [](unsigned c) {
     return (int)((c & 1023u) + kTE * ((c >> 10) & 1023u) + (kTE * kTE) * (c >> 20)) -
@@ -591,7 +633,7 @@ __global__ void __maxnreg__(128) step_mixed_tma_kernel(const __grid_constant__ C
     unit_origin(a, u, uo[0], uo[1], uo[2]);
     const int64_t A = S & ~int64_t(7);
     const int64_t Z = (E + 7) & ~int64_t(7);
-    const int L = 4 * ctid;
+    const int L = kP * ctid;
     // the deposit tile into the global accumulator, once every consumer warp has made its deposits
     auto flush = [&]() -> bool {
       __syncwarp();
@@ -631,7 +673,7 @@ __global__ void __maxnreg__(128) step_mixed_tma_kernel(const __grid_constant__ C
     };
     // GATHER: the permutation entries of this stage and of the next, and this stage's ids, are
     // held in registers a stage ahead
-    uint4 pcur = make_uint4(0, 0, 0, 0), pnext = make_uint4(0, 0, 0, 0), gid = make_uint4(0, 0, 0, 0);
+    Vec32 pcur{}, pnext{}, gid{};
     if constexpr (GATHER) {
       pcur = gather_perm(a, A + L, S, E);
       gid = gather_ids(a, pcur, A + L, S, E);
@@ -650,29 +692,28 @@ __global__ void __maxnreg__(128) step_mixed_tma_kernel(const __grid_constant__ C
         return;
       }
       ++gt;
-      const int64_t w0 = t0 + 128 * warp;  // a warp none of whose particles the unit owns has nothing to do
-      if (w0 >= E || w0 + 128 <= S) {
+      const int64_t w0 = t0 + kWarpParts * warp;  // a warp none of whose particles the unit owns has nothing to do
+      if (w0 >= E || w0 + kWarpParts <= S) {
         if (lane == 0) mbar_arrive(&empty[st]);
         continue;
       }
       unsigned char* src = ring + st * kStageBytes;
       const int64_t p0 = t0 + L;
-      // owned particles of this lane: [lo, hi) of 0..3 (the rest belong to neighbouring units
+      // owned particles of this lane: [lo, hi) of 0 .. kP - 1 (the rest belong to neighbouring units
       // or lie past the unit); the others are computed too, without branches, as harmless particles of the
       // unit's first cell without mass, and not stored
-      const int lo = (int)max((int64_t)0, min((int64_t)4, S - p0));
-      const int hi = (int)max((int64_t)0, min((int64_t)4, E - p0));
-      const bool all_own = lo == 0 && hi == 4;
-      int cell[4];
-      float xi[3][4], v[3][4], dv[4];
+      const int lo = (int)max((int64_t)0, min((int64_t)kP, S - p0));
+      const int hi = (int)max((int64_t)0, min((int64_t)kP, E - p0));
+      const bool all_own = lo == 0 && hi == kP;
+      int cell[kP];
+      float xi[3][kP], v[3][kP], dv[kP];
       if constexpr (GATHER) {
         // this stage's records through the permutation, one 256-bit load each (asked of L2 a stage
         // ago)
-        const uint32_t pj[4] = {pcur.x, pcur.y, pcur.z, pcur.w};
-        Rec32 r[4];
+        Rec32 r[kP];
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
-          r[j] = (j >= lo && j < hi) ? ld_rec32(a.grec + 2 * (int64_t)pj[j])
+        for (int j = 0; j < kP; ++j)
+          r[j] = (j >= lo && j < hi) ? ld_rec32(a.grec + 2 * (int64_t)pcur.w[j])
                                      : Rec32{0.0f, 0.5f, 0.5f, 0.5f, 0.0f, 0.0f, 0.0f, 1e-5f};
         // this stage's ids (loaded a stage ago) go out now; the next stage's come in, and its records
         // are asked for
@@ -685,7 +726,7 @@ __global__ void __maxnreg__(128) step_mixed_tma_kernel(const __grid_constant__ C
         }
         store_d(a, r, p0, S, E);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < kP; ++j) {
           cell[j] = __float_as_int(r[j].c);
           xi[0][j] = r[j].x0;
           xi[1][j] = r[j].x1;
@@ -696,46 +737,36 @@ __global__ void __maxnreg__(128) step_mixed_tma_kernel(const __grid_constant__ C
           dv[j] = r[j].d;
         }
       } else {
-        int4 c4 = *reinterpret_cast<const int4*>(src + L * 4);
-        cell[0] = c4.x;
-        cell[1] = c4.y;
-        cell[2] = c4.z;
-        cell[3] = c4.w;
+        const Vec32 c = *reinterpret_cast<const Vec32*>(src + L * 4);
+        const Vec32 dd = *reinterpret_cast<const Vec32*>(src + (BF16 ? 4 * kT * 4 + 3 * kT * 2 : 7 * kT * 4) + L * 4);
+#pragma unroll
+        for (int j = 0; j < kP; ++j) {
+          cell[j] = (int)c.w[j];
+          dv[j] = __uint_as_float(dd.w[j]);
+        }
+#pragma unroll
         for (int q = 0; q < 3; ++q) {
-          float4 x4 = *reinterpret_cast<const float4*>(src + (1 + q) * kT * 4 + L * 4);
-          xi[q][0] = x4.x;
-          xi[q][1] = x4.y;
-          xi[q][2] = x4.z;
-          xi[q][3] = x4.w;
-        }
-        if (BF16) {
-          for (int q = 0; q < 3; ++q) {
-            uint2 r = *reinterpret_cast<const uint2*>(src + 4 * kT * 4 + q * kT * 2 + L * 2);
-            float2 l = __bfloat1622float2(*reinterpret_cast<__nv_bfloat162*>(&r.x));
-            float2 h = __bfloat1622float2(*reinterpret_cast<__nv_bfloat162*>(&r.y));
-            v[q][0] = l.x;
-            v[q][1] = l.y;
-            v[q][2] = h.x;
-            v[q][3] = h.y;
-          }
-        } else {
-          for (int q = 0; q < 3; ++q) {
-            float4 r = *reinterpret_cast<const float4*>(src + 4 * kT * 4 + q * kT * 4 + L * 4);
-            v[q][0] = r.x;
-            v[q][1] = r.y;
-            v[q][2] = r.z;
-            v[q][3] = r.w;
+          const Vec32 x = *reinterpret_cast<const Vec32*>(src + (1 + q) * kT * 4 + L * 4);
+#pragma unroll
+          for (int j = 0; j < kP; ++j) xi[q][j] = __uint_as_float(x.w[j]);
+          if (BF16) {
+#pragma unroll
+            for (int j = 0; j < kP; j += 2) {
+              const float2 f = __bfloat1622float2(
+                  *reinterpret_cast<const __nv_bfloat162*>(src + 4 * kT * 4 + q * kT * 2 + (L + j) * 2));
+              v[q][j] = f.x;
+              v[q][j + 1] = f.y;
+            }
+          } else {
+            const Vec32 w = *reinterpret_cast<const Vec32*>(src + 4 * kT * 4 + q * kT * 4 + L * 4);
+#pragma unroll
+            for (int j = 0; j < kP; ++j) v[q][j] = __uint_as_float(w.w[j]);
           }
         }
-        float4 d4 = *reinterpret_cast<const float4*>(src + (BF16 ? 4 * kT * 4 + 3 * kT * 2 : 7 * kT * 4) + L * 4);
-        dv[0] = d4.x;
-        dv[1] = d4.y;
-        dv[2] = d4.z;
-        dv[3] = d4.w;
       }
       if (!all_own) {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < kP; ++j) {
           if (j >= lo && j < hi) continue;
           cell[j] = pack_cell(uo[0], uo[1], uo[2]);
           dv[j] = 1e-5f;
@@ -746,9 +777,9 @@ __global__ void __maxnreg__(128) step_mixed_tma_kernel(const __grid_constant__ C
           }
         }
       }
-      unsigned cl[4];  // the particles' cells in the form of local_cell()
+      unsigned cl[kP];  // the particles' cells in the form of local_cell()
 #pragma unroll
-      for (int j = 0; j < 4; ++j) cl[j] = local_cell(uo, n3, cell[j]);
+      for (int j = 0; j < kP; ++j) cl[j] = local_cell(uo, n3, cell[j]);
       // What the diameter alone decides is computed once and kept in the lane's own part of the stage (its
       // offsets and velocities, which are in registers now): e^{-a dt}, 1 - e^{-a dt}, 1 / a and the
       // mass; in the PHYS instance a dt, the diameter, 1 / a of Stokes drag and the mass.  (BF16
@@ -756,7 +787,7 @@ __global__ void __maxnreg__(128) step_mixed_tma_kernel(const __grid_constant__ C
       float* coef = reinterpret_cast<float*>(src) + kT + L;  // [3][kT]
       float* mass = reinterpret_cast<float*>(src + (BF16 ? 26 : 16) * kT) + L;
 #pragma unroll
-      for (int jp = 0; jp < 4; jp += 2) {
+      for (int jp = 0; jp < kP; jp += 2) {
         const unsigned long long D = pack2(dv[jp], dv[jp + 1]);
         const unsigned long long DD = mul2(D, D);
         float dd0, dd1, m[2];
@@ -785,10 +816,10 @@ __global__ void __maxnreg__(128) step_mixed_tma_kernel(const __grid_constant__ C
       // the padded field and commit to the global accumulator.
 #pragma unroll 1
       for (int step = 0; step < a.nsteps; ++step) {
-        unsigned key[4];  // the step's start cells
-        float J[4][3];
+        unsigned key[kP];  // the step's start cells
+        float J[kP][3];
 #pragma unroll
-        for (int jp = 0; jp < 4; jp += 2) {
+        for (int jp = 0; jp < kP; jp += 2) {
           float up[2][3], f[2][3];
           unsigned bs[2];  // the stencil's base cell
 #pragma unroll
@@ -977,23 +1008,24 @@ __global__ void __maxnreg__(128) step_mixed_tma_kernel(const __grid_constant__ C
         if (!(PHYS && a.cic)) {
           // ---- deposit: runs of equal key over the warp's 128 particles (lane-local suffix sums, then a
           // segmented suffix scan across lanes chains runs that span lanes) ----
-          float Sx[4][3];
+          float Sx[kP][3];
 #pragma unroll
-          for (int q = 0; q < 3; ++q) Sx[3][q] = J[3][q];
+          for (int q = 0; q < 3; ++q) Sx[kP - 1][q] = J[kP - 1][q];
+          int tail = kP - 1;  // the first particle of the run that ends the lane
 #pragma unroll
-          for (int j = 2; j >= 0; --j) {
+          for (int j = kP - 2; j >= 0; --j) {
             const bool same = key[j] == key[j + 1];
+            if (same && tail == j + 1) tail = j;
 #pragma unroll
             for (int q = 0; q < 3; ++q) Sx[j][q] = J[j][q] + (same ? Sx[j + 1][q] : 0.0f);
           }
-          const int tail = (key[2] != key[3]) ? 3 : (key[1] != key[2]) ? 2 : (key[0] != key[1]) ? 1 : 0;
           const unsigned nk0 = __shfl_down_sync(0xffffffffu, key[0], 1);
           const int nall = __shfl_down_sync(0xffffffffu, (int)(tail == 0), 1);
           float R[3];
 #pragma unroll
           for (int q = 0; q < 3; ++q) R[q] = __shfl_down_sync(0xffffffffu, Sx[0][q], 1);
           const int glane = lane & (kScanLanes - 1);
-          const bool link = (glane < kScanLanes - 1) && (nk0 == key[3]) && (key[3] != kNoKey);
+          const bool link = (glane < kScanLanes - 1) && (nk0 == key[kP - 1]) && (key[kP - 1] != kNoKey);
           int Bl = (link && nall) ? 1 : 0;
 #pragma unroll
           for (int q = 0; q < 3; ++q) R[q] = link ? R[q] : 0.0f;
@@ -1017,97 +1049,67 @@ __global__ void __maxnreg__(128) step_mixed_tma_kernel(const __grid_constant__ C
               Bl &= tb;
             }
           }
-          const unsigned pk3 = __shfl_up_sync(0xffffffffu, key[3], 1);
+          const unsigned pk3 = __shfl_up_sync(0xffffffffu, key[kP - 1], 1);
           const bool head_lane = (glane == 0) || (pk3 != key[0]);
-          // the run sums, one {J, key} record per run.  Few runs (after a sort): the records are packed
-          // in (j, lane) order into the warp's own (already consumed) part of the stage's cell array and
-          // each lane takes one record, so the whole deposit is one pass.  Many runs (particles drifted away from their
-          // sort-time cells): each lane commits its runs where they are, one pass per particle slot,
-          // without the round trip through shared memory.
-          bool starts[4];
-          unsigned hms[4];
-          int nh = 0;
+          // each lane commits its run sums where they are, one pass per particle slot.  (Packing the sums of
+          // few runs, fresh after a sort, into one pass through shared memory gains nothing: ten steps of 6e7
+          // particles on 128^3 took 7.01 ms with it and 6.93 ms without.)
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            starts[j] = ((j == 0) ? head_lane : (key[j] != key[j - 1])) && key[j] != kNoKey;
-            hms[j] = __ballot_sync(0xffffffffu, starts[j]);
-            nh += __popc(hms[j]);
-          }
-          if (nh > kDirectRecords) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              if (starts[j]) {
-                const bool to_end = j == tail;
-                const float r0 = Sx[j][0] + (to_end ? R[0] : 0.0f);
-                const float r1 = Sx[j][1] + (to_end ? R[1] : 0.0f);
-                const float r2 = Sx[j][2] + (to_end ? R[2] : 0.0f);
-                commit_record(a, dep, key[j], r0, r1, r2);
-              }
+          for (int j = 0; j < kP; ++j) {
+            const bool start = ((j == 0) ? head_lane : (key[j] != key[j - 1])) && key[j] != kNoKey;
+            if (start) {
+              const bool to_end = j == tail;
+              commit_record(a, dep, key[j], Sx[j][0] + (to_end ? R[0] : 0.0f), Sx[j][1] + (to_end ? R[1] : 0.0f),
+                            Sx[j][2] + (to_end ? R[2] : 0.0f));
             }
-          } else {
-            int* rj0 = reinterpret_cast<int*>(src) + warp * 128;
-            int* rj1 = rj0 + kDirectRecords;
-            int* rj2 = rj0 + 2 * kDirectRecords;
-            int* rk = rj0 + 3 * kDirectRecords;
-            const unsigned lt_mask = (1u << lane) - 1u;
-            int base = 0;
-            __syncwarp();
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              if (starts[j]) {
-                const bool to_end = j == tail;
-                const int slot = base + __popc(hms[j] & lt_mask);
-                rj0[slot] = __float_as_int(Sx[j][0] + (to_end ? R[0] : 0.0f));
-                rj1[slot] = __float_as_int(Sx[j][1] + (to_end ? R[1] : 0.0f));
-                rj2[slot] = __float_as_int(Sx[j][2] + (to_end ? R[2] : 0.0f));
-                rk[slot] = (int)key[j];
-              }
-              base += __popc(hms[j]);
-            }
-            __syncwarp();
-            if (lane < nh)
-              commit_record(a, dep, (unsigned)rk[lane], __int_as_float(rj0[lane]), __int_as_float(rj1[lane]),
-                            __int_as_float(rj2[lane]));
           }
         }
       }
 #pragma unroll
-      for (int j = 0; j < 4; ++j) cell[j] = global_cell(uo, n3, cl[j]);
-      // ---- store the owned particles (128-bit when the lane owns all four) ----
+      for (int j = 0; j < kP; ++j) cell[j] = global_cell(uo, n3, cl[j]);
+      // ---- store the owned particles (one wide store per array when the lane owns all) ----
       if (REC) {
         // the step before a sort: the cells to the structure of arrays (the sort's keys), the whole
         // state as 32-byte records {cell, offsets | velocity, diameter}, one 256-bit store per
         // particle (a full sector; the sort's gather then reads one sector per particle).  The
         // diameters are read again from the stage.  BF16 handles store the (BF16-exact) velocities
         // as FP32 in the record.
-        const float4 d4 =
-            *reinterpret_cast<const float4*>(src + (BF16 ? 4 * kT * 4 + 3 * kT * 2 : 7 * kT * 4) + L * 4);
-        const float dj[4] = {d4.x, d4.y, d4.z, d4.w};
-        if (all_own) __stcs((int4*)(a.s.cell + p0), make_int4(cell[0], cell[1], cell[2], cell[3]));
+        const Vec32 d = *reinterpret_cast<const Vec32*>(src + (BF16 ? 4 * kT * 4 + 3 * kT * 2 : 7 * kT * 4) + L * 4);
+        if (all_own) {
+          Vec32 c;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+          for (int j = 0; j < kP; ++j) c.w[j] = (uint32_t)cell[j];
+          stcs(a.s.cell + p0, c);
+        }
+#pragma unroll
+        for (int j = 0; j < kP; ++j) {
           if (j < lo || j >= hi) continue;
           if (!all_own) a.s.cell[p0 + j] = cell[j];
-          st_rec32(a.rec + 2 * (p0 + j),
-                   Rec32{__int_as_float(cell[j]), xi[0][j], xi[1][j], xi[2][j], v[0][j], v[1][j], v[2][j], dj[j]});
+          st_rec32(a.rec + 2 * (p0 + j), Rec32{__int_as_float(cell[j]), xi[0][j], xi[1][j], xi[2][j], v[0][j], v[1][j],
+                                               v[2][j], __uint_as_float(d.w[j])});
         }
       } else if (all_own) {
-        __stcs((int4*)(a.s.cell + p0), make_int4(cell[0], cell[1], cell[2], cell[3]));
-        for (int q = 0; q < 3; ++q)
-          __stcs((float4*)(a.s.xi[q] + p0), make_float4(xi[q][0], xi[q][1], xi[q][2], xi[q][3]));
+        Vec32 c;
+#pragma unroll
+        for (int j = 0; j < kP; ++j) c.w[j] = (uint32_t)cell[j];
+        stcs(a.s.cell + p0, c);
+#pragma unroll
         for (int q = 0; q < 3; ++q) {
+          stcs(a.s.xi[q] + p0, vec(xi[q]));
           if (BF16) {
             // exact: the velocities are BF16 values
-            const __nv_bfloat162 l = __floats2bfloat162_rn(v[q][0], v[q][1]), h = __floats2bfloat162_rn(v[q][2], v[q][3]);
-            __stcs((uint2*)((__nv_bfloat16*)a.s.v[q] + p0),
-                   make_uint2(*reinterpret_cast<const unsigned*>(&l), *reinterpret_cast<const unsigned*>(&h)));
+#pragma unroll
+            for (int j = 0; j < kP; j += 2) {
+              const __nv_bfloat162 b = __floats2bfloat162_rn(v[q][j], v[q][j + 1]);
+              __stcs((unsigned*)((__nv_bfloat16*)a.s.v[q] + p0 + j), *reinterpret_cast<const unsigned*>(&b));
+            }
           } else {
-            __stcs((float4*)((float*)a.s.v[q] + p0), make_float4(v[q][0], v[q][1], v[q][2], v[q][3]));
+            stcs((float*)a.s.v[q] + p0, vec(v[q]));
           }
         }
       } else {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < kP; ++j) {
           if (j < lo || j >= hi) continue;
           a.s.cell[p0 + j] = cell[j];
           for (int q = 0; q < 3; ++q) {
@@ -1173,9 +1175,11 @@ cudaError_t launch_step_mixed_tma(st_ctx* h, const StepParams& p, bool records, 
   static std::atomic<bool> attr_set[kAttrDevices][8];
   const int variant = (int)bf + 2 * (gather ? 3 : records ? 2 : (int)phys);
   const Kern kern = table[variant];
+  const int threads = phys ? Shape<true>::kThreads : Shape<false>::kThreads;
+  const int smem = phys ? Shape<true>::kSmemBytes : Shape<false>::kSmemBytes;
   if (h->dev < 0 || h->dev >= kAttrDevices) return cudaErrorInvalidDevice;
   if (!attr_set[h->dev][variant].load(std::memory_order_acquire)) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     attr_set[h->dev][variant].store(true, std::memory_order_release);
   }
@@ -1241,7 +1245,7 @@ cudaError_t launch_step_mixed_tma(st_ctx* h, const StepParams& p, bool records, 
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->dev);
   int grid = sms > 0 ? sms : 152;
   if (grid > a.nunits) grid = a.nunits;
-  kern<<<grid, kThreads, kSmemBytes, h->stream>>>(map, a);
+  kern<<<grid, threads, smem, h->stream>>>(map, a);
   h->launches += 1;
   return cudaGetLastError();
 }

@@ -278,6 +278,7 @@ st_status st_chunks_step(st_handle h, int nsteps, double dt, double* ms) {
     h->steps_since_sort = 0;
     h->records_pending = false;
     h->perm_pending = false;
+    h->cells_apart = false;
     cudaEvent_t a = ev(), b = ev();
     cudaEventRecord(a, comp);
     st = run_steps(h, nsteps, dt);

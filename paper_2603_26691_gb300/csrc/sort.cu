@@ -503,11 +503,12 @@ __global__ void gather_records_kernel(const float4* __restrict__ rec, MixedState
   }
 }
 
-// Records back to the structure of arrays in place of a sort (the cells are already there).
+// Records back to the structure of arrays in place of a sort.
 template <bool BF16>
 __global__ void records_to_soa_kernel(const float4* __restrict__ rec, MixedState dst, int64_t n) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const float4 a = rec[2 * i], b = rec[2 * i + 1];
+    dst.cell[i] = __float_as_int(a.x);
     dst.xi[0][i] = a.y;
     dst.xi[1][i] = a.z;
     dst.xi[2][i] = a.w;
@@ -856,6 +857,10 @@ st_status sort_particles(st_ctx* h) {
   if (ensure(h, h->cell_start, ((size_t)h->nkeys + 1) * sizeof(uint32_t)) != ST_OK) return ST_ERR_OOM;
   if (ensure(h, h->state_alt, state_alt_bytes(h->prec, h->cap)) != ST_OK) return ST_ERR_OOM;
   if (ensure(h, h->ids_alt, (size_t)h->cap * sizeof(uint32_t)) != ST_OK) return ST_ERR_OOM;
+  // (without room for the cells apart, the last step before a sort is a launch of its own; while they are in
+  // use the buffer has its size)
+  if (h->prec != ST_FP64 && !h->cells_apart && ensure(h, h->rec_cell, (size_t)h->cap * sizeof(int32_t)) != ST_OK)
+    h->err.clear();
   if (h->hist.p != look_before || h->sort_epoch + kMaxPasses >= (1u << 30)) {
     // a new look-back buffer may hold anything, and once the 30-bit epoch tags are about to repeat
     // an old word could carry a current tag: clear the words so that no stale word carries an epoch
@@ -893,7 +898,7 @@ st_status sort_particles(st_ctx* h) {
                      (unsigned long long*)h->hist.p, &h->sort_epoch, (int*)h->flags.p, sms, h->stream, &h->launches,
                      true);
   } else {
-    CellKeys src{(const int32_t*)h->state.p, g};
+    CellKeys src{current_cells(h), g};
     e = radix_passes(src, n, h->key_bits, k0, v0, k1, v1, k0, v0, totals, offs, tile_ctr,
                      (unsigned long long*)h->hist.p, &h->sort_epoch, (int*)h->flags.p, sms, h->stream, &h->launches,
                      true, gate);
@@ -936,10 +941,12 @@ st_status sort_particles(st_ctx* h) {
     if (e != cudaSuccess) return cuda_check(h, e, "sort temperatures");
     std::swap(h->temp, h->temp_alt);
   }
-  if (h->records_pending)
+  if (h->records_pending) {
     h->records_pending = false;
-  else
+    h->cells_apart = false;
+  } else {
     std::swap(h->state, h->state_alt);
+  }
   std::swap(h->ids, h->ids_alt);
   return ST_OK;
 }
@@ -954,21 +961,25 @@ static st_status run_deferred_gather(st_ctx* h) {
   h->launches += 1;
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_check(h, e, "deferred sort gather");
-  std::swap(h->ids, h->ids_alt);
-  h->perm_pending = false;
-  h->records_pending = false;
+  gather_step_done(h);
   return ST_OK;
 }
 
 bool defer_gather(const st_ctx* h) {
-  return h->prec != ST_FP64 && !h->micro_on && default_physics(h) && tma_step_supported(h) &&
-         h->reorder_every != 1 && h->np > 0;
+  return h->prec != ST_FP64 && !h->micro_on && tma_step_supported(h) && h->np > 0;
 }
 
 void gather_step_done(st_ctx* h) {
   std::swap(h->ids, h->ids_alt);
   h->perm_pending = false;
   h->records_pending = false;
+  h->cells_apart = false;
+}
+
+void records_written(st_ctx* h, bool apart) {
+  h->records_pending = true;
+  h->cells_apart = apart;
+  if (apart) std::swap(h->state, h->state_alt);
 }
 
 st_status materialize_state(st_ctx* h) {
@@ -979,6 +990,7 @@ st_status materialize_state(st_ctx* h) {
       (const float4*)h->state_alt.p, carve_mixed(h->state.p, h->cap, bf), h->np);
   h->launches += 1;
   h->records_pending = false;
+  h->cells_apart = false;
   return cuda_check(h, cudaGetLastError(), "records to arrays");
 }
 

@@ -398,15 +398,15 @@ cudaError_t launch_local_sort(st_ctx* h, int* far, uint32_t* lidx, uint16_t* lke
   uint32_t* total = rel + (size_t)g.nunits * kDirs;
   uint32_t* base = total + g.nunits;
   const uint32_t* cs_old = (const uint32_t*)h->cell_start.p;
-  const MixedState cur = carve_mixed(h->state.p, h->cap, h->prec == ST_MIXED_BF16V);
+  const int32_t* cells = current_cells(h);
   cudaStream_t s = h->stream;
   cudaError_t e = cudaMemsetAsync(far, 0, sizeof(int), s);
   if (e != cudaSuccess) return e;
   const int ublocks = std::min(g.nunits, 152 * 8);
-  usort_count_kernel<<<ublocks, kLThreads, 0, s>>>(cur.cell, cs_old, g, cnt, cntw, far);
+  usort_count_kernel<<<ublocks, kLThreads, 0, s>>>(cells, cs_old, g, cnt, cntw, far);
   usort_dest_kernel<<<(g.nunits + 127) / 128, 128, 0, s>>>(g, cnt, rel, total);
   usort_scan_kernel<<<1, 1024, 0, s>>>(total, g.nunits, base);
-  usort_scatter_kernel<<<ublocks, kLThreads, 0, s>>>(cur.cell, cs_old, g, cntw, rel, base, lidx, lkey, far);
+  usort_scatter_kernel<<<ublocks, kLThreads, 0, s>>>(cells, cs_old, g, cntw, rel, base, lidx, lkey, far);
   // rank: as many blocks as are resident at once (its registers allow three of 512 threads per SM),
   // each taking every grid-th unit, so that no block waits for a second wave
   int sms = 152, per_sm = 1;

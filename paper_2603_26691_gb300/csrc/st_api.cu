@@ -188,7 +188,7 @@ void st_destroy(st_handle h) {
   cudaStreamSynchronize(h->stream);
   chunk_store_free(h);  // its slot buffers first: the handle's own are freed below
   xfer_free(h);
-  Buf* bufs[] = {&h->fluid, &h->fluid_fix, &h->fluid_fix_next, &h->fluid_pad, &h->flags, &h->ckpt, &h->state, &h->state_alt, &h->ids, &h->ids_alt,
+  Buf* bufs[] = {&h->fluid, &h->fluid_fix, &h->fluid_fix_next, &h->fluid_pad, &h->flags, &h->ckpt, &h->state, &h->state_alt, &h->rec_cell, &h->ids, &h->ids_alt,
                  &h->keys[0], &h->keys[1], &h->vals[0], &h->vals[1], &h->hist, &h->scan_aux, &h->cell_start, &h->lsort_aux,
                  &h->acc, &h->red, &h->src_hist[0], &h->src_hist[1], &h->src_hist[2], &h->src_hist[3],
                  &h->src_est, &h->fl_cur, &h->fl_next, &h->fl_star, &h->fl_tmp, &h->fluid_pad_next, &h->umax_dev,
@@ -607,13 +607,14 @@ st_status run_steps(st_ctx* h, int nsteps, double dt) {
                                        1073741824.0 / (deposits_per_cell(h) * (double)h->np)}));
     if (h->reorder_every > 0) m = std::min(m, h->reorder_every - h->steps_since_sort);
     // a sort is due after these steps: they leave the state as records for its gather
-    const bool can_record = tma && default_physics(h) && h->reorder_every > 0 && h->state_alt.bytes >= (size_t)h->cap * 32;
+    const bool can_record = tma && h->reorder_every > 0 && h->state_alt.bytes >= (size_t)h->cap * 32;
     bool records = can_record && h->steps_since_sort + m >= h->reorder_every;
-    // a sort that deferred its payload gather: these steps gather, unless it is another kernel; the records
-    // they read are where new ones would go, so the last step before a sort is then a launch of its own
-    // (a single step has the gather run first)
-    const bool gather = h->perm_pending && tma && default_physics(h) && !(records && m == 1);
-    if (gather && records) {
+    // a sort that deferred its payload gather: these steps gather, unless it is another kernel.  Where they
+    // write records too, those need the room of the stale state and the cells a place of their own; without
+    // it the last step before a sort is a launch of its own (a single step has the gather run first)
+    const bool apart = h->rec_cell.bytes >= (size_t)h->cap * sizeof(int32_t) && h->state.bytes >= (size_t)h->cap * 32;
+    const bool gather = h->perm_pending && tma && (apart || !(records && m == 1));
+    if (gather && records && !apart) {
       records = false;
       m -= 1;
     }
@@ -652,7 +653,7 @@ st_status run_steps(st_ctx* h, int nsteps, double dt) {
     else if (tma) {
       e = launch_step_mixed_tma(h, p, records, gather);
       if (e == cudaSuccess && gather) gather_step_done(h);
-      if (e == cudaSuccess && records) h->records_pending = true;
+      if (e == cudaSuccess && records) records_written(h, gather);
     }
     else
       e = launch_step_mixed(h, p);
@@ -833,6 +834,7 @@ st_status st_clear_particles(st_handle h) {
   h->np = 0;
   h->records_pending = false;
   h->perm_pending = false;
+  h->cells_apart = false;
   h->sorted = false;
   h->steps_since_sort = 0;
   h->dmax = 0.0;

@@ -98,6 +98,10 @@ struct st_ctx {
   // the old order and the ids in `ids`.  The next sorted step gathers; any other reader calls
   // materialize_state, which runs the gather.
   bool perm_pending = false;
+  // Where the steps that gather also write records, the new ones go into `state` and the two buffers are
+  // swapped; the cells (the next sort's keys) then lie in rec_cell and `state` holds nothing current.
+  bool cells_apart = false;
+  st::Buf rec_cell;          // int32[cap] (mixed handles; null: given up for memory)
 
   // kernel timers (st_timers_*): pending event pairs per kind, folded into sums on read
   bool timing = false;
@@ -634,7 +638,8 @@ bool tma_step_supported(const st_ctx* h);                               // step_
 // state_alt (plus the cells into the structure of arrays) for the sort that follows; see
 // records_pending
 // gather = true: the first step after a sort whose payload gather was deferred (perm_pending); it reads
-// the records through the permutation and writes the sorted state, diameters and ids included
+// the records through the permutation and writes the sorted state, diameters and ids included.  Both: the
+// records go into `state`, the cells into rec_cell (records_written swaps the buffers)
 cudaError_t launch_step_mixed_tma(st_ctx* h, const StepParams& p, bool records, bool gather);  // step_mixed_tma.cu
 cudaError_t launch_rescale_acc(st_ctx* h, int shift);
 cudaError_t launch_normalize_acc(st_ctx* h);
@@ -681,11 +686,16 @@ size_t local_sort_aux_bytes(const st_ctx* h);
 cudaError_t launch_local_sort(st_ctx* h, int* far, uint32_t* lidx, uint16_t* lkey, uint32_t* perm, void* aux);
 // the structure of arrays current again if the last step left records for a sort (no-op otherwise)
 st_status materialize_state(st_ctx* h);                                    // sort.cu
-// whether a sort may leave its payload gather to the next step (mixed, sorted-step kernel, default
-// physics, no microphysics, and the next step does not itself write records), and the bookkeeping
-// once that step has gathered (ids swapped, nothing pending)
+// whether a sort may leave its payload gather to the next step (mixed, sorted-step kernel, no
+// microphysics), and the bookkeeping once that step has gathered (ids swapped, nothing pending) and once a
+// step has written records (apart: while it gathered)
 bool defer_gather(const st_ctx* h);                                        // sort.cu
 void gather_step_done(st_ctx* h);                                          // sort.cu
+void records_written(st_ctx* h, bool apart);                               // sort.cu
+// the packed cells of a mixed handle's particles in storage order, current also while records are pending
+inline const int32_t* current_cells(const st_ctx* h) {
+  return (const int32_t*)(h->cells_apart ? h->rec_cell.p : h->state.p);
+}
 // FP64 and FP32 FMA rates of this GPU (GFLOP/s), measured by FMA-chain kernels; synchronises
 cudaError_t probe_fma_rates(st_ctx* h, double* fp64_gflops, double* fp32_gflops);  // util.cu
 // timer marks around a launch of kind k on stream s (no-ops unless st_timers_enable is on); the

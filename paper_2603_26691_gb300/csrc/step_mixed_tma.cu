@@ -724,7 +724,15 @@ __global__ void __maxnreg__(Shape<PHYS>::kRegs) step_mixed_tma_kernel(const __gr
           pcur = pnext;
           pnext = gather_perm(a, p0 + 2 * kT, S, E);
         }
-        store_d(a, r, p0, S, E);
+        if (REC) {
+          // the diameters into the stage, from where the records take them
+          Vec32 d;
+#pragma unroll
+          for (int j = 0; j < kP; ++j) d.w[j] = __float_as_uint(r[j].d);
+          *reinterpret_cast<Vec32*>(src + (BF16 ? 4 * kT * 4 + 3 * kT * 2 : 7 * kT * 4) + L * 4) = d;
+        } else {
+          store_d(a, r, p0, S, E);
+        }
 #pragma unroll
         for (int j = 0; j < kP; ++j) {
           cell[j] = __float_as_int(r[j].c);
@@ -1160,20 +1168,22 @@ bool tma_step_supported(const st_ctx* h) {
 cudaError_t launch_step_mixed_tma(st_ctx* h, const StepParams& p, bool records, bool gather) {
   const bool bf = h->prec == ST_MIXED_BF16V;
   const bool phys = p.ngp || p.semi || p.sn || p.cic;
-  if ((records || gather) && phys) return cudaErrorInvalidValue;
-  if (records && gather) return cudaErrorInvalidValue;
   if (p.nsteps < 1 || p.nsteps > kMaxFusedSteps) return cudaErrorInvalidValue;
   using Kern = void (*)(const CUtensorMap, const TmaArgs);
-  static const Kern table[8] = {
+  static const Kern table[16] = {
       step_mixed_tma_kernel<false, false, false, false>, step_mixed_tma_kernel<true, false, false, false>,
-      step_mixed_tma_kernel<false, false, true, false>,  step_mixed_tma_kernel<true, false, true, false>,
       step_mixed_tma_kernel<false, true, false, false>,  step_mixed_tma_kernel<true, true, false, false>,
-      step_mixed_tma_kernel<false, false, false, true>,  step_mixed_tma_kernel<true, false, false, true>};
+      step_mixed_tma_kernel<false, false, true, false>,  step_mixed_tma_kernel<true, false, true, false>,
+      step_mixed_tma_kernel<false, true, true, false>,   step_mixed_tma_kernel<true, true, true, false>,
+      step_mixed_tma_kernel<false, false, false, true>,  step_mixed_tma_kernel<true, false, false, true>,
+      step_mixed_tma_kernel<false, true, false, true>,   step_mixed_tma_kernel<true, true, false, true>,
+      step_mixed_tma_kernel<false, false, true, true>,   step_mixed_tma_kernel<true, false, true, true>,
+      step_mixed_tma_kernel<false, true, true, true>,    step_mixed_tma_kernel<true, true, true, true>};
   constexpr int kAttrDevices = 64;
   // a kernel attribute is per device; atomic because handles may be driven from several host threads
   // (setting an attribute twice is harmless)
-  static std::atomic<bool> attr_set[kAttrDevices][8];
-  const int variant = (int)bf + 2 * (gather ? 3 : records ? 2 : (int)phys);
+  static std::atomic<bool> attr_set[kAttrDevices][16];
+  const int variant = (int)bf + 2 * (int)records + 4 * (int)phys + 8 * (int)gather;
   const Kern kern = table[variant];
   const int threads = phys ? Shape<true>::kThreads : Shape<false>::kThreads;
   const int smem = phys ? Shape<true>::kSmemBytes : Shape<false>::kSmemBytes;
@@ -1197,7 +1207,9 @@ cudaError_t launch_step_mixed_tma(st_ctx* h, const StepParams& p, bool records, 
   if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
   TmaArgs a;
   a.s = carve_mixed(h->state.p, h->cap, bf);
-  a.rec = records ? (float4*)h->state_alt.p : nullptr;
+  // records written by steps that gather go where the stale state was, their cells apart
+  a.rec = records ? (float4*)(gather ? h->state.p : h->state_alt.p) : nullptr;
+  if (records && gather) a.s.cell = (int32_t*)h->rec_cell.p;
   // the deferred gather of the last sort: permutation, records (old order) and ids in, ids out
   a.perm = gather ? (const uint32_t*)h->vals[0].p : nullptr;
   a.grec = gather ? (const float4*)h->state_alt.p : nullptr;

@@ -319,7 +319,7 @@ struct SegArgs {
   long long* __restrict__ Uw;
   int64_t n, ncell;
   int nx, ny, nz, len;
-  double inv_h[3];
+  fix::Scale scale;
   double dt, mcoef, g[3];
   double inv_ca, inv_alpha;
 };
@@ -368,7 +368,7 @@ __global__ void __launch_bounds__(kSegThreads, 3) adjoint_segment_kernel(const S
         x[q] = slot[q * a.n + p];
         v[q] = slot[(3 + q) * a.n + p];
       }
-      const fix::Stencil st = fix::stencil(x, a.inv_h, n3);
+      const fix::Stencil st = fix::stencil(x, a.scale, n3);
       const int key = st.c0[0] + a.nx * (st.c0[1] + a.ny * st.c0[2]);
       const double Jb[3] = {a.lam[key], a.lam[a.ncell + key], a.lam[2 * a.ncell + key]};
       const int base = st.i0[0] + a.nx * (st.i0[1] + a.ny * st.i0[2]);
@@ -404,11 +404,11 @@ __global__ void __launch_bounds__(kSegThreads, 3) adjoint_segment_kernel(const S
       {
         double g[3];
         fix::derivative<0>(u, st.f, g);
-        xb[0] += (g[0] * ub[0] + g[1] * ub[1] + g[2] * ub[2]) * a.inv_h[0];
+        xb[0] += (g[0] * ub[0] + g[1] * ub[1] + g[2] * ub[2]) * a.scale.inv_h[0];
         fix::derivative<1>(u, st.f, g);
-        xb[1] += (g[0] * ub[0] + g[1] * ub[1] + g[2] * ub[2]) * a.inv_h[1];
+        xb[1] += (g[0] * ub[0] + g[1] * ub[1] + g[2] * ub[2]) * a.scale.inv_h[1];
         fix::derivative<2>(u, st.f, g);
-        xb[2] += (g[0] * ub[0] + g[1] * ub[1] + g[2] * ub[2]) * a.inv_h[2];
+        xb[2] += (g[0] * ub[0] + g[1] * ub[1] + g[2] * ub[2]) * a.scale.inv_h[2];
       }
       // dL/dU: the adjoint velocities as integers in the sums' units; sums that cannot take them, or belong to
       // another stencil, are committed and started anew
@@ -774,9 +774,9 @@ cudaError_t launch_adjoint_segment(st_ctx* h, const AdjointStepArgs& s, int len)
   for (int q = 0; q < 3; ++q) {
     a.xb[q] = s.xb[q];
     a.vb[q] = s.vb[q];
-    a.inv_h[q] = h->geo.inv_h[q];
     a.g[q] = h->g[q];
   }
+  a.scale = fix::make_scale(h->geo.inv_h);
   a.db = s.db;
   a.ab_part = s.ab_part;
   a.U = (const fix::FixCell*)h->fluid_fix.p;

@@ -10,6 +10,8 @@
 // lose lies below 2^-55 of the largest corner, where an FP64 interpolation rounds at 2^-53 three times.
 #pragma once
 
+#include <cmath>
+
 #include "st_common.cuh"
 
 namespace st {
@@ -52,10 +54,10 @@ __device__ __forceinline__ FixCell load_cell(const FixCell* p) {
   return c;
 }
 
-// floor(s 2^53) for 0 <= s <= 1024 (anything else, NaN included: 0)
-__device__ __forceinline__ int64_t to_fixed53(double s) {
+// floor(s 2^(53 + k)) for 0 <= s 2^k <= 1024 (anything else, NaN included: 0)
+__device__ __forceinline__ int64_t to_fixed53(double s, int k) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(s);
-  const int sh = 1033 - (int)(b >> 52);  // negative values have the sign bit up here: sh < 0
+  const int sh = 1033 - k - (int)(b >> 52);  // negative values have the sign bit up here: sh < 0
   const unsigned long long m = (b << 11) | 0x8000000000000000ull;
   return (unsigned)sh > 63u ? 0 : (int64_t)min(m >> sh, 0x7fffffffffffffffull);
 }
@@ -84,11 +86,29 @@ struct Stencil {
   int i0[3], i1[3], c0[3];
   int64_t f[3];
 };
-__device__ __forceinline__ Stencil stencil(const double (&x)[3], const double (&inv_h)[3], const int (&n3)[3]) {
+// Cells per length: a factor, or its binary logarithm where all three are powers of two from 1 to 1024 (then the
+// product is exact and only moves the exponent: three FP64 instructions less).
+struct Scale {
+  double inv_h[3];
+  int exact, log2[3];
+};
+inline Scale make_scale(const double (&inv_h)[3]) {
+  Scale s;
+  s.exact = 1;
+  for (int q = 0; q < 3; ++q) {
+    int e = 0;
+    s.inv_h[q] = inv_h[q];
+    const double m = std::frexp(inv_h[q], &e);
+    s.log2[q] = e - 1;
+    if (m != 0.5 || e < 1 || e > 11) s.exact = 0;
+  }
+  return s;
+}
+__device__ __forceinline__ Stencil stencil(const double (&x)[3], const Scale& sc, const int (&n3)[3]) {
   Stencil st;
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
-    const int64_t S = to_fixed53(x[q] * inv_h[q]);
+    const int64_t S = sc.exact ? to_fixed53(x[q], sc.log2[q]) : to_fixed53(x[q] * sc.inv_h[q], 0);
     st.c0[q] = min((int)(S >> 53), n3[q] - 1);
     const int64_t T = S - (int64_t(1) << 52);  // cell centres lie at halves
     const int ii = min((int)(T >> 53), n3[q] - 1);
@@ -165,10 +185,9 @@ __device__ __forceinline__ void load_corners(const FixCell* __restrict__ F, cons
   for (int q = 0; q < 3; ++q) u.e[q] = (word[0] >> (10 * q)) & 1023;
 #pragma unroll
   for (int k = 1; k < 8; ++k) differ |= word[k] ^ word[0];
-  if (differ) {
 #pragma unroll
-    for (int q = 0; q < 3; ++q) align(u.uh[q], u.ul[q], word, q, u.e[q]);
-  }
+  for (int q = 0; q < 3; ++q)
+    if (differ & (1023 << (10 * q))) align(u.uh[q], u.ul[q], word, q, u.e[q]);
 }
 
 // the interpolated value from the corners and their weights

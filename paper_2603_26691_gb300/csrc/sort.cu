@@ -178,26 +178,26 @@ __global__ void __launch_bounds__(kSortThreads) digit_totals_kernel(Src src, int
   }
 }
 
-// exclusive scan of each pass's 256 digit totals (one block of 256 threads)
+// exclusive scan of each pass's 256 digit totals (one block of 256 threads per pass: by one thread each they took
+// 4 us a pass, a third of a small sort)
 __global__ void digit_offsets_kernel(const uint32_t* __restrict__ totals, int passes, uint32_t* __restrict__ offs,
                                      const int* __restrict__ gate) {
   if (gated_off(gate)) return;
-  __shared__ uint32_t s[kRadix];
-  for (int p = 0; p < passes; ++p) {
-    s[threadIdx.x] = totals[p * kRadix + threadIdx.x];
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      uint32_t acc = 0;
-      for (int d = 0; d < kRadix; ++d) {
-        const uint32_t c = s[d];
-        s[d] = acc;
-        acc += c;
-      }
-    }
-    __syncthreads();
-    offs[p * kRadix + threadIdx.x] = s[threadIdx.x];
-    __syncthreads();
+  __shared__ uint32_t wsum[kRadix / 32];
+  const int p = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (p >= passes) return;
+  const uint32_t c = totals[p * kRadix + threadIdx.x];
+  uint32_t inc = c;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += y;
   }
+  if (lane == 31) wsum[w] = inc;
+  __syncthreads();
+  uint32_t before = 0;
+  for (int k = 0; k < w; ++k) before += wsum[k];
+  offs[p * kRadix + threadIdx.x] = before + inc - c;
 }
 
 // shared memory of a pass: two staging buffers (each a key-or-cell array and a value array of a
@@ -793,7 +793,7 @@ cudaError_t radix_passes(Src src, int64_t n, int key_bits, uint32_t* ka, uint32_
   if (e != cudaSuccess) return e;
   digit_totals_kernel<Src><<<grid_for((n + kItems - 1) / kItems), kSortThreads, 0, s>>>(src, n, key_bits, totals,
                                                                                        gate);
-  digit_offsets_kernel<<<1, kRadix, 0, s>>>(totals, passes, offs, gate);
+  digit_offsets_kernel<<<passes, kRadix, 0, s>>>(totals, passes, offs, gate);
   *launches += 2;
   int64_t grid = (int64_t)sms * kPassBlocksPerSM;
   if (grid > ntiles) grid = ntiles;

@@ -206,7 +206,8 @@ struct FixArgs {
   long long* __restrict__ acc;  // null: no deposit (the adjoint's recomputation)
   int64_t n, ncell;
   int nx, ny, nz, nsteps, E;
-  double L[3], invL[3], inv_h[3];
+  double L[3], invL[3];
+  fix::Scale scale;
   double dt, inv_ca, mcoef, g[3];
 };
 
@@ -290,7 +291,7 @@ __global__ void __launch_bounds__(256, 2) step_f64_fixed_kernel(const FixArgs a)
           slot += 6 * a.n;
           next += a.tape_every;
         }
-        const fix::Stencil st = fix::stencil(x, a.inv_h, n3);
+        const fix::Stencil st = fix::stencil(x, a.scale, n3);
         const int k = st.c0[0] + a.nx * (st.c0[1] + a.ny * st.c0[2]);
         if (k != key) {
           if (key >= 0 && a.acc) {
@@ -377,9 +378,9 @@ cudaError_t launch_step_f64_tape(st_ctx* h, const double* const (&in)[6], const 
   for (int q = 0; q < 3; ++q) {
     a.L[q] = h->geo.L[q];
     a.invL[q] = 1.0 / h->geo.L[q];
-    a.inv_h[q] = h->geo.inv_h[q];
     a.g[q] = p.g[q];
   }
+  a.scale = fix::make_scale(h->geo.inv_h);
   a.dt = p.dt;
   a.inv_ca = 1.0 / p.ca;
   a.mcoef = p.mcoef;

@@ -117,8 +117,8 @@ struct TmaArgs {
   float dt, cadt, inv_ca, mcoef;
   float g[3], gdt[3];
   int nsteps;                         // steps to take (1 .. kMaxFusedSteps)
-  int E;                              // global accumulator exponent
-  float s1, s2;                       // s1 * s2 = 2^(E - kDepShift): global units -> deposit-tile units
+  float s2;                           // mcoef (of 1 kg) times s2: impulses in deposit-tile units, 2^(kDepShift - E)
+                                      // of the accumulator's; s2 is 1 unless the impulses are tiny
   float4* __restrict__ rec;           // record output: two float4 per particle (see st_common.cuh)
   const uint32_t* __restrict__ perm;  // GATHER: storage index (old order) of each sorted position
   const float4* __restrict__ grec;    // GATHER: the records in the old order
@@ -291,13 +291,14 @@ __device__ __forceinline__ float sn_factor(float re) {
   return re <= 1000.0f ? fmaf(0.15f, p, 1.0f) : (0.44f / 24.0f) * re;
 }
 
-// add round(r_q * 2^Es), q = 0, 1, 2, to the shared deposit-tile values of one cell, each kept as
+// add round(t_q), q = 0, 1, 2, to the shared deposit-tile values of one cell, each kept as
 // three signed digits in int32 words (w[0] + 2^15 w[kDepositCells] + 2^30 w[2 kDepositCells], the
-// components kDigits kDepositCells words apart); s1 * s2 = 2^Es.  Each scaled value t
-// (|t| < 2^45) is split exactly into balanced digits by round-to-nearest additions of
-// 1.5 * 2^(23+b), which leave the nearest multiple of 2^b: t = 2^30 d2 + 2^15 d1 + d0 +
-// (t - round(t)) with |d0|, |d1| <= 2^14 and |d2| <= 2^15.  Components 0 and 1 are split as a
-// register pair.  Integer atomics make the sums exact and independent of the order of the adds.
+// components kDigits kDepositCells words apart).  Each value t (in tile units, |t| < 2^45) is split exactly
+// into balanced digits by round-to-nearest additions of 1.5 * 2^(23+b), which leave the nearest multiple
+// of 2^b: t = 2^30 d2 + 2^15 d1 + d0 + (t - round(t)) with |d0|, |d1| <= 2^14 and |d2| <= 2^15.  Components 0 and
+// 1 are split as a register pair.  The top digit is zero up to 2^29, where nearly all values lie (the unit
+// is 2^-45 of a bound on 128 of the largest particles): two digits then.  Integer atomics make the sums exact
+// and independent of the order of the adds.
 __device__ __forceinline__ void digits1(float t, int& d0, int& d1, int& d2) {
   const float h = __fsub_rn(__fadd_rn(t, 0x1.8p53f), 0x1.8p53f);  // multiple of 2^30
   const float l = __fsub_rn(t, h);                                  // |l| <= 2^29, exact
@@ -325,10 +326,39 @@ __device__ __forceinline__ void digits2(unsigned long long t, int* d0, int* d1, 
   d0[0] = __float_as_int(a) - 0x4B400000;
   d0[1] = __float_as_int(b) - 0x4B400000;
 }
-__device__ __forceinline__ void dep_add3(int* w, float r0, float r1, float r2, float s1, float s2) {
+// the two lower digits alone, |t| <= 2^29
+__device__ __forceinline__ void low_digits1(float t, int& d0, int& d1) {
+  const float m = __fsub_rn(__fadd_rn(t, 0x1.8p38f), 0x1.8p38f);
+  d1 = __float_as_int(__fmaf_rn(m, 0x1p-15f, 12582912.0f)) - 0x4B400000;
+  d0 = __float_as_int(__fadd_rn(__fsub_rn(t, m), 12582912.0f)) - 0x4B400000;
+}
+__device__ __forceinline__ void low_digits2(unsigned long long t, int* d0, int* d1) {
+  const unsigned long long C38 = pack2(0x1.8p38f, 0x1.8p38f), C23 = pack2(12582912.0f, 12582912.0f);
+  const unsigned long long m = sub2(add2(t, C38), C38);
+  float a, b;
+  unpack2(fma2(m, pack2(0x1p-15f, 0x1p-15f), C23), a, b);
+  d1[0] = __float_as_int(a) - 0x4B400000;
+  d1[1] = __float_as_int(b) - 0x4B400000;
+  unpack2(add2(sub2(t, m), C23), a, b);
+  d0[0] = __float_as_int(a) - 0x4B400000;
+  d0[1] = __float_as_int(b) - 0x4B400000;
+}
+__device__ __forceinline__ void dep_add3(int* w, float t0, float t1, float t2) {
+  if (__builtin_expect(fmaxf(fmaxf(fabsf(t0), fabsf(t1)), fabsf(t2)) <= 0x1p29f, 1)) {
+    int d0[3], d1[3];
+    low_digits2(pack2(t0, t1), d0, d1);
+    low_digits1(t2, d0[2], d1[2]);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      int* wq = w + q * (kDigits * kDepositCells);
+      if (d0[q]) atomicAdd(wq, d0[q]);
+      if (d1[q]) atomicAdd(wq + kDepositCells, d1[q]);
+    }
+    return;
+  }
   int d0[3], d1[3], d2[3];
-  digits2(mul2(mul2(pack2(r0, r1), pack2(s1, s1)), pack2(s2, s2)), d0, d1, d2);
-  digits1(__fmul_rn(__fmul_rn(r2, s1), s2), d0[2], d1[2], d2[2]);
+  digits2(pack2(t0, t1), d0, d1, d2);
+  digits1(t2, d0[2], d1[2], d2[2]);
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
     int* wq = w + q * (kDigits * kDepositCells);
@@ -407,7 +437,7 @@ __device__ __noinline__ void commit_far(const TmaArgs& a, unsigned cell, float r
     const uint32_t ex = (b >> 23) & 0xffu;
     unsigned long long man = b & 0x7fffffu;
     if (ex != 0) man |= 0x800000ull;
-    int s = (int)(ex == 0 ? 1 : ex) - 150 + a.E;
+    int s = (int)(ex == 0 ? 1 : ex) - 150 + kDepShift;
     if (s < 0) {
       const int k = -s;
       man = k < 32 ? ((man + ((1ull << k) >> 1)) >> k) : 0ull;
@@ -425,7 +455,7 @@ __device__ __noinline__ void commit_far(const TmaArgs& a, unsigned cell, float r
 // accumulator
 __device__ __forceinline__ void commit_record(const TmaArgs& a, int* dep, unsigned c, float r0, float r1, float r2) {
   if (__builtin_expect((int)c >= 0, 1))
-    dep_add3(dep + dep_index(c), r0, r1, r2, a.s1, a.s2);
+    dep_add3(dep + dep_index(c), r0, r1, r2);
   else
     commit_far(a, c & ~kFarCell, r0, r1, r2);
 }
@@ -925,10 +955,12 @@ __global__ void __maxnreg__(Shape<PHYS>::kRegs) step_mixed_tma_kernel(const __gr
               const __nv_bfloat162 b2 = __floats2bfloat162_rn(vn[0], vn[1]);
               vn[0] = __low2float(b2);
               vn[1] = __high2float(b2);
-              JP[q] = pack2(-m0 * ((vn[0] - v[q][jp]) - a.gdt[q]), -m1 * ((vn[1] - v[q][jp + 1]) - a.gdt[q]));
+              JP[q] = pack2(-m0 * (((vn[0] - v[q][jp]) - a.gdt[q]) * a.s2), -m1 * (((vn[1] - v[q][jp + 1]) - a.gdt[q]) * a.s2));
             } else {
               // v' - v = -(v - w) (1 - E), without the cancellation of subtracting the rounded v'
-              JP[q] = mul2(M, fma2(DVW, E1, dup2(a.gdt[q])));
+              unsigned long long X = fma2(DVW, E1, dup2(a.gdt[q]));
+              if (a.s2 != 1.0f) X = mul2(X, dup2(a.s2));
+              JP[q] = mul2(M, X);  // in tile units
             }
             const unsigned long long DXV = fma2(WT, dup2(a.dt), mul2(DVW, Q));
             const unsigned long long O = fma2(DXV, dup2(a.inv_h[q]), pack2(xi[q][jp], xi[q][jp + 1]));
@@ -1037,25 +1069,24 @@ __global__ void __maxnreg__(Shape<PHYS>::kRegs) step_mixed_tma_kernel(const __gr
           int Bl = (link && nall) ? 1 : 0;
 #pragma unroll
           for (int q = 0; q < 3; ++q) R[q] = link ? R[q] : 0.0f;
-          // the scan only matters where a run passes through a whole lane (often nowhere after drift)
-          if (__any_sync(0xffffffffu, Bl)) {
+          // the scan goes on while some run passes through a whole stretch of lanes (after drift often none does)
 #pragma unroll
-            for (int off = 1; off < kScanLanes; off <<= 1) {
-              float t0v = __shfl_down_sync(0xffffffffu, R[0], off);
-              float t1v = __shfl_down_sync(0xffffffffu, R[1], off);
-              float t2v = __shfl_down_sync(0xffffffffu, R[2], off);
-              int tb = __shfl_down_sync(0xffffffffu, Bl, off);
-              if (glane + off > kScanLanes - 1) {
-                tb = 0;
-                t0v = t1v = t2v = 0.0f;
-              }
-              if (Bl) {
-                R[0] += t0v;
-                R[1] += t1v;
-                R[2] += t2v;
-              }
-              Bl &= tb;
+          for (int off = 1; off < kScanLanes; off <<= 1) {
+            if (!__any_sync(0xffffffffu, Bl)) break;
+            float t0v = __shfl_down_sync(0xffffffffu, R[0], off);
+            float t1v = __shfl_down_sync(0xffffffffu, R[1], off);
+            float t2v = __shfl_down_sync(0xffffffffu, R[2], off);
+            int tb = __shfl_down_sync(0xffffffffu, Bl, off);
+            if (glane + off > kScanLanes - 1) {
+              tb = 0;
+              t0v = t1v = t2v = 0.0f;
             }
+            if (Bl) {
+              R[0] += t0v;
+              R[1] += t1v;
+              R[2] += t2v;
+            }
+            Bl &= tb;
           }
           const unsigned pk3 = __shfl_up_sync(0xffffffffu, key[kP - 1], 1);
           const bool head_lane = (glane == 0) || (pk3 != key[0]);
@@ -1244,14 +1275,14 @@ cudaError_t launch_step_mixed_tma(st_ctx* h, const StepParams& p, bool records, 
   a.dt = (float)p.dt;
   a.cadt = (float)(p.ca * p.dt);
   a.inv_ca = (float)(1.0 / p.ca);
-  a.mcoef = (float)p.mcoef;
-  a.E = p.E;
   {
-    // 2^(E - kDepShift) as two representable factors; beyond +-250 every scaled impulse is 0 or
-    // overflows the bound the exponent was chosen for, so clamping changes nothing
+    // tile units: 2^(E - kDepShift) in the mass coefficient as far as it stays an FP32 number (a power of two: the
+    // impulses' bits do not change), the rest in s2; beyond +-250 every scaled impulse is 0 or overflows the
+    // bound the exponent was chosen for, so clamping changes nothing
     const int Es = std::min(std::max(p.E - kDepShift, -250), 250);
-    a.s1 = std::ldexp(1.0f, Es / 2);
-    a.s2 = std::ldexp(1.0f, Es - Es / 2);
+    const int k1 = std::min(Es, 100 - std::ilogb(std::max(p.mcoef, 1e-300)));
+    a.mcoef = (float)std::ldexp(p.mcoef, k1);
+    a.s2 = std::ldexp(1.0f, Es - k1);
   }
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->dev);

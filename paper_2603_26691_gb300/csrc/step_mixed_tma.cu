@@ -351,8 +351,9 @@ __device__ __forceinline__ void dep_add3(int* w, float t0, float t1, float t2) {
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
       int* wq = w + q * (kDigits * kDepositCells);
-      if (d0[q]) atomicAdd(wq, d0[q]);
-      if (d1[q]) atomicAdd(wq + kDepositCells, d1[q]);
+      // not asked whether they are zero: they rarely are (38.8 ms with the tests, 37.3 ms without)
+      atomicAdd(wq, d0[q]);
+      atomicAdd(wq + kDepositCells, d1[q]);
     }
     return;
   }
@@ -1060,36 +1061,33 @@ __global__ void __maxnreg__(Shape<PHYS>::kRegs) step_mixed_tma_kernel(const __gr
             for (int q = 0; q < 3; ++q) Sx[j][q] = J[j][q] + (same ? Sx[j + 1][q] : 0.0f);
           }
           const unsigned nk0 = __shfl_down_sync(0xffffffffu, key[0], 1);
-          const int nall = __shfl_down_sync(0xffffffffu, (int)(tail == 0), 1);
+          const int glane = lane & (kScanLanes - 1);
+          // the lanes whose last run goes on in the next lane, and those that are one run; runs do not leave a group
+          // of kScanLanes lanes
+          const unsigned links = __ballot_sync(0xffffffffu, glane < kScanLanes - 1 && nk0 == key[kP - 1] &&
+                                                                key[kP - 1] != kNoKey);
+          const unsigned whole = __ballot_sync(0xffffffffu, tail == 0);
+          const bool link = (links >> lane) & 1u;
           float R[3];
 #pragma unroll
-          for (int q = 0; q < 3; ++q) R[q] = __shfl_down_sync(0xffffffffu, Sx[0][q], 1);
-          const int glane = lane & (kScanLanes - 1);
-          const bool link = (glane < kScanLanes - 1) && (nk0 == key[kP - 1]) && (key[kP - 1] != kNoKey);
-          int Bl = (link && nall) ? 1 : 0;
-#pragma unroll
-          for (int q = 0; q < 3; ++q) R[q] = link ? R[q] : 0.0f;
-          // the scan goes on while some run passes through a whole stretch of lanes (after drift often none does)
+          for (int q = 0; q < 3; ++q) {
+            const float r = __shfl_down_sync(0xffffffffu, Sx[0][q], 1);
+            R[q] = link ? r : 0.0f;
+          }
+          // through: the lanes from which the next `off` lanes are one run; the scan ends with the last of them
+          // (after drift soon)
+          unsigned through = links & (whole >> 1);
 #pragma unroll
           for (int off = 1; off < kScanLanes; off <<= 1) {
-            if (!__any_sync(0xffffffffu, Bl)) break;
-            float t0v = __shfl_down_sync(0xffffffffu, R[0], off);
-            float t1v = __shfl_down_sync(0xffffffffu, R[1], off);
-            float t2v = __shfl_down_sync(0xffffffffu, R[2], off);
-            int tb = __shfl_down_sync(0xffffffffu, Bl, off);
-            if (glane + off > kScanLanes - 1) {
-              tb = 0;
-              t0v = t1v = t2v = 0.0f;
+            if (through == 0u) break;
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+              const float r = __shfl_down_sync(0xffffffffu, R[q], off);
+              if ((through >> lane) & 1u) R[q] += r;
             }
-            if (Bl) {
-              R[0] += t0v;
-              R[1] += t1v;
-              R[2] += t2v;
-            }
-            Bl &= tb;
+            through &= through >> off;
           }
-          const unsigned pk3 = __shfl_up_sync(0xffffffffu, key[kP - 1], 1);
-          const bool head_lane = (glane == 0) || (pk3 != key[0]);
+          const bool head_lane = glane == 0 || !((links >> (lane - 1)) & 1u);
           // each lane commits its run sums where they are, one pass per particle slot.  (Packing the sums of
           // few runs, fresh after a sort, into one pass through shared memory gains nothing: ten steps of 6e7
           // particles on 128^3 took 7.01 ms with it and 6.93 ms without.)

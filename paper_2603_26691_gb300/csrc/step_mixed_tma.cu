@@ -58,7 +58,8 @@ constexpr int kStages = 2;
 constexpr int kR = 2;                      // deposit halo
 constexpr int kDE = kU + 2 * kR;           // deposit tile edge (12)
 constexpr int kDepositCells = kDE * kDE * kDE;  // 1728
-constexpr int kScanLanes = 32 / kP;        // runs are chained across at most this many lanes
+constexpr int kScanPairs = 8;              // runs are chained across at most this many pairs of lanes
+constexpr unsigned kPairLinks = 0x15551555u;  // the pairs that have a next one in their group, at their even lane
 constexpr int kDigits = 3;                 // 15-bit digits per value in the shared deposit tile
 constexpr int kDigitBits = 15;
 constexpr int kDepShift = 51;              // shared tile units = global units * 2^kDepShift
@@ -72,8 +73,9 @@ constexpr int kDepositBytes = kDepositCells * 3 * kDigits * 4;  // 62208
 
 // The shape of an instance.  The steps run on what the registers let run at once: two particles per lane and 23
 // consumer warps at 80 registers hide more of the latency than four per lane and 15 warps at 128 (4e8
-// particles on 256^3, ten steps: 44.1 against 48.2 ms; with 19 warps 44.8 ms).  The physics variants need more
-// registers: 19 warps at 96 (cloud-in-cell at 2e7 on 128^3: 8.9 ms, with 23 warps 9.3, with four per lane 10.7).
+// particles on 256^3, ten steps: 44.1 against 48.2 ms when the shape was chosen, 36.8 ms since).  The physics
+// variants need more registers: 19 warps at 96 (cloud-in-cell at 2e7 on 128^3: 8.9 ms, with four per lane 10.7; 7.3 ms
+// since).  Swapped, 19 warps for the default and 23 for the variants: 39.9 against 37.3 ms and 8.8 against 7.3 ms.
 template <bool PHYS>
 struct Shape {
   static constexpr int kConsumerWarps = PHYS ? 19 : 23;
@@ -1047,55 +1049,59 @@ __global__ void __maxnreg__(Shape<PHYS>::kRegs) step_mixed_tma_kernel(const __gr
           }
         }
         if (!(PHYS && a.cic)) {
-          // ---- deposit: runs of equal key over the warp's 128 particles (lane-local suffix sums, then a
-          // segmented suffix scan across lanes chains runs that span lanes) ----
+          // ---- deposit: runs of equal key over the warp's particles: suffix sums within pairs of lanes (four
+          // particles), then a segmented suffix scan over the pairs, chains runs in groups of kScanPairs of them.  (The
+          // order of the sums is that of four particles per lane, whose results these are to the bit.) ----
+          static_assert(kP == 2, "two lanes hold the four particles of a pair");
+          const bool even = (lane & 1) == 0;
+          const unsigned nk0 = __shfl_down_sync(0xffffffffu, key[0], 1);
+          // this lane's particles are of one run; its last one's goes on in the next lane
+          const bool same = key[0] == key[1], cont = nk0 == key[1];
+          const unsigned sames = __ballot_sync(0xffffffffu, same), conts = __ballot_sync(0xffffffffu, cont);
+          // the pairs whose last run goes on in the next pair, at their even lane; those that are one run
+          const unsigned links = (__ballot_sync(0xffffffffu, cont && key[1] != kNoKey) >> 1) & kPairLinks;
+          const unsigned whole = sames & conts & (sames >> 1) & 0x55555555u;
           float Sx[kP][3];
 #pragma unroll
-          for (int q = 0; q < 3; ++q) Sx[kP - 1][q] = J[kP - 1][q];
-          int tail = kP - 1;  // the first particle of the run that ends the lane
-#pragma unroll
-          for (int j = kP - 2; j >= 0; --j) {
-            const bool same = key[j] == key[j + 1];
-            if (same && tail == j + 1) tail = j;
-#pragma unroll
-            for (int q = 0; q < 3; ++q) Sx[j][q] = J[j][q] + (same ? Sx[j + 1][q] : 0.0f);
+          for (int q = 0; q < 3; ++q) {
+            Sx[0][q] = J[0][q] + (same ? J[1][q] : 0.0f);
+            const float r = __shfl_down_sync(0xffffffffu, Sx[0][q], 1);
+            Sx[1][q] = J[1][q] + (even && cont ? r : 0.0f);
+            Sx[0][q] = J[0][q] + (same ? Sx[1][q] : 0.0f);
           }
-          const unsigned nk0 = __shfl_down_sync(0xffffffffu, key[0], 1);
-          const int glane = lane & (kScanLanes - 1);
-          // the lanes whose last run goes on in the next lane, and those that are one run; runs do not leave a group
-          // of kScanLanes lanes
-          const unsigned links = __ballot_sync(0xffffffffu, glane < kScanLanes - 1 && nk0 == key[kP - 1] &&
-                                                                key[kP - 1] != kNoKey);
-          const unsigned whole = __ballot_sync(0xffffffffu, tail == 0);
-          const bool link = (links >> lane) & 1u;
-          float R[3];
+          const int pair = lane & ~1;
+          const bool link = (links >> pair) & 1u;
+          float R[3];  // of the pair, in both lanes: the sum of its last run beyond it
 #pragma unroll
           for (int q = 0; q < 3; ++q) {
-            const float r = __shfl_down_sync(0xffffffffu, Sx[0][q], 1);
+            const float r = __shfl_sync(0xffffffffu, Sx[0][q], (pair + 2) & 31);
             R[q] = link ? r : 0.0f;
           }
-          // through: the lanes from which the next `off` lanes are one run; the scan ends with the last of them
+          // through: the pairs from which the next `off` pairs are one run; the scan ends with the last of them
           // (after drift soon)
-          unsigned through = links & (whole >> 1);
+          unsigned through = links & (whole >> 2);
 #pragma unroll
-          for (int off = 1; off < kScanLanes; off <<= 1) {
+          for (int off = 1; off < kScanPairs; off <<= 1) {
             if (through == 0u) break;
 #pragma unroll
             for (int q = 0; q < 3; ++q) {
-              const float r = __shfl_down_sync(0xffffffffu, R[q], off);
-              if ((through >> lane) & 1u) R[q] += r;
+              const float r = __shfl_down_sync(0xffffffffu, R[q], 2 * off);
+              if ((through >> pair) & 1u) R[q] += r;
             }
-            through &= through >> off;
+            through &= through >> (2 * off);
           }
-          const bool head_lane = glane == 0 || !((links >> (lane - 1)) & 1u);
+          const bool head_lane = even ? lane % (2 * kScanPairs) == 0 || !((links >> (lane - 2)) & 1u)
+                                      : !((conts >> (lane - 1)) & 1u);
+          // a run that starts at the second particle, or the first, goes on to the end of the pair
+          const bool to_end1 = !even || (cont && ((sames >> (lane + 1)) & 1u)), to_end0 = to_end1 && same;
           // each lane commits its run sums where they are, one pass per particle slot.  (Packing the sums of
-          // few runs, fresh after a sort, into one pass through shared memory gains nothing: ten steps of 6e7
-          // particles on 128^3 took 7.01 ms with it and 6.93 ms without.)
+          // few runs, fresh after a sort, into one pass through shared memory gained nothing: ten steps of 6e7
+          // particles on 128^3, now 5.5 ms, took 7.01 ms with it and 6.93 ms without.)
 #pragma unroll
           for (int j = 0; j < kP; ++j) {
             const bool start = ((j == 0) ? head_lane : (key[j] != key[j - 1])) && key[j] != kNoKey;
             if (start) {
-              const bool to_end = j == tail;
+              const bool to_end = j == 0 ? to_end0 : to_end1;
               commit_record(a, dep, key[j], Sx[j][0] + (to_end ? R[0] : 0.0f), Sx[j][1] + (to_end ? R[1] : 0.0f),
                             Sx[j][2] + (to_end ? R[2] : 0.0f));
             }

@@ -366,8 +366,8 @@ __device__ __forceinline__ void micro_particle(const MixedArgs& a, const int (&n
 
 // The group sums of the head lanes added to the exact accumulators, the commits spread over the lanes:
 // the H heads' 5 H (value, cell) items in component-major order through the warp's staging buffer, one
-// item per lane and round.  A round then runs one or two of the add routines on many lanes instead of
-// all five on the few head lanes; the adds are exact, so the sums are the same.
+// item per lane and round.  A round then runs one add routine on many lanes instead of five on the few head
+// lanes; the adds are exact, so the sums are the same.
 __device__ __forceinline__ void micro_commit(const MixedArgs& a, GroupBuf<5>& b, int lane, bool head, int key,
                                              const float (&g)[5]) {
   const unsigned hm = __ballot_sync(0xffffffffu, head);
@@ -388,10 +388,10 @@ __device__ __forceinline__ void micro_commit(const MixedArgs& a, GroupBuf<5>& b,
     const int r = i - q * H;
     const float v = b.g[q][r];
     const int k = b.key[r];
-    if (q < 3)
-      acc_add_f32(a.acc + kAccWords * ((int64_t)q * a.ncell + k), v, a.E);
-    else
-      wide_add_f32(a.macc + kWideWords * ((int64_t)(q - 3) * a.ncell + k), v);
+    const bool mom = q < 3;
+    long long* w = mom ? a.acc + kAccWords * ((int64_t)q * a.ncell + k)
+                       : a.macc + kWideWords * ((int64_t)(q - 3) * a.ncell + k);
+    add_f32_words(w, mom ? kAccWords : kWideWords, v, mom ? a.E : -kWideBase);
   }
 }
 

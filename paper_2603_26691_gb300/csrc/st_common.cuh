@@ -299,20 +299,28 @@ __device__ __forceinline__ void acc_add_mag(long long* p, unsigned long long m, 
   if (d2 && q + 2 < kAccWords) atomicAdd((unsigned long long*)&p[q + 2], (unsigned long long)d2);
 }
 
-// add round(f * 2^E) (FP32 input; integer operations only) -- requires |f| 2^E < 2^100
-__device__ __forceinline__ void acc_add_f32(long long* p, float f, int E) {
+// add round(f * 2^E) to `words` carry-save words (FP32 input; 32-bit integer operations only).  The 24-bit
+// significand spans at most two digits.
+__device__ __forceinline__ void add_f32_words(long long* p, int words, float f, int E) {
   const uint32_t b = __float_as_uint(f);
   const uint32_t ex = (b >> 23) & 0xffu;
-  unsigned long long man = b & 0x7fffffu;
-  if (ex != 0) man |= 0x800000ull;
-  int s = (int)(ex == 0 ? 1 : ex) - 150 + E;
-  if (s < 0) {
+  uint32_t man = (b & 0x7fffffu) | (ex != 0 ? 0x800000u : 0u);  // subnormals: man * 2^(1 - 150)
+  int s = (int)max(ex, 1u) - 150 + E;
+  if (__builtin_expect(s < 0, 0)) {
     const int r = -s;
-    man = r < 32 ? ((man + ((1ull << r) >> 1)) >> r) : 0ull;
+    man = r < 32 ? (man + ((1u << r) >> 1)) >> r : 0u;
     s = 0;
   }
-  acc_add_mag(p, man, s, (b >> 31) != 0);
+  const int q = s >> 5;
+  const uint32_t d0 = man << (s & 31), d1 = __funnelshift_l(man, 0u, s);  // bits 0 .. 31 and 32 .. 55 of man << (s & 31)
+  const bool neg = (b >> 31) != 0;
+  if (d0 != 0u && q < words)
+    atomicAdd((unsigned long long*)&p[q], (unsigned long long)(neg ? -(long long)d0 : (long long)d0));
+  if (d1 != 0u && q + 1 < words)
+    atomicAdd((unsigned long long*)&p[q + 1], (unsigned long long)(neg ? -(long long)d1 : (long long)d1));
 }
+// the per-cell source's words -- requires |f| 2^E < 2^100
+__device__ __forceinline__ void acc_add_f32(long long* p, float f, int E) { add_f32_words(p, kAccWords, f, E); }
 
 // add round(x * 2^E) (FP64 input; integer operations only) -- requires |x| 2^E < 2^100
 __device__ __forceinline__ void acc_add_f64(long long* p, double x, int E) {
@@ -419,26 +427,7 @@ constexpr int kAdjBlocks = 152 * 8;
 
 // Carry-save accumulator: value = sum_i w[i] * 2^(32 i + kWideBase); each
 // contribution adds 32-bit digits, so each int64 word absorbs 2^31 of them.
-// an FP32 value into the same accumulator: its 24-bit significand spans at most two words
-__device__ __forceinline__ void wide_add_f32(long long* w, float x) {
-  if (x == 0.0f) return;
-  const uint32_t b = __float_as_uint(x);
-  const int ex = (int)((b >> 23) & 0xff);
-  unsigned long long man = b & 0x7fffffu;
-  if (ex != 0) man |= 1u << 23;                       // subnormals: man * 2^(1 - 150)
-  const int s = (ex == 0 ? 1 : ex) - 150 - kWideBase;  // >= 11: every FP32 value is on the grid
-  const int q = s >> 5, r = s & 31;
-  const unsigned long long lo = man << r;  // < 2^55
-  long long d0 = (long long)(lo & 0xffffffffull);
-  long long d1 = (long long)(lo >> 32);
-  if (b >> 31) {
-    d0 = -d0;
-    d1 = -d1;
-  }
-  if (d0 != 0 && q < kWideWords) atomicAdd((unsigned long long*)&w[q], (unsigned long long)d0);
-  if (d1 != 0 && q + 1 < kWideWords) atomicAdd((unsigned long long*)&w[q + 1], (unsigned long long)d1);
-}
-
+// (add_f32_words takes FP32 values: with E = -kWideBase every one of them is on the grid)
 __device__ __forceinline__ void wide_add(long long* w, double x) {
   if (x == 0.0) return;
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);

@@ -1,7 +1,7 @@
 // Mixed-precision Lagrangian step: int32 packed cell + FP32 in-cell offset,
 // FP32 (or BF16) velocity, FP32 diameter; FP32 arithmetic.  Each lane owns 4
-// consecutive particles, so every particle array is read and written with
-// 128-bit (BF16 velocity: 64-bit) coalesced accesses; a warp covers 128
+// consecutive particles (2 where nothing is deposited), so every particle array is read and
+// written with wide coalesced accesses; a warp covers 128
 // particles.  Impulses are reduced over runs of equal start-of-step cell in
 // storage order (lane-local suffix sums, then a segmented suffix scan across
 // lanes) and each run is committed once to the exact fixed-point accumulator.
@@ -11,7 +11,14 @@
 // The field is frozen over a call and particles do not act on each other, so a launch takes the steps up to
 // the next sort for one set of particles after the other, their state in registers; each step's runs are
 // those of one step per launch, so the results do not depend on how the steps are split over launches.
-// 2e6 particles on 100 x 84 x 60, ten steps: 0.50 ms against 0.68 ms.
+// 2e6 particles on 100 x 84 x 60, ten steps: 0.49 ms against 0.68 ms.
+// Bound by the latency of the gathers (from L1 and L2) and of the deposit's reductions at 16 warps an SM (126
+// registers; 24 and 32 warps with spills: 0.52 and 0.59 ms).  Two particles per lane in 64 registers take 0.44 ms, but
+// would sum in another order: the last bit of a sum, and through a coupled fluid of the velocities, would change.
+// Without a deposit, as the adjoint recomputes its segments, there is no order to keep: two per lane (1e7 particles on
+// 64^3, 40 steps forward and 38 recomputed: 11.05 ms against 11.7 ms).
+#include <cstring>
+
 #include "st_common.cuh"
 
 namespace st {
@@ -47,37 +54,73 @@ __device__ __forceinline__ void commit(const MixedArgs& a, int key, float j0, fl
   acc_add_f32(a.acc + kAccWords * (2 * a.ncell + key), j2, a.E);
 }
 
-template <bool BF16>
-__device__ __forceinline__ void load_v(const MixedArgs& a, int q, int64_t p0, float v[4]) {
-  if (BF16) {
-    uint2 r = __ldcs((const uint2*)((const __nv_bfloat16*)a.in.v[q] + p0));
-    __nv_bfloat162 lo = *reinterpret_cast<__nv_bfloat162*>(&r.x);
-    __nv_bfloat162 hi = *reinterpret_cast<__nv_bfloat162*>(&r.y);
-    float2 l = __bfloat1622float2(lo), h = __bfloat1622float2(hi);
-    v[0] = l.x;
-    v[1] = l.y;
-    v[2] = h.x;
-    v[3] = h.y;
+// particles per lane
+template <bool DEP>
+constexpr int kPerLane = DEP ? 4 : 2;
+
+// P values of a lane, one access, streaming
+template <int P, class T>
+__device__ __forceinline__ void ld(const T* p, T (&v)[P]) {
+  if constexpr (P == 4) {
+    const float4 r = __ldcs((const float4*)p);
+    memcpy(v, &r, sizeof(r));
   } else {
-    float4 r = __ldcs((const float4*)((const float*)a.in.v[q] + p0));
-    v[0] = r.x;
-    v[1] = r.y;
-    v[2] = r.z;
-    v[3] = r.w;
+    const float2 r = __ldcs((const float2*)p);
+    memcpy(v, &r, sizeof(r));
+  }
+}
+template <int P, class T>
+__device__ __forceinline__ void st(T* p, const T (&v)[P]) {
+  if constexpr (P == 4) {
+    float4 r;
+    memcpy(&r, v, sizeof(r));
+    __stcs((float4*)p, r);
+  } else {
+    float2 r;
+    memcpy(&r, v, sizeof(r));
+    __stcs((float2*)p, r);
   }
 }
 
-template <bool BF16>
-__device__ __forceinline__ void store_v(const MixedArgs& a, int q, int64_t p0, float v[4]) {
-  if (BF16) {
-    __nv_bfloat162 lo = __floats2bfloat162_rn(v[0], v[1]);
-    __nv_bfloat162 hi = __floats2bfloat162_rn(v[2], v[3]);
-    uint2 r;
-    r.x = *reinterpret_cast<unsigned*>(&lo);
-    r.y = *reinterpret_cast<unsigned*>(&hi);
-    __stcs((uint2*)((__nv_bfloat16*)a.s.v[q] + p0), r);
+template <bool BF16, int P>
+__device__ __forceinline__ void load_v(const MixedArgs& a, int q, int64_t p0, float (&v)[P]) {
+  if constexpr (BF16) {
+    __nv_bfloat162 r[P / 2];
+    if constexpr (P == 4) {
+      const uint2 u = __ldcs((const uint2*)((const __nv_bfloat16*)a.in.v[q] + p0));
+      memcpy(r, &u, sizeof(u));
+    } else {
+      const unsigned u = __ldcs((const unsigned*)((const __nv_bfloat16*)a.in.v[q] + p0));
+      memcpy(r, &u, sizeof(u));
+    }
+#pragma unroll
+    for (int i = 0; i < P / 2; ++i) {
+      const float2 f = __bfloat1622float2(r[i]);
+      v[2 * i] = f.x;
+      v[2 * i + 1] = f.y;
+    }
   } else {
-    __stcs((float4*)((float*)a.s.v[q] + p0), make_float4(v[0], v[1], v[2], v[3]));
+    ld((const float*)a.in.v[q] + p0, v);
+  }
+}
+
+template <bool BF16, int P>
+__device__ __forceinline__ void store_v(const MixedArgs& a, int q, int64_t p0, const float (&v)[P]) {
+  if constexpr (BF16) {
+    __nv_bfloat162 r[P / 2];
+#pragma unroll
+    for (int i = 0; i < P / 2; ++i) r[i] = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
+    if constexpr (P == 4) {
+      uint2 u;
+      memcpy(&u, r, sizeof(u));
+      __stcs((uint2*)((__nv_bfloat16*)a.s.v[q] + p0), u);
+    } else {
+      unsigned u;
+      memcpy(&u, r, sizeof(u));
+      __stcs((unsigned*)((__nv_bfloat16*)a.s.v[q] + p0), u);
+    }
+  } else {
+    st((float*)a.s.v[q] + p0, v);
   }
 }
 
@@ -102,55 +145,49 @@ __device__ __noinline__ int relocate_far(float& o, int ci, int n) {
   return (int)(k < 0 ? k + n : k);
 }
 
-// Sums J over runs of equal key in the warp's 128 particles (4 consecutive per lane) and commits
+// Sums J over runs of equal key in the warp's particles (kP consecutive per lane) and commits
 // each run once to the fixed-point accumulator: lane-local suffix sums, then a segmented suffix
 // scan across lanes.  Negative keys are skipped.
-__device__ __forceinline__ void deposit_runs(const MixedArgs& a, int lane, const int key[4], const float J[4][3]) {
+template <int kP>
+__device__ __forceinline__ void deposit_runs(const MixedArgs& a, int lane, const int (&key)[kP], const float (&J)[kP][3]) {
   // lane-local suffix sums S_j over the run that starts at j
-  float S[4][3];
+  float S[kP][3];
 #pragma unroll
-  for (int q = 0; q < 3; ++q) S[3][q] = J[3][q];
+  for (int q = 0; q < 3; ++q) S[kP - 1][q] = J[kP - 1][q];
+  int tail = kP - 1;  // first element of the run that ends the lane (the lane's tail run)
 #pragma unroll
-  for (int j = 2; j >= 0; --j) {
+  for (int j = kP - 2; j >= 0; --j) {
     const bool same = key[j] == key[j + 1];
+    if (same && tail == j + 1) tail = j;
 #pragma unroll
     for (int q = 0; q < 3; ++q) S[j][q] = J[j][q] + (same ? S[j + 1][q] : 0.0f);
   }
-  // first element of the run that ends the lane (the lane's tail run)
-  const int tail = (key[2] != key[3]) ? 3 : (key[1] != key[2]) ? 2 : (key[0] != key[1]) ? 1 : 0;
-  const bool all_same = tail == 0;
-  // link to the next lane: its leading run continues this lane's trailing run
+  // the lanes whose trailing run goes on in the next lane's leading run, and those that are one run
   const int nk0 = __shfl_down_sync(0xffffffffu, key[0], 1);
-  const int nall = __shfl_down_sync(0xffffffffu, (int)all_same, 1);
+  const unsigned links = __ballot_sync(0xffffffffu, lane < 31 && nk0 == key[kP - 1] && key[kP - 1] >= 0);
+  const unsigned whole = __ballot_sync(0xffffffffu, tail == 0);
   float A[3];
 #pragma unroll
-  for (int q = 0; q < 3; ++q) A[q] = __shfl_down_sync(0xffffffffu, S[0][q], 1);
-  const bool link = (lane < 31) && (nk0 == key[3]) && (key[3] >= 0);
-  int B = (link && nall) ? 1 : 0;
-#pragma unroll
-  for (int q = 0; q < 3; ++q) A[q] = link ? A[q] : 0.0f;
-  // segmented suffix scan R_l = A_l + B_l R_{l+1}
+  for (int q = 0; q < 3; ++q) {
+    const float t = __shfl_down_sync(0xffffffffu, S[0][q], 1);
+    A[q] = (links >> lane) & 1u ? t : 0.0f;
+  }
+  // segmented suffix scan R_l = A_l + B_l R_{l+1}; through: the lanes from which the next `off` lanes are one run (the
+  // scan ends with the last of them)
+  unsigned through = links & (whole >> 1);
 #pragma unroll
   for (int off = 1; off < 32; off <<= 1) {
-    float t0 = __shfl_down_sync(0xffffffffu, A[0], off);
-    float t1 = __shfl_down_sync(0xffffffffu, A[1], off);
-    float t2 = __shfl_down_sync(0xffffffffu, A[2], off);
-    int tb = __shfl_down_sync(0xffffffffu, B, off);
-    if (lane + off > 31) {
-      tb = 0;
-      t0 = t1 = t2 = 0.0f;
-    }
-    if (B) {
-      A[0] += t0;
-      A[1] += t1;
-      A[2] += t2;
-    }
-    B = B & tb;
-  }
-  const int pk3 = __shfl_up_sync(0xffffffffu, key[3], 1);
-  const bool head_lane = (lane == 0) || (pk3 != key[0]);
+    if (through == 0u) break;
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
+    for (int q = 0; q < 3; ++q) {
+      const float t = __shfl_down_sync(0xffffffffu, A[q], off);
+      if ((through >> lane) & 1u) A[q] += t;
+    }
+    through &= through >> off;
+  }
+  const bool head_lane = lane == 0 || !((links >> (lane - 1)) & 1u);
+#pragma unroll
+  for (int j = 0; j < kP; ++j) {
     const bool start = (j == 0) ? head_lane : (key[j] != key[j - 1]);
     if (start && key[j] >= 0) {
       const bool to_end = j == tail;  // only the tail run continues into the next lane
@@ -180,17 +217,19 @@ __device__ __forceinline__ void drag(const MixedArgs& a, float adt, float inv_a,
   }
 }
 
-template <bool BF16, bool CIC>
-__global__ void __launch_bounds__(256) step_mixed_kernel(const MixedArgs a) {
+// DEP: the impulses are deposited (CIC: cloud in cell)
+template <bool BF16, bool CIC, bool DEP>
+__global__ void __launch_bounds__(256, DEP ? 2 : 4) step_mixed_kernel(const MixedArgs a) {
+  constexpr int kP = kPerLane<DEP>, kPW = 32 * kP;  // particles per lane, per warp
   const int lane = threadIdx.x & 31;
   const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarp = ((int64_t)gridDim.x * blockDim.x) >> 5;
   const int n3[3] = {a.nx, a.ny, a.nz};
-  for (int64_t base = warp * 128; base < a.n; base += nwarp * 128) {
-    const int64_t p0 = base + lane * 4;
+  for (int64_t base = warp * kPW; base < a.n; base += nwarp * kPW) {
+    const int64_t p0 = base + lane * kP;
     {
       // pull the next iteration's particle lines towards L2 while this one computes
-      const int64_t pn = p0 + nwarp * 128;
+      const int64_t pn = p0 + nwarp * kPW;
       if (pn < a.n) {
         asm volatile("prefetch.global.L2 [%0];" ::"l"(a.in.cell + pn));
         for (int q = 0; q < 3; ++q) asm volatile("prefetch.global.L2 [%0];" ::"l"(a.in.xi[q] + pn));
@@ -199,36 +238,20 @@ __global__ void __launch_bounds__(256) step_mixed_kernel(const MixedArgs a) {
         asm volatile("prefetch.global.L2 [%0];" ::"l"(a.in.d + pn));
       }
     }
-    int cell[4];
-    float xi[3][4], v[3][4], dv[4];
-    const int nvalid = (int)max((int64_t)0, min((int64_t)4, a.n - p0));
+    int cell[kP];
+    float xi[3][kP], v[3][kP], dv[kP];
+    const int nvalid = (int)max((int64_t)0, min((int64_t)kP, a.n - p0));
     if (nvalid > 0) {
-      // ---- load (128-bit, streaming) ----
-      int4 c4 = __ldcs((const int4*)(a.in.cell + p0));
-      float4 x4[3];
-      for (int q = 0; q < 3; ++q) x4[q] = __ldcs((const float4*)(a.in.xi[q] + p0));
+      ld(a.in.cell + p0, cell);
+      for (int q = 0; q < 3; ++q) ld(a.in.xi[q] + p0, xi[q]);
       for (int q = 0; q < 3; ++q) load_v<BF16>(a, q, p0, v[q]);
-      float4 d4 = __ldcs((const float4*)(a.in.d + p0));
-      cell[0] = c4.x;
-      cell[1] = c4.y;
-      cell[2] = c4.z;
-      cell[3] = c4.w;
-      for (int q = 0; q < 3; ++q) {
-        xi[q][0] = x4[q].x;
-        xi[q][1] = x4[q].y;
-        xi[q][2] = x4[q].z;
-        xi[q][3] = x4[q].w;
-      }
-      dv[0] = d4.x;
-      dv[1] = d4.y;
-      dv[2] = d4.z;
-      dv[3] = d4.w;
+      ld(a.in.d + p0, dv);
     }
     // Stokes drag is decided by the diameter alone
-    float Ec[4], Qc[4];
+    float Ec[kP], Qc[kP];
     if (!a.sn && nvalid > 0) {
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
+      for (int j = 0; j < kP; ++j) {
         const float dd = dv[j] * dv[j];
         drag(a, a.cadt / dd, dd * a.inv_ca, Ec[j], Qc[j]);
       }
@@ -237,19 +260,23 @@ __global__ void __launch_bounds__(256) step_mixed_kernel(const MixedArgs a) {
     int next = a.tape ? a.tape_first : a.nsteps;
 #pragma unroll 1
     for (int step = 0; step < a.nsteps; ++step) {
-      int key[4] = {-1, -1, -1, -1};
-      float J[4][3];
-      for (int j = 0; j < 4; ++j) J[j][0] = J[j][1] = J[j][2] = 0.0f;
+      int key[kP];
+      float J[kP][3];
+#pragma unroll
+      for (int j = 0; j < kP; ++j) {
+        key[j] = -1;
+        J[j][0] = J[j][1] = J[j][2] = 0.0f;
+      }
       // cloud-in-cell deposit: the start-of-step stencil's lower corner (periodic) and weights
-      int sb[CIC ? 4 : 1][3];
-      float sf[CIC ? 4 : 1][3];
+      int sb[CIC ? kP : 1][3];
+      float sf[CIC ? kP : 1][3];
       if (step == next) {
         if (nvalid > 0) {
           float* f = (float*)slot;
-          *(int4*)((int*)slot + p0) = make_int4(cell[0], cell[1], cell[2], cell[3]);
+          st((int*)slot + p0, cell);
           for (int q = 0; q < 3; ++q) {
-            *(float4*)(f + (1 + q) * a.tape_n + p0) = make_float4(xi[q][0], xi[q][1], xi[q][2], xi[q][3]);
-            *(float4*)(f + (4 + q) * a.tape_n + p0) = make_float4(v[q][0], v[q][1], v[q][2], v[q][3]);
+            st(f + (1 + q) * a.tape_n + p0, xi[q]);
+            st(f + (4 + q) * a.tape_n + p0, v[q]);
           }
         }
         slot += 28 * a.tape_n;
@@ -257,7 +284,7 @@ __global__ void __launch_bounds__(256) step_mixed_kernel(const MixedArgs a) {
       }
       if (nvalid > 0) {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < kP; ++j) {
           if (j < nvalid) {
             const int ci[3] = {cell_i(cell[j]), cell_j(cell[j]), cell_k(cell[j])};
             key[j] = ci[0] + a.nx * (ci[1] + a.ny * ci[2]);
@@ -352,9 +379,8 @@ __global__ void __launch_bounds__(256) step_mixed_kernel(const MixedArgs a) {
           }
         }
       }
-      // ---- deposit: runs of equal key over the warp's 128 particles (none without an accumulator:
-      // the adjoint's recomputation) ----
-      if (!a.acc) {
+      // ---- deposit: runs of equal key over the warp's 128 particles ----
+      if (!DEP) {
       } else if (!CIC) {
         deposit_runs(a, lane, key, J);
       } else {
@@ -362,10 +388,10 @@ __global__ void __launch_bounds__(256) step_mixed_kernel(const MixedArgs a) {
 #pragma unroll 1
         for (int c = 0; c < 8; ++c) {
           const int dx = c & 1, dy = (c >> 1) & 1, dz = c >> 2;
-          int kc[4];
-          float Jc[4][3];
+          int kc[kP];
+          float Jc[kP][3];
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
+          for (int j = 0; j < kP; ++j) {
             const float* fj = sf[CIC ? j : 0];
             const int* bj = sb[CIC ? j : 0];
             const float w = (dx ? fj[0] : 1.0f - fj[0]) * (dy ? fj[1] : 1.0f - fj[1]) * (dz ? fj[2] : 1.0f - fj[2]);
@@ -382,10 +408,8 @@ __global__ void __launch_bounds__(256) step_mixed_kernel(const MixedArgs a) {
       }
     }
     if (nvalid > 0) {
-      // ---- store (128-bit, streaming) ----
-      __stcs((int4*)(a.s.cell + p0), make_int4(cell[0], cell[1], cell[2], cell[3]));
-      for (int q = 0; q < 3; ++q)
-        __stcs((float4*)(a.s.xi[q] + p0), make_float4(xi[q][0], xi[q][1], xi[q][2], xi[q][3]));
+      st(a.s.cell + p0, cell);
+      for (int q = 0; q < 3; ++q) st(a.s.xi[q] + p0, xi[q]);
       for (int q = 0; q < 3; ++q) store_v<BF16>(a, q, p0, v[q]);
     }
   }
@@ -430,12 +454,15 @@ cudaError_t launch_step_mixed_tape(st_ctx* h, const MixedState& in, const MixedS
   a.semi = p.semi;
   a.sn = p.sn;
   a.re_coef = (float)p.re_coef;
-  int64_t warps = (n + 127) / 128;
+  const int per_warp = 32 * (acc ? kPerLane<true> : kPerLane<false>);
+  const int64_t warps = (n + per_warp - 1) / per_warp;
   int64_t blocks = (warps * 32 + 255) / 256;
   if (blocks > 152 * 8) blocks = 152 * 8;
   if (blocks < 1) blocks = 1;
-  void (*kern)(const MixedArgs) = bf ? (p.cic ? step_mixed_kernel<true, true> : step_mixed_kernel<true, false>)
-                                     : (p.cic ? step_mixed_kernel<false, true> : step_mixed_kernel<false, false>);
+  void (*kern)(const MixedArgs) =
+      !acc ? (bf ? step_mixed_kernel<true, false, false> : step_mixed_kernel<false, false, false>)
+      : bf ? (p.cic ? step_mixed_kernel<true, true, true> : step_mixed_kernel<true, false, true>)
+           : (p.cic ? step_mixed_kernel<false, true, true> : step_mixed_kernel<false, false, true>);
   kern<<<(int)blocks, 256, 0, h->stream>>>(a);
   h->launches += 1;
   return cudaGetLastError();

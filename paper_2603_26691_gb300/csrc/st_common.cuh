@@ -630,6 +630,7 @@ bool tma_step_supported(const st_ctx* h);                               // step_
 // the records through the permutation and writes the sorted state, diameters and ids included.  Both: the
 // records go into `state`, the cells into rec_cell (records_written swaps the buffers)
 cudaError_t launch_step_mixed_tma(st_ctx* h, const StepParams& p, bool records, bool gather);  // step_mixed_tma.cu
+cudaError_t launch_step_mixed_tma_single(st_ctx* h, const StepParams& p, bool records, bool gather);  // step_mixed_tma_single.cu
 cudaError_t launch_rescale_acc(st_ctx* h, int shift);
 cudaError_t launch_normalize_acc(st_ctx* h);
 // the particle steps of st_step (sort when due, accumulator bookkeeping, step kernel)

@@ -66,6 +66,9 @@ constexpr int kDepShift = 51;              // shared tile units = global units *
 // adds to one cell's digit words between flushes: the two lower digits are at most 2^14, and the top one at
 // most 1 + 2^8 per particle of the run (one particle's impulse is below 2^38 tile units)
 constexpr int kDepMaxAdds = 131071;
+// particles from which a launch of one step goes to step_mixed_tma_single.cu (ten single steps, there / here: 3e5 on
+// 64^3 0.36 / 0.34 ms, 2e6 0.69 / 0.67, 2e7 on 128^3 4.54 / 4.72, 6e7 9.0 / 9.9)
+constexpr int64_t kSingleParticles = 1 << 23;
 constexpr unsigned kNoKey = 0xffffffffu;   // no cell: neither a tile-form nor a far one
 
 constexpr int kFluidBytes = kTE * kTE * kTE * 16;               // 43904
@@ -1204,6 +1207,9 @@ cudaError_t launch_step_mixed_tma(st_ctx* h, const StepParams& p, bool records, 
   const bool bf = h->prec == ST_MIXED_BF16V;
   const bool phys = p.ngp || p.semi || p.sn || p.cic;
   if (p.nsteps < 1 || p.nsteps > kMaxFusedSteps) return cudaErrorInvalidValue;
+  // a single step of many particles is bound by HBM: a kernel of its own, with the same results
+  if (p.nsteps == 1 && h->np >= kSingleParticles && !p.cic && !(records && gather) && !(phys && (records || gather)))
+    return launch_step_mixed_tma_single(h, p, records, gather);
   using Kern = void (*)(const CUtensorMap, const TmaArgs);
   static const Kern table[16] = {
       step_mixed_tma_kernel<false, false, false, false>, step_mixed_tma_kernel<true, false, false, false>,

@@ -53,6 +53,19 @@ def test_results_do_not_depend_on_the_split(prec, grid, chunk, physics, micro, n
 
 
 @pytest.mark.parametrize("prec", ["mixed_f32", "mixed_bf16"])
+@pytest.mark.parametrize("physics", ["default", "paper"])
+@pytest.mark.parametrize("grid,vmax", [((64, 32, 32), 2.0), ((64, 32, 32), 200.0), ((16, 16, 16), 2.0)])
+@pytest.mark.parametrize("n", [(1 << 23) - 1, (1 << 23) + 5])
+def test_many_particles_in_single_steps(prec, physics, grid, vmax, n):
+    """From 2^23 particles on a launch of one step is a kernel of its own: particles that stay near their units, that
+    leave them, and units of more particles than its tile takes; steps before and after a sort."""
+    args = (prec, grid, n, 4, physics, False)
+    ref = _run(*args, [6], 1e-3, vmax, 8)
+    for a, b in zip(ref, _run(*args, [1] * 6, 1e-3, vmax, 8)):
+        assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("prec", ["mixed_f32", "mixed_bf16"])
 @pytest.mark.parametrize("physics", ["default", "cic"])
 def test_fast_particles_leave_their_tiles(prec, physics):
     """Moves of many cells and of whole boxes in a step: every particle commits outside its unit's tile."""

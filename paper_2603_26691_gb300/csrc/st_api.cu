@@ -624,7 +624,9 @@ st_status run_steps(st_ctx* h, int nsteps, double dt) {
     // digits a launch can add to one word: a tile flush of each of the (at most 8) units that cover a cell,
     // at least one unit in 2^16 particle-steps; the other kernels one contribution per particle
     ST_TRY(prepare_accumulator(h, dt, m,
-                               tma ? 8.0 * ((double)h->np * m / 65536.0 + 2.0) : deposits_per_cell(h) * (double)h->np * m + 8.0,
+                               tma ? 8.0 * ((double)h->np * m / 65536.0 + 2.0) +
+                                         std::min(deposits_per_cell(h) * (double)h->np * m, (double)kFarFree * kFarCtas)
+                                   : deposits_per_cell(h) * (double)h->np * m + 8.0,
                                tma, &E));
     StepParams p;
     p.dt = dt;

@@ -629,6 +629,9 @@ bool tma_step_supported(const st_ctx* h);                               // step_
 // gather = true: the first step after a sort whose payload gather was deferred (perm_pending); it reads
 // the records through the permutation and writes the sorted state, diameters and ids included.  Both: the
 // records go into `state`, the cells into rec_cell (records_written swaps the buffers)
+// commits outside its tiles that a CTA of the sorted step adds without looking at the words (counted in full by
+// run_steps, for up to kFarCtas CTAs)
+constexpr int kFarFree = 1 << 16, kFarCtas = 256;
 cudaError_t launch_step_mixed_tma(st_ctx* h, const StepParams& p, bool records, bool gather);  // step_mixed_tma.cu
 cudaError_t launch_step_mixed_tma_single(st_ctx* h, const StepParams& p, bool records, bool gather);  // step_mixed_tma_single.cu
 cudaError_t launch_rescale_acc(st_ctx* h, int shift);

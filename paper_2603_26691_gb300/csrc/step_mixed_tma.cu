@@ -87,7 +87,7 @@ struct Shape {
   static constexpr int kRegs = 65536 / kThreads / 8 * 8;
   static constexpr int kStageBytes = kT * 32;             // the FP32 layout; BF16 uses less
   static constexpr int kSmemBytes = kFluidBytes + kDepositBytes + kStages * kStageBytes + 16 * 8;
-  static_assert(kSmemBytes <= 232448, "shared memory of a block");
+  static_assert(kSmemBytes + 16 <= 232448, "shared memory of a block");
   static_assert(kT * kMaxFusedSteps <= kDepMaxAdds, "a stage's deposits fit the digit words");
 };
 
@@ -420,12 +420,26 @@ __device__ __forceinline__ int32_t global_cell(const int (&uo)[3], const int (&n
   return (c & kFarCell) ? (int32_t)(c & ~kFarCell) : pack_cell(g[0], g[1], g[2]);
 }
 
-// A commit outside the deposit tile (rare), straight to the global accumulator.  Nothing bounds how many of
-// these one word gets in a launch, so a word found beyond 2^60 passes 2^34 of its value on to the next
+// A commit outside the deposit tile, straight to the global accumulator.  A CTA's first kFarFree of a launch are plain
+// reductions that nothing waits for; the count of adds allows for them.  Nothing bounds how many more one word gets
+// in a launch, so these look at it: a word found beyond 2^60 passes 2^34 of its value on to the next
 // word: each such add then takes more off than it put on, and the adds in flight on a GPU (fewer than
-// 2^19 of less than 2^32) cannot carry a word from there to 2^62.  The sum over the words is unchanged.
-__device__ __forceinline__ void far_digit(long long* p, int k, long long d) {
+// 2^19 of less than 2^32) cannot carry a word from there to 2^62.  The sum over the words is unchanged.  (All of
+// them waiting for the word: ten steps of 5e8 particles on 256^3 48.2 ms against 46.8 ms.)
+__device__ __forceinline__ int* far_count() {  // the CTA's commits of this launch, up to about kFarFree
+  __shared__ int n;
+  return &n;
+}
+__device__ __forceinline__ bool far_free() {
+  volatile int* n = far_count();
+  return *n < kFarFree && atomicAdd(far_count(), 1) < kFarFree;
+}
+__device__ __forceinline__ void far_digit(long long* p, int k, long long d, bool free) {
   if (d == 0 || k >= kAccWords) return;
+  if (free) {
+    atomicAdd((unsigned long long*)&p[k], (unsigned long long)d);
+    return;
+  }
   const long long old = (long long)atomicAdd((unsigned long long*)&p[k], (unsigned long long)d);
   constexpr long long lim = 1ll << 60;
   if (k + 1 < kAccWords && (old > lim || old < -lim)) {
@@ -437,6 +451,7 @@ __device__ __forceinline__ void far_digit(long long* p, int k, long long d) {
 __device__ __noinline__ void commit_far(const TmaArgs& a, unsigned cell, float r0, float r1, float r2) {
   const int64_t c = cell_i((int32_t)cell) + (int64_t)a.nx * (cell_j((int32_t)cell) + (int64_t)a.ny * cell_k((int32_t)cell));
   const float r[3] = {r0, r1, r2};
+  const bool free = far_free();
 #pragma unroll 1
   for (int q = 0; q < 3; ++q) {
     const uint32_t b = __float_as_uint(r[q]);
@@ -452,8 +467,8 @@ __device__ __noinline__ void commit_far(const TmaArgs& a, unsigned cell, float r
     const unsigned long long lo = man << (s & 31);  // man < 2^24: below 2^55
     const long long sg = (b >> 31) ? -1ll : 1ll;
     long long* p = a.acc + kAccWords * (q * a.ncell + c);
-    far_digit(p, s >> 5, sg * (long long)(lo & 0xffffffffull));
-    far_digit(p, (s >> 5) + 1, sg * (long long)(lo >> 32));
+    far_digit(p, s >> 5, sg * (long long)(lo & 0xffffffffull), free);
+    far_digit(p, (s >> 5) + 1, sg * (long long)(lo >> 32), free);
   }
 }
 
@@ -562,6 +577,7 @@ __global__ void __maxnreg__(Shape<PHYS>::kRegs) step_mixed_tma_kernel(const __gr
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
+    *far_count() = 0;
     for (int s = 0; s < kStages; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], kConsumerWarps);
@@ -1297,7 +1313,7 @@ cudaError_t launch_step_mixed_tma(st_ctx* h, const StepParams& p, bool records, 
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->dev);
   int grid = sms > 0 ? sms : 152;
-  if (grid > a.nunits) grid = a.nunits;
+  grid = std::min(std::min(grid, a.nunits), kFarCtas);
   kern<<<grid, threads, smem, h->stream>>>(map, a);
   h->launches += 1;
   return cudaGetLastError();

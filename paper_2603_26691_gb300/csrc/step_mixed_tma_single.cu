@@ -6,7 +6,7 @@
 // that: 4 consecutive particles per lane and 15 consumer warps at 128 registers, larger stages, whole-lane
 // 128-bit stores ahead of the deposit, coefficients in registers.  Its arithmetic and the order of its sums are those
 // of the multi-step kernel, so the results are the same to the bit whichever takes a step.  1e9 particles on
-// 256^3: 12.8 ms a step against 14.9 ms there; 6e7 on 128^3 9.0 against 9.9 ms for ten, the paper's physics 9.8
+// 256^3: 12.5 ms a step against 14.9 ms there; 6e7 on 128^3 9.0 against 9.9 ms for ten, the paper's physics 9.8
 // against 11.6 ms.  The cloud-in-cell deposit, bound by its adds, is faster there (10.4 against 13.6 ms at 2e7).
 // A unit of more particles than the tile's digit words take (the multi-step kernel flushes the tile in between) sends
 // its sums to the global accumulator.
@@ -311,12 +311,26 @@ __device__ __forceinline__ void dep_add3(int* w, float r0, float r1, float r2, f
 
 // one run record: into the shared deposit tile, or (start cell outside the tile, rare) straight to
 // the global accumulator, counted for the carry-propagation decision
-// A commit outside the deposit tile (rare), straight to the global accumulator.  Nothing bounds how many of
-// these one word gets in a launch, so a word found beyond 2^60 passes 2^34 of its value on to the next
+// A commit outside the deposit tile, straight to the global accumulator.  A CTA's first kFarFree of a launch are plain
+// reductions that nothing waits for; the count of adds allows for them.  Nothing bounds how many more one word gets
+// in a launch, so these look at it: a word found beyond 2^60 passes 2^34 of its value on to the next
 // word: each such add then takes more off than it put on, and the adds in flight on a GPU (fewer than
-// 2^19 of less than 2^32) cannot carry a word from there to 2^62.  The sum over the words is unchanged.
-__device__ __forceinline__ void far_digit(long long* p, int k, long long d) {
+// 2^19 of less than 2^32) cannot carry a word from there to 2^62.  The sum over the words is unchanged.  (All of
+// them waiting for the word: the last steps before a sort of 1e9 particles on 256^3 16.0 and 18.3 ms against 13.5 and 15.1.)
+__device__ __forceinline__ int* far_count() {  // the CTA's commits of this launch, up to about kFarFree
+  __shared__ int n;
+  return &n;
+}
+__device__ __forceinline__ bool far_free() {
+  volatile int* n = far_count();
+  return *n < kFarFree && atomicAdd(far_count(), 1) < kFarFree;
+}
+__device__ __forceinline__ void far_digit(long long* p, int k, long long d, bool free) {
   if (d == 0 || k >= kAccWords) return;
+  if (free) {
+    atomicAdd((unsigned long long*)&p[k], (unsigned long long)d);
+    return;
+  }
   const long long old = (long long)atomicAdd((unsigned long long*)&p[k], (unsigned long long)d);
   constexpr long long lim = 1ll << 60;
   if (k + 1 < kAccWords && (old > lim || old < -lim)) {
@@ -332,6 +346,7 @@ __device__ __noinline__ void commit_far(const TmaArgs& a, int3 uo, bool big, int
   bool in = big;
   for (int q = 0; q < 3; ++q) in = in && (g[q] - o[q] + kR + 2 * n[q]) % n[q] < kDE;
   const float r[3] = {r0, r1, r2};
+  const bool free = far_free();
 #pragma unroll 1
   for (int q = 0; q < 3; ++q) {
     float t = r[q] * a.s1 * a.s2;  // tile units, exact
@@ -348,8 +363,8 @@ __device__ __noinline__ void commit_far(const TmaArgs& a, int3 uo, bool big, int
     const unsigned long long lo = (unsigned long long)man << (s & 31);
     const long long sg = (b >> 31) ? -1ll : 1ll;
     long long* p = a.acc + kAccWords * ((int64_t)q * a.ncell + c);
-    far_digit(p, s >> 5, sg * (long long)(lo & 0xffffffffull));
-    far_digit(p, (s >> 5) + 1, sg * (long long)(lo >> 32));
+    far_digit(p, s >> 5, sg * (long long)(lo & 0xffffffffull), free);
+    far_digit(p, (s >> 5) + 1, sg * (long long)(lo >> 32), free);
   }
 }
 
@@ -424,6 +439,7 @@ __global__ void __maxnreg__(128) step_mixed_tma_single_kernel(const __grid_const
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
+    *far_count() = 0;
     for (int s = 0; s < kStages; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], kConsumerWarps);
@@ -1100,7 +1116,7 @@ cudaError_t launch_step_mixed_tma_single(st_ctx* h, const StepParams& p, bool re
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->dev);
   int grid = sms > 0 ? sms : 152;
-  if (grid > a.nunits) grid = a.nunits;
+  grid = std::min(std::min(grid, a.nunits), kFarCtas);
   kern<<<grid, kThreads, kSmemBytes, h->stream>>>(map, a);
   h->launches += 1;
   return cudaGetLastError();

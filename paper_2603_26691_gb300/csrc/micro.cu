@@ -395,7 +395,8 @@ __device__ __forceinline__ void micro_commit(const MixedArgs& a, GroupBuf<5>& b,
   }
 }
 
-template <bool BF16>
+// ONE: one step, without the loop (ten single steps of 2e7 droplets on 128^3: 8.5 -> 8.2 ms)
+template <bool BF16, bool ONE>
 __global__ void __launch_bounds__(kMicroThreads) micro_mixed_kernel(const MixedArgs a) {
   __shared__ GroupBuf<5> perm[kMicroThreads / 32];
   const int lane = threadIdx.x & 31;
@@ -422,7 +423,7 @@ __global__ void __launch_bounds__(kMicroThreads) micro_mixed_kernel(const MixedA
     // own, so the results do not depend on how the steps are split over launches
     GroupBuf<5>& gb = perm[threadIdx.x >> 5];
 #pragma unroll 1
-    for (int step = 0; step < a.nsteps; ++step) {
+    for (int step = 0; step < (ONE ? 1 : a.nsteps); ++step) {
       int key = -1;
       float gain[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
       if (p < a.n) micro_particle<BF16>(a, n3, px, pxy, cell, xi, v, dhi, st, key, gain);
@@ -673,9 +674,9 @@ cudaError_t launch_micro_step(st_ctx* h, const StepParams& p, bool records) {
     a.E = p.E;
     a.c = micro_const<float>(h);
     if (bf)
-      micro_mixed_kernel<true><<<blocks, kMicroThreads, 0, h->stream>>>(a);
+      (a.nsteps == 1 ? micro_mixed_kernel<true, true> : micro_mixed_kernel<true, false>)<<<blocks, kMicroThreads, 0, h->stream>>>(a);
     else
-      micro_mixed_kernel<false><<<blocks, kMicroThreads, 0, h->stream>>>(a);
+      (a.nsteps == 1 ? micro_mixed_kernel<false, true> : micro_mixed_kernel<false, false>)<<<blocks, kMicroThreads, 0, h->stream>>>(a);
   }
   h->launches += 1;
   return cudaGetLastError();

@@ -217,8 +217,9 @@ __device__ __forceinline__ void drag(const MixedArgs& a, float adt, float inv_a,
   }
 }
 
-// DEP: the impulses are deposited (CIC: cloud in cell)
-template <bool BF16, bool CIC, bool DEP>
+// DEP: the impulses are deposited (CIC: cloud in cell); ONE: one step and no tape, without the loop
+// (ten single steps of 2e7 particles on 100 x 84 x 60: 5.08 -> 4.93 ms, of 2e6 0.73 -> 0.71)
+template <bool BF16, bool CIC, bool DEP, bool ONE>
 __global__ void __launch_bounds__(256, DEP ? 2 : 4) step_mixed_kernel(const MixedArgs a) {
   constexpr int kP = kPerLane<DEP>, kPW = 32 * kP;  // particles per lane, per warp
   const int lane = threadIdx.x & 31;
@@ -257,9 +258,9 @@ __global__ void __launch_bounds__(256, DEP ? 2 : 4) step_mixed_kernel(const Mixe
       }
     }
     char* slot = a.tape;
-    int next = a.tape ? a.tape_first : a.nsteps;
+    int next = ONE ? -1 : a.tape ? a.tape_first : a.nsteps;
 #pragma unroll 1
-    for (int step = 0; step < a.nsteps; ++step) {
+    for (int step = 0; step < (ONE ? 1 : a.nsteps); ++step) {
       int key[kP];
       float J[kP][3];
 #pragma unroll
@@ -270,7 +271,7 @@ __global__ void __launch_bounds__(256, DEP ? 2 : 4) step_mixed_kernel(const Mixe
       // cloud-in-cell deposit: the start-of-step stencil's lower corner (periodic) and weights
       int sb[CIC ? kP : 1][3];
       float sf[CIC ? kP : 1][3];
-      if (step == next) {
+      if (!ONE && step == next) {
         if (nvalid > 0) {
           float* f = (float*)slot;
           st((int*)slot + p0, cell);
@@ -459,10 +460,15 @@ cudaError_t launch_step_mixed_tape(st_ctx* h, const MixedState& in, const MixedS
   int64_t blocks = (warps * 32 + 255) / 256;
   if (blocks > 152 * 8) blocks = 152 * 8;
   if (blocks < 1) blocks = 1;
-  void (*kern)(const MixedArgs) =
-      !acc ? (bf ? step_mixed_kernel<true, false, false> : step_mixed_kernel<false, false, false>)
-      : bf ? (p.cic ? step_mixed_kernel<true, true, true> : step_mixed_kernel<true, false, true>)
-           : (p.cic ? step_mixed_kernel<false, true, true> : step_mixed_kernel<false, false, true>);
+  const bool one = p.nsteps == 1 && !tape;
+  static void (*const dep[8])(const MixedArgs) = {
+      step_mixed_kernel<false, false, true, false>, step_mixed_kernel<true, false, true, false>,
+      step_mixed_kernel<false, true, true, false>,  step_mixed_kernel<true, true, true, false>,
+      step_mixed_kernel<false, false, true, true>,  step_mixed_kernel<true, false, true, true>,
+      step_mixed_kernel<false, true, true, true>,   step_mixed_kernel<true, true, true, true>};
+  void (*kern)(const MixedArgs) = acc  ? dep[(int)bf + 2 * (int)(p.cic != 0) + 4 * (int)one]
+                                  : bf ? step_mixed_kernel<true, false, false, false>
+                                       : step_mixed_kernel<false, false, false, false>;
   kern<<<(int)blocks, 256, 0, h->stream>>>(a);
   h->launches += 1;
   return cudaGetLastError();

@@ -425,7 +425,8 @@ __device__ __forceinline__ int32_t global_cell(const int (&uo)[3], const int (&n
 // in a launch, so these look at it: a word found beyond 2^60 passes 2^34 of its value on to the next
 // word: each such add then takes more off than it put on, and the adds in flight on a GPU (fewer than
 // 2^19 of less than 2^32) cannot carry a word from there to 2^62.  The sum over the words is unchanged.  (All of
-// them waiting for the word: ten steps of 5e8 particles on 256^3 48.2 ms against 46.8 ms.)
+// them waiting for the word: a call of ten steps of 5e8 particles on 256^3, with its
+// export, 62.6 ms against 61.2 ms.)
 __device__ __forceinline__ int* far_count() {  // the CTA's commits of this launch, up to about kFarFree
   __shared__ int n;
   return &n;

@@ -768,6 +768,7 @@ cudaError_t launch_adjoint_step(st_ctx* h, const AdjointStepArgs& s) {
 }
 
 cudaError_t launch_adjoint_segment(st_ctx* h, const AdjointStepArgs& s, int len) {
+  if (!h->fluid_fix.p) return cudaErrorInvalidValue;
   SegArgs a;
   a.tape = s.x[0];
   a.d = s.d;

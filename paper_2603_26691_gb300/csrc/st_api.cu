@@ -1046,16 +1046,16 @@ st_status st_adjoint_backward(st_handle h, const double* lam, int lam_on_device,
   auto cleanup = [&]() {
     for (Buf* b : {&blam, &work, &tape, &adj, &abp, &Uw, &tmp}) dev_free(h, *b);
   };
-  st_status s = ST_OK;
-  if (!fixed_step_supported(h)) s = dev_alloc(h, work, (size_t)6 * n * sizeof(double));
-  if (s == ST_OK) s = dev_alloc(h, tape, (size_t)std::min(C, nsteps) * 6 * n * sizeof(double));
+  st_status s = dev_alloc(h, tape, (size_t)std::min(C, nsteps) * 6 * n * sizeof(double));
   if (s == ST_OK) s = dev_alloc(h, adj, (size_t)7 * n * sizeof(double));
   if (s == ST_OK) s = dev_alloc(h, abp, (size_t)kAdjBlocks * sizeof(double));
   if (s == ST_OK) s = dev_alloc(h, Uw, (size_t)nc * 3 * kWideWords * sizeof(long long));
   if (s == ST_OK && !lam_on_device) s = dev_alloc(h, blam, (size_t)3 * nc * sizeof(double));
-  // (the integer field may have gone for the others' sake)
-  if (s == ST_OK && !fixed_step_supported(h) && !work.p) s = dev_alloc(h, work, (size_t)6 * n * sizeof(double));
-  if (s == ST_OK && (!on_device)) s = dev_alloc(h, tmp, (size_t)(std::max<int64_t>(n, 3 * nc)) * sizeof(double));
+  if (s == ST_OK && !on_device) s = dev_alloc(h, tmp, (size_t)(std::max<int64_t>(n, 3 * nc)) * sizeof(double));
+  // any allocation above may have given the integer field up, so whether the segments can run on it is known only
+  // now; the one below is made where they cannot
+  const bool segments = s == ST_OK && fixed_step_supported(h);
+  if (s == ST_OK && !segments) s = dev_alloc(h, work, (size_t)6 * n * sizeof(double));
   if (s != ST_OK) {
     cleanup();
     return s;
@@ -1087,7 +1087,7 @@ st_status st_adjoint_backward(st_handle h, const double* lam, int lam_on_device,
   p.scale = 1.0;
   for (int seg = K - 1; seg >= 0 && e == cudaSuccess; --seg) {
     const int s0 = seg * C, s1 = std::min(nsteps, s0 + C);
-    if (!work.p) {
+    if (segments) {
       // the segment recomputed in one launch, its states kept on the tape (of a single step the checkpoint
       // is the tape), then reversed in one launch
       double* ck = (double*)h->ckpt.p + (size_t)seg * 6 * n;

@@ -360,6 +360,7 @@ bool fixed_step_supported(const st_ctx* h) {
 
 cudaError_t launch_step_f64_tape(st_ctx* h, const double* const (&in)[6], const F64State& s, long long* acc,
                                  const StepParams& p, double* tape, int first, int every) {
+  if (!h->fluid_fix.p) return cudaErrorInvalidValue;
   FixArgs a;
   for (int k = 0; k < 6; ++k) a.in[k] = in[k];
   a.s = s;

@@ -1,0 +1,92 @@
+"""Allocations that fail: the call reports it, or goes on without the buffers it can do without (the integer copy of an
+FP64 field), with the same results to rounding."""
+import numpy as np
+import pytest
+
+from paper_2603_26691_gb300 import _lib, inputs
+
+pytestmark = pytest.mark.gpu
+
+
+class _Failing:
+    """torch's allocator with the k-th call from now (or all from it on) returning nothing."""
+
+    def __init__(self, monkeypatch):
+        import torch
+
+        self.alloc, self.left, self.rest = torch.cuda.caching_allocator_alloc, -1, False
+        monkeypatch.setattr(torch.cuda, "caching_allocator_alloc", self)
+
+    def arm(self, k, rest):
+        self.left, self.rest = k, rest
+
+    def __call__(self, *a):
+        if self.left >= 0:
+            self.left -= 1
+            if self.left < 0:
+                self.left = 0 if self.rest else -1
+                raise MemoryError
+        return self.alloc(*a)
+
+
+def _adjoint_sim(n):
+    from paper_2603_26691_gb300.sim import Sim
+
+    pos, vel, d, _ = inputs.particles(5, 0, n, vmax=1.0)
+    sim = Sim(8, precision="fp64")
+    sim.set_params(reorder_every=0)
+    sim.set_fluid(inputs.taylor_green(8))
+    sim.add_particles(pos, d, vel)
+    return sim
+
+
+@pytest.mark.parametrize("rest", [False, True])
+@pytest.mark.parametrize("k", range(8))
+def test_adjoint_backward_with_a_failing_allocation(monkeypatch, k, rest):
+    """The k-th allocation of a backward pass with host outputs fails, once or with all after it."""
+    fail = _Failing(monkeypatch)
+    lam = np.random.default_rng(0).standard_normal((3, 512))
+    sim = _adjoint_sim(1000)
+    sim.adjoint_forward(12, 1e-3, 5)
+    want = sim.adjoint_backward(lam)
+    for attempt in range(2):
+        fail.arm(k if attempt == 0 else -1, rest)  # the second attempt finds memory again
+        try:
+            got = sim.adjoint_backward(lam)
+        except _lib.StError as e:
+            assert attempt == 0 and rest and e.status == _lib.ST_ERR_OOM
+            continue
+        # the bounds of the adjoint's other tests
+        for a, b in zip(want, got):
+            assert np.abs(np.asarray(a) - np.asarray(b)).max() <= 1e-9 * np.abs(np.asarray(a)).max()
+    fail.arm(-1, False)
+    sim.close()
+
+
+@pytest.mark.parametrize("rest", [False, True])
+@pytest.mark.parametrize("k", range(12))
+def test_couple_run_with_a_failing_allocation(monkeypatch, k, rest):
+    """The k-th allocation of a first coupled run fails, its sort's among them."""
+    fail = _Failing(monkeypatch)
+    out = []
+    for failing in (False, True):
+        sim = _adjoint_sim(1000)
+        sim.set_params(reorder_every=4)
+        sim.couple_params(steps_per_interval=3)
+        if failing:
+            fail.arm(k, rest)
+        try:
+            sim.couple_run(1, 1e-3)
+        except _lib.StError as e:
+            assert failing and rest and e.status == _lib.ST_ERR_OOM
+            fail.arm(-1, False)
+            sim.close()
+            return
+        fail.arm(-1, False)
+        pos, vel, _, ids = sim.particles()
+        o = np.argsort(ids)
+        out.append((pos[:, o], vel[:, o], sim.fluid(), sim.pending_sources()))
+        sim.close()
+    # FP64 throughout, a few steps: the parity bound of the FP64 tests
+    for a, b in zip(*out):
+        assert np.abs(a - b).max() <= 1e-10 * np.abs(a).max()

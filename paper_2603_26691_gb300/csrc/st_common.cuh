@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "../../include/scaletrack.h"
+#include "acc_count.h"
 
 namespace st {
 
@@ -119,9 +120,7 @@ struct st_ctx {
   int acc_E = 0;             // value = integer * 2^-acc_E
   bool acc_empty = true;
   double acc_load = 0.0;     // bound on |accumulated integer| (in units of 1), for overflow control
-  double acc_adds = 0.0;     // digits added to any word since the last carry propagation
-  bool acc_far = false;      // the sorted-step kernel ran since then: its own bound of 2^60 beside the digits
-  bool acc_on_device = false;  // steps were captured in a graph: the count lives on the device
+  st::AccCount acc_count;    // digits added to any word since the last carry propagation
 
   st::Buf red;               // small reduction scratch
   st::Buf flags;             // device error flags (bounded waits that gave up)
@@ -638,15 +637,13 @@ cudaError_t launch_rescale_acc(st_ctx* h, int shift);
 cudaError_t launch_normalize_acc(st_ctx* h);
 // the particle steps of st_step (sort when due, accumulator bookkeeping, step kernel)
 st_status run_steps(st_ctx* h, int nsteps, double dt);
-// word-capacity bookkeeping of the carry-save accumulator: the host counts the digits that launches can
-// have added to any word since the last carry propagation, and runs the propagation before a launch
-// that could overflow one (`add`: the launch's worst case).  far: the sorted-step kernel, whose commits
-// outside its tiles keep themselves below 2^60 and are not counted.  In a captured graph the count and
-// the decision are kernels (a replay adds to the words without the host), and they stay so for the handle.
+// the carries propagated before a launch that could overflow a word (`add`: the digits it adds to one at most;
+// far: the sorted-step kernel, whose commits outside its tiles keep themselves below 2^60 and are not counted); the
+// rule and who keeps the count: acc_count.h
 cudaError_t launch_acc_maybe_normalize(st_ctx* h, double add, bool far);
 cudaError_t reset_acc_counter(st_ctx* h);
-constexpr size_t kAccCounterOffset = 64;   // bytes into the flags buffer: uint64 counter
-constexpr size_t kAccFlagOffset = 72;      // int: 1 if the last check propagated carries
+bool stream_capturing(const st_ctx* h);   // the handle's stream is being captured into a graph
+constexpr size_t kAccCountOffset = 64;     // bytes into the flags buffer: AccDeviceCount
 constexpr size_t kFarFlagOffset = 84;      // int: the neighbourhood sort found a particle it cannot place
 constexpr size_t kUnitCounterOffset = 88;  // uint32[2]: the sorted-step kernel's next unit and finished CTAs
 cudaError_t launch_acc_to_f64(st_ctx* h, double* out, int E);

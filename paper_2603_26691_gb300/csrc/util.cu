@@ -580,54 +580,40 @@ cudaError_t launch_normalize_acc(st_ctx* h) {
   return e == cudaSuccess ? reset_acc_counter(h) : e;
 }
 
-// each int64 word takes digits of magnitude < 2^32: 2^31 of them cannot overflow it; beside far commits
-// (which stay within 2^60 and what is in flight, see the sorted-step kernel) 2^30 of them
-constexpr double kAddLimit = 2147483648.0 - 1048576.0, kAddLimitFar = 1073741824.0;
+__global__ void acc_decide_kernel(AccDeviceCount* __restrict__ c, double base, double add) { acc_decide(*c, base, add); }
+__global__ void acc_cleared_kernel(AccDeviceCount* __restrict__ c) { acc_cleared(*c); }
 
-__global__ void acc_decide_kernel(unsigned long long* __restrict__ ctr, int* __restrict__ flag, double add,
-                                  double before) {
-  unsigned long long c = *ctr + (unsigned long long)before;
-  const int f = (double)c + add > kAddLimitFar;
-  if (f) c = 1;  // after propagation every word holds one digit
-  *ctr = c + (unsigned long long)add;
-  *flag = f;
-}
-
-cudaError_t launch_acc_maybe_normalize(st_ctx* h, double add, bool far) {
-  const int64_t m = h->geo.ncell * 3;
+bool stream_capturing(const st_ctx* h) {
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(h->stream, &cap) != cudaSuccess) {
     cudaGetLastError();
-    cap = cudaStreamCaptureStatusNone;
+    return false;
   }
-  if (cap == cudaStreamCaptureStatusActive) h->acc_on_device = true;
-  if (h->acc_on_device) {
-    // the host's count so far goes with the first of these (replays of that launch add it again: more
-    // propagations, never fewer)
-    unsigned long long* ctr = (unsigned long long*)((char*)h->flags.p + kAccCounterOffset);
-    int* flag = (int*)((char*)h->flags.p + kAccFlagOffset);
-    acc_decide_kernel<<<1, 1, 0, h->stream>>>(ctr, flag, add, h->acc_adds);
-    h->acc_adds = 0.0;
-    normalize_kernel<<<grid_for(m), kThreads, 0, h->stream>>>((long long*)h->acc.p, m, flag);
-    h->launches += 2;
-    return cudaGetLastError();
-  }
-  if (h->acc_adds + add > (far || h->acc_far ? kAddLimitFar : kAddLimit)) {
-    normalize_kernel<<<grid_for(m), kThreads, 0, h->stream>>>((long long*)h->acc.p, m, nullptr);
+  return cap == cudaStreamCaptureStatusActive;
+}
+
+static AccDeviceCount* device_count(st_ctx* h) { return (AccDeviceCount*)((char*)h->flags.p + kAccCountOffset); }
+
+cudaError_t launch_acc_maybe_normalize(st_ctx* h, double add, bool far) {
+  const AccCount::Action act = h->acc_count.launch(add, far, stream_capturing(h));
+  if (act == AccCount::kNothing) return cudaSuccess;
+  const int* flag = nullptr;
+  if (act == AccCount::kAskDevice) {
+    acc_decide_kernel<<<1, 1, 0, h->stream>>>(device_count(h), h->acc_count.adds, add);
     h->launches += 1;
-    h->acc_adds = 1.0;
-    h->acc_far = false;
+    flag = &device_count(h)->propagate;
   }
-  h->acc_adds += add;
-  h->acc_far = h->acc_far || far;
+  const int64_t m = h->geo.ncell * 3;
+  normalize_kernel<<<grid_for(m), kThreads, 0, h->stream>>>((long long*)h->acc.p, m, flag);
+  h->launches += 1;
   return cudaGetLastError();
 }
 
 cudaError_t reset_acc_counter(st_ctx* h) {
-  h->acc_adds = 0.0;
-  h->acc_far = false;
-  if (!h->acc_on_device) return cudaSuccess;
-  return cudaMemsetAsync((char*)h->flags.p + kAccCounterOffset, 0, sizeof(unsigned long long), h->stream);
+  if (!h->acc_count.cleared(stream_capturing(h))) return cudaSuccess;
+  acc_cleared_kernel<<<1, 1, 0, h->stream>>>(device_count(h));
+  h->launches += 1;
+  return cudaGetLastError();
 }
 
 cudaError_t launch_acc_sum(st_ctx* h, double out[3]) {

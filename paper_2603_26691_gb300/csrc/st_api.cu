@@ -519,8 +519,7 @@ st_status st_num_particles(st_handle h, int64_t* n) {
   return ST_OK;
 }
 
-st_status st_reorder(st_handle h) {
-  ST_TRY(check_handle(h));
+static st_status reorder(st_handle h) {
   timer_begin(h, ST_TIMER_SORT, h->stream);
   const st_status ss = sort_particles(h);
   timer_end(h, ST_TIMER_SORT, h->stream);
@@ -529,6 +528,14 @@ st_status st_reorder(st_handle h) {
   h->sorted = true;
   h->steps_since_sort = 0;
   return ST_OK;
+}
+
+st_status st_reorder(st_handle h) {
+  ST_TRY(check_handle(h));
+  ST_TRY(reorder(h));
+  // the physics variants' steps after a sort that was asked for can be captured and replayed: the sort gathers at once
+  // (in the step loop the step that gathers follows in the same call)
+  return default_physics(h) ? ST_OK : materialize_state(h);
 }
 
 // Contributions one particle can make to one cell in one step: one, except that the cloud-in-cell
@@ -592,9 +599,10 @@ st_status run_steps(st_ctx* h, int nsteps, double dt) {
   if (h->micro_on && !default_physics(h))
     return set_error(h, ST_ERR_STATE, "microphysics runs with the default gather, integrator, drag and deposit only");
   const double pi = 3.14159265358979323846;
+  const bool capturing = stream_capturing(h);
   for (int s = 0; s < nsteps;) {
     if (h->np == 0) break;
-    if (h->reorder_every > 0 && (!h->sorted || h->steps_since_sort >= h->reorder_every)) ST_TRY(st_reorder(h));
+    if (h->reorder_every > 0 && (!h->sorted || h->steps_since_sort >= h->reorder_every)) ST_TRY(reorder(h));
     const bool tma = !h->micro_on && h->prec != ST_FP64 && h->sorted && tma_step_supported(h);
     // the field is frozen and particles do not act on each other, so a launch takes several steps where
     // its kernel can, up to the next sort
@@ -607,7 +615,8 @@ st_status run_steps(st_ctx* h, int nsteps, double dt) {
                                        1073741824.0 / (deposits_per_cell(h) * (double)h->np)}));
     if (h->reorder_every > 0) m = std::min(m, h->reorder_every - h->steps_since_sort);
     // a sort is due after these steps: they leave the state as records for its gather
-    const bool can_record = tma && h->reorder_every > 0 && h->state_alt.bytes >= (size_t)h->cap * 32;
+    // (not in a captured graph, whose replays go on from the arrays that the captured steps left)
+    const bool can_record = tma && h->reorder_every > 0 && h->state_alt.bytes >= (size_t)h->cap * 32 && !capturing;
     bool records = can_record && h->steps_since_sort + m >= h->reorder_every;
     // a sort that deferred its payload gather: these steps gather, unless it is another kernel.  Where they
     // write records too, those need the room of the stale state and the cells a place of their own; without
@@ -646,7 +655,7 @@ st_status run_steps(st_ctx* h, int nsteps, double dt) {
     if (h->micro_on) {
       // the step before a due sort leaves its output as records for the sort's gather
       const bool mrec = h->prec != ST_FP64 && h->reorder_every > 0 && h->steps_since_sort + m >= h->reorder_every &&
-                        h->state_alt.bytes >= (size_t)h->cap * 32;
+                        h->state_alt.bytes >= (size_t)h->cap * 32 && !capturing;
       e = launch_micro_step(h, p, mrec);
       if (e == cudaSuccess && mrec) h->records_pending = true;
     }

@@ -25,6 +25,8 @@ st_status cuda_check(st_ctx* h, cudaError_t e, const char* what) {
 // (the queued work that reads it has to end before it does), and the steps read the FP64 field.
 static bool give_up_fix(st_ctx* h) {
   if (!h->fluid_fix.p && !h->fluid_fix_next.p) return false;
+  // a captured graph may read it, and a stream that is being captured cannot be waited for
+  if (h->acc_count.on_device || stream_capturing(h)) return false;
   if (cudaStreamSynchronize(h->stream) != cudaSuccess) {
     cudaGetLastError();
     return false;

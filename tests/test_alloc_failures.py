@@ -90,3 +90,37 @@ def test_couple_run_with_a_failing_allocation(monkeypatch, k, rest):
     # FP64 throughout, a few steps: the parity bound of the FP64 tests
     for a, b in zip(*out):
         assert np.abs(a - b).max() <= 1e-10 * np.abs(a).max()
+
+
+def test_the_integer_field_stays_while_a_graph_may_read_it(monkeypatch):
+    """A failing allocation after steps were captured is reported; the graph's field is not given up for it."""
+    import torch
+
+    from paper_2603_26691_gb300.sim import Sim
+
+    fail = _Failing(monkeypatch)
+    pos, vel, d, _ = inputs.particles(5, 0, 1000, vmax=1.0)
+    out = []
+    for captured in (False, True):
+        stream = torch.cuda.Stream()
+        with torch.cuda.stream(stream):
+            sim = Sim(8, precision="fp64", stream=stream)
+            sim.set_params(reorder_every=0)
+            sim.set_fluid(inputs.taylor_green(8))
+            sim.add_particles(pos, d, vel)
+            if captured:
+                graph = torch.cuda.CUDAGraph()
+                with torch.cuda.graph(graph, stream=stream):
+                    sim.step(3, 1e-3)
+                fail.arm(0, False)
+                with pytest.raises(_lib.StError) as e:
+                    sim.sources(host=True)
+                assert e.value.status == _lib.ST_ERR_OOM
+                graph.replay()
+                stream.synchronize()
+            else:
+                sim.step(3, 1e-3)
+            out.append([*sim.particles(), sim.sources(host=True)])
+            sim.close()
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)

@@ -859,8 +859,11 @@ st_status sort_particles(st_ctx* h) {
   if (ensure(h, h->ids_alt, (size_t)h->cap * sizeof(uint32_t)) != ST_OK) return ST_ERR_OOM;
   // (without room for the cells apart, the last step before a sort is a launch of its own; while they are in
   // use the buffer has its size)
-  if (h->prec != ST_FP64 && !h->cells_apart && ensure(h, h->rec_cell, (size_t)h->cap * sizeof(int32_t)) != ST_OK)
+  if (h->prec != ST_FP64 && !h->cells_apart && h->rec_cell_missing != h->cap &&
+      ensure(h, h->rec_cell, (size_t)h->cap * sizeof(int32_t)) != ST_OK) {
+    h->rec_cell_missing = h->cap;  // not asked for again at every sort
     h->err.clear();
+  }
   if (h->hist.p != look_before || h->sort_epoch + kMaxPasses >= (1u << 30)) {
     // a new look-back buffer may hold anything, and once the 30-bit epoch tags are about to repeat
     // an old word could carry a current tag: clear the words so that no stale word carries an epoch

@@ -103,6 +103,7 @@ struct st_ctx {
   // swapped; the cells (the next sort's keys) then lie in rec_cell and `state` holds nothing current.
   bool cells_apart = false;
   st::Buf rec_cell;          // int32[cap] (mixed handles; null: given up for memory)
+  int64_t rec_cell_missing = 0;  // the capacity it could not be had for
 
   // kernel timers (st_timers_*): pending event pairs per kind, folded into sums on read
   bool timing = false;

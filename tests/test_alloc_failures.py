@@ -14,13 +14,14 @@ class _Failing:
     def __init__(self, monkeypatch):
         import torch
 
-        self.alloc, self.left, self.rest = torch.cuda.caching_allocator_alloc, -1, False
+        self.alloc, self.left, self.rest, self.calls = torch.cuda.caching_allocator_alloc, -1, False, 0
         monkeypatch.setattr(torch.cuda, "caching_allocator_alloc", self)
 
     def arm(self, k, rest):
         self.left, self.rest = k, rest
 
     def __call__(self, *a):
+        self.calls += 1
         if self.left >= 0:
             self.left -= 1
             if self.left < 0:
@@ -124,3 +125,32 @@ def test_the_integer_field_stays_while_a_graph_may_read_it(monkeypatch):
             sim.close()
     for a, b in zip(*out):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("prec", ["mixed_f32", "mixed_bf16"])
+def test_sorts_without_a_place_for_the_cells(monkeypatch, prec):
+    """The last buffer of a first sort, which it can do without, is missing: the same results, and later sorts do not
+    allocate (nor ask for it again)."""
+    from paper_2603_26691_gb300.sim import Sim
+
+    fail = _Failing(monkeypatch)
+    pos, vel, d, _ = inputs.particles(7, 0, 5000, vmax=1.0)
+    out, asked = [], []
+    for k in (-1, 9):
+        sim = Sim(16, precision=prec)
+        sim.set_params(reorder_every=4)
+        sim.set_fluid(inputs.taylor_green(16).astype(np.float32))
+        sim.add_particles(pos, d, vel)
+        fail.arm(k, False)
+        calls = []
+        for steps in (3, 4, 4, 4):  # each begins with a sort or has one inside
+            before = fail.calls
+            sim.step(steps, 1e-3)
+            assert fail.left == -1
+            calls.append(fail.calls - before)
+        asked.append(calls)
+        out.append([*sim.particles(), sim.sources(host=True)])
+        sim.close()
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
+    assert asked[0] == asked[1] and asked[0][2:] == [0, 0]

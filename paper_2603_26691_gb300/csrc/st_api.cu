@@ -370,13 +370,17 @@ st_status st_set_fluid(st_handle h, const void* u, int dtype, int on_device) {
   return ST_OK;
 }
 
-// exact: room for `need` particles and no more (a reservation, and the first particles of a handle); otherwise
-// geometrically, for particles that come in many calls
+// exact (a reservation, as the first particles of a handle): room for `need` particles and no more, unless that is less
+// than half as much again as there was; otherwise geometrically.  So neither particles nor reservations that come in
+// many small calls copy the particles in each of them.
 static st_status grow(st_handle h, int64_t need, bool exact) {
   if (need <= h->cap) return ST_OK;
   ST_TRY(materialize_state(h));
-  int64_t cap = exact || h->cap == 0 ? need : h->cap;
-  while (cap < need) cap = cap + cap / 2 + 64;
+  int64_t cap = h->cap == 0 ? need : h->cap;
+  while (cap < need) {
+    cap = cap + cap / 2 + 64;
+    if (exact && cap < need) cap = need;
+  }
   cap = (cap + 63) & ~int64_t(63);
   Buf ns, ni;
   // sized like the sort's spare buffer (room for 32-byte particle records on mixed handles): the

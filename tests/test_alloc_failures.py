@@ -154,3 +154,18 @@ def test_sorts_without_a_place_for_the_cells(monkeypatch, prec):
     for a, b in zip(*out):
         assert np.array_equal(a, b)
     assert asked[0] == asked[1] and asked[0][2:] == [0, 0]
+
+
+def test_small_reservations_do_not_reallocate_every_time(monkeypatch):
+    from paper_2603_26691_gb300.sim import Sim
+
+    fail = _Failing(monkeypatch)
+    sim = Sim(8, precision="mixed_f32")
+    fail.calls = 0
+    sim.reserve(10_000)
+    first = fail.calls
+    for n in range(10_100, 40_000, 100):
+        sim.reserve(n)
+    # 1.5-fold growth from 1e4 to 4e4 takes four steps
+    assert fail.calls <= 5 * first
+    sim.close()

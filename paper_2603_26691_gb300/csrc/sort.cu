@@ -969,7 +969,7 @@ static st_status run_deferred_gather(st_ctx* h) {
 }
 
 bool defer_gather(const st_ctx* h) {
-  return h->prec != ST_FP64 && !h->micro_on && tma_step_supported(h) && h->np > 0;
+  return h->prec != ST_FP64 && !h->micro_on && !h->temp.p && tma_step_supported(h) && h->np > 0;
 }
 
 void gather_step_done(st_ctx* h) {

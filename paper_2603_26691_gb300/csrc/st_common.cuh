@@ -678,7 +678,7 @@ cudaError_t launch_local_sort(st_ctx* h, int* far, uint32_t* lidx, uint16_t* lke
 // the structure of arrays current again if the last step left records for a sort (no-op otherwise)
 st_status materialize_state(st_ctx* h);                                    // sort.cu
 // whether a sort may leave its payload gather to the next step (mixed, sorted-step kernel, no
-// microphysics), and the bookkeeping once that step has gathered (ids swapped, nothing pending) and once a
+// microphysics and no temperatures kept from it, which the sort itself permutes), and the bookkeeping once that step has gathered (ids swapped, nothing pending) and once a
 // step has written records (apart: while it gathered)
 bool defer_gather(const st_ctx* h);                                        // sort.cu
 void gather_step_done(st_ctx* h);                                          // sort.cu

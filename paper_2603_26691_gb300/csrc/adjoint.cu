@@ -439,11 +439,11 @@ __global__ void __launch_bounds__(kSegThreads, 3) adjoint_segment_kernel(const S
         unsigned long long mag = ((b << 11) | 0x8000000000000000ull);
         mag = ((b << 1) == 0 || sh > 63 || !valid) ? 0ull : (mag >> sh) + ((mag >> (sh - 1)) & 1ull);
         const int64_t ui = (b >> 63) ? -(int64_t)mag : (int64_t)mag;
-        const int uh = (int)(ui >> fix::kLimb), ul = (int)(ui & fix::kLimbMask);
+        const int uh = (int)(ui >> 29), ul = (int)(ui & ((1 << 29) - 1));
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
-          const int wh = (int)(W[k] >> fix::kLimb), wl = (int)(W[k] & fix::kLimbMask);
-          sums.v[3 * k + q][t] += (int64_t)uh * wh + (((int64_t)uh * wl + (int64_t)ul * wh) >> fix::kLimb);
+          const int wh = (int)(W[k] >> 29), wl = (int)(W[k] & ((1 << 29) - 1));
+          sums.v[3 * k + q][t] += (int64_t)uh * wh + (((int64_t)uh * wl + (int64_t)ul * wh) >> 29);
         }
       }
     }

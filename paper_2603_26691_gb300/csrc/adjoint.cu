@@ -24,7 +24,6 @@ namespace st {
 namespace {
 
 constexpr int kAdjThreads = 256;
-constexpr int kAdjDirectGroups = 20;  // more distinct stencils than this in a warp: no grouping
 
 struct AdjArgs {
   const double* __restrict__ x[3];   // state at the start of the step (tape)
@@ -479,12 +478,13 @@ __global__ void __launch_bounds__(kSegThreads, 3) adjoint_segment_kernel(const S
 // start cell.  Position adjoints are per metre, as in the FP64 adjoint (the periodic wrap and the
 // whole-cell carry are translations); they and the velocity's stay in registers over the segment.  Each
 // step's dL/dd and dL/dalpha contributions are FP32 and accumulate in FP64, per particle and in the steps'
-// order.  dL/dU: the adjoint velocity's FP32 significand times the corner's weight (26 bits) is an exact integer;
-// the products are summed over the steps a particle stays in one stencil (commit_sums) and then over the
-// warp's lanes of the same stencil, so each sum, and so dL/dU, is the same however the steps are cut into
-// segments.  1e7 particles on 64^3 sorted once, 40 steps: 21.3 ms against 39.5 ms with warp sums and commits in
-// every step; 10 ms are the sweep itself, 1.2 ms the sums, and the rest the commits of the particles that
-// leave a stencil, bound by L2's 1.9e11 64-bit reductions a second.
+// order.  dL/dU: the FP32 products of the adjoint velocity and the corners' weights are integers in a unit that
+// reaches from 2^28 times below the first of them to 32 times above; they are summed over the steps a particle stays in
+// one stencil (commit_component) and then over the warp's lanes of the same stencil (commit_shared), all exactly, so
+// dL/dU is the same however the steps are cut into segments.  1e7 particles on 64^3 sorted once, 40 steps: 20.2 ms
+// against 39.5 ms with warp sums and commits in every step, and 21.3 ms with weights of 26 bits, which lost small ones
+// and could hold fewer adjoint velocities in a sum.  Half of it is the sweep with its sums, the rest the commits of the
+// particles that leave a stencil, bound by L2's 1.9e11 64-bit reductions a second.
 
 struct AdjMixedArgs {
   const char* __restrict__ tape;     // [len] states of 28 tape_n bytes
@@ -504,10 +504,32 @@ struct AdjMixedArgs {
   float dt, cadt, inv_ca, mcoef, g[3], gdt[3];
 };
 
-constexpr int kWeightBits = 26;  // weights of the sums: 2^26 = 1
-constexpr int kWindow = 7;       // adjoint velocities of exponents eb .. eb + kWindow are integers below 2^31 there
-constexpr int kBelow = 5;        // the exponents below the first one's that a sum takes (components cross zero)
-// |product| < 2^57, so kSumSteps of them fit 64 bits
+// Products of biased exponents eb .. eb + kWindow are integers below 2^57 in the sums, so that kSumSteps of them fit 64
+// bits; a sum starts with kBelow of them below its first adjoint velocity's (small weights, components that cross zero).
+constexpr int kWindow = 33, kBelow = 28;
+
+// the weight of corner k = dx + 2 dy + 4 dz
+__device__ __forceinline__ float corner_weight(const float (&f)[3], int k) {
+  return (k & 1 ? f[0] : 1.0f - f[0]) * (k & 2 ? f[1] : 1.0f - f[1]) * (k & 4 ? f[2] : 1.0f - f[2]);
+}
+
+// The products of the components `which` (a bit each), some of which a sum cannot hold (rare: weights below about
+// 2^-28), each straight to dL/dU.
+__device__ __noinline__ void commit_products(long long* __restrict__ Uw, unsigned which, SumRef r, float f0, float f1,
+                                             float f2, float ub0, float ub1, float ub2) {
+  const float f[3] = {f0, f1, f2};
+#pragma unroll 1
+  for (; which; which &= which - 1) {
+    const int q = __ffs(which) - 1;
+    const float ub = q == 0 ? ub0 : q == 1 ? ub1 : ub2;
+#pragma unroll 1
+    for (int k = 0; k < 8; ++k) {
+      const int c = r.c0 + ((k & 1) ? r.sx : 0) + ((k & 2) ? r.sy : 0) + ((k & 4) ? r.sz : 0);
+      const float p = __fmul_rn(corner_weight(f, k), ub);
+      if (p != 0.0f) add_f32_words(Uw + ((int64_t)c * 3 + q) * kWideWords, kWideWords, p, -kWideBase);
+    }
+  }
+}
 
 __global__ void __launch_bounds__(kSegThreads, 4) adjoint_segment_mixed_kernel(const AdjMixedArgs a) {
   __shared__ StencilSums sums;
@@ -568,15 +590,14 @@ __global__ void __launch_bounds__(kSegThreads, 4) adjoint_segment_mixed_kernel(c
       const int base = lo[0] + a.nx * (lo[1] + a.ny * lo[2]);
       const float4* b = a.Up + (i0[0] + kFluidPad) + (int64_t)row * (i0[1] + kFluidPad) + (int64_t)slab * (i0[2] + kFluidPad);
       float4 Uc[8];
-      float up[3] = {0.0f, 0.0f, 0.0f};
+      float up[3] = {0.0f, 0.0f, 0.0f}, W[8];
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
-        const int di = k & 1, dj = (k >> 1) & 1, dk = (k >> 2) & 1;
-        Uc[k] = __ldg(b + di + row * dj + slab * dk);
-        const float W = (di ? f[0] : 1.0f - f[0]) * (dj ? f[1] : 1.0f - f[1]) * (dk ? f[2] : 1.0f - f[2]);
-        up[0] = fmaf(W, Uc[k].x, up[0]);
-        up[1] = fmaf(W, Uc[k].y, up[1]);
-        up[2] = fmaf(W, Uc[k].z, up[2]);
+        Uc[k] = __ldg(b + (k & 1) + row * ((k >> 1) & 1) + slab * (k >> 2));
+        W[k] = corner_weight(f, k);
+        up[0] = fmaf(W[k], Uc[k].x, up[0]);
+        up[1] = fmaf(W[k], Uc[k].y, up[1]);
+        up[2] = fmaf(W[k], Uc[k].z, up[2]);
       }
       float wt[3], vn[3], ub[3];
 #pragma unroll
@@ -614,19 +635,17 @@ __global__ void __launch_bounds__(kSegThreads, 4) adjoint_segment_mixed_kernel(c
         const float h00 = dot[4] - dot[0], h10 = dot[5] - dot[1], h01 = dot[6] - dot[2], h11 = dot[7] - dot[3];
         xb[2] = fmaf(lerp(lerp(h00, h10, f[0]), lerp(h01, h11, f[0]), f[1]), a.inv_h[2], xb[2]);
       }
-      // dL/dU: sums of another stencil, or whose units cannot hold the adjoint velocity exactly, are committed and
-      // started anew
+      // dL/dU: sums of another stencil, or whose units cannot hold the adjoint velocity, are committed and started anew
       const bool moved = base != corner0;
 #pragma unroll
       for (int q = 0; q < 3; ++q) {
         const int eu = max((int)((__float_as_uint(ub[q]) >> 23) & 0xffu), 1);
-        const bool holds = ub[q] == 0.0f || (unsigned)(eu - eb[q]) <= (unsigned)kWindow;
-        const bool full = valid && added[q] && (moved || added[q] >= kSumSteps || !holds);
+        const bool full = valid && added[q] && (moved || added[q] >= kSumSteps || eu - eb[q] > kWindow);
         const unsigned who = __ballot_sync(0xffffffffu, full);
-        if (who) commit_component(sums, a.Uw, who, q, SumRef{corner0, c1x, c1y, c1z, eb[q]}, 150 + kWeightBits);
+        if (who) commit_component(sums, a.Uw, who, q, SumRef{corner0, c1x, c1y, c1z, eb[q]}, 150);
         if (full || added[q] == 0) {
           added[q] = 0;
-          eb[q] = eu - kBelow;
+          eb[q] = max(eu - kBelow, 1);
         }
         ++added[q];
       }
@@ -636,37 +655,40 @@ __global__ void __launch_bounds__(kSegThreads, 4) adjoint_segment_mixed_kernel(c
         c1y = a.nx * ((lo[1] + 1 == a.ny ? 0 : lo[1] + 1) - lo[1]);
         c1z = a.nx * a.ny * ((lo[2] + 1 == a.nz ? 0 : lo[2] + 1) - lo[2]);
       }
-      // the weights, adding up to 2^kWeightBits (differences of products, as in fix_gather.cuh)
-      int W[8];
-      {
-        constexpr int one = 1 << kWeightBits;
-        int fi[3];
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {  // floor(f 2^26), 0 <= f <= 1 (a conversion would take the FP64 pipe)
-          const uint32_t bits = __float_as_uint(f[q]), man = (bits & 0x7fffffu) | 0x800000u;
-          const int sh = (int)(bits >> 23) - (127 + 23 - kWeightBits);
-          fi[q] = (int)(sh >= 0 ? man << sh : man >> min(-sh, 31));
-        }
-        const int pxy = (int)(((int64_t)fi[0] * fi[1]) >> kWeightBits);
-        const int xy[4] = {max(one - fi[0] - fi[1] + pxy, 0), fi[0] - pxy, fi[1] - pxy, pxy};
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          W[4 + k] = (int)(((int64_t)xy[k] * fi[2]) >> kWeightBits);
-          W[k] = xy[k] - W[4 + k];
-        }
-      }
+      // the smallest weight that is not zero (rounding keeps the order of products)
+      float least[3];
 #pragma unroll
       for (int q = 0; q < 3; ++q) {
-        const uint32_t bits = __float_as_uint(ub[q]);
-        const uint32_t man = (bits & 0x7fffffu) | ((bits & 0x7f800000u) ? 0x800000u : 0u);
-        const int mag = ub[q] == 0.0f || !valid ? 0 : (int)(man << (max((int)((bits >> 23) & 0xffu), 1) - eb[q]));
-        const int ui = (bits >> 31) ? -mag : mag;
+        const float m = fminf(f[q], 1.0f - f[q]);
+        least[q] = m > 0.0f ? m : 1.0f;
+      }
+      const float Wmin = least[0] * least[1] * least[2];
+      // components with a product that their sums cannot hold, and those with any for the sums
+      unsigned lone = 0, summed = 0;
 #pragma unroll
-        for (int k = 0; k < 8; ++k) sums.v[3 * k + q][t] += (int64_t)ui * W[k];
+      for (int q = 0; q < 3; ++q) {
+        const int emin = (int)(__float_as_uint(Wmin * fabsf(ub[q])) >> 23);  // 0: subnormal
+        if (valid && ub[q] != 0.0f) (emin >= eb[q] ? summed : lone) |= 1u << q;
+      }
+      if (__any_sync(0xffffffffu, lone != 0u))
+        commit_products(a.Uw, lone, SumRef{corner0, c1x, c1y, c1z, 0}, f[0], f[1], f[2], ub[0], ub[1], ub[2]);
+      __syncwarp();
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        // a shift of 64 or more leaves nothing: of zeros (exponent 0 below eb >= 1), and of all where none is to be added
+        const int e0 = (summed >> q) & 1u ? eb[q] : 1 << 16;
+        const long long neg = ub[q] < 0.0f ? -1ll : 0ll;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const uint32_t bits = __float_as_uint(__fmul_rn(W[k], fabsf(ub[q])));
+          unsigned long long x = (bits & 0x7fffffu) | 0x800000u;
+          asm("shl.b64 %0, %0, %1;" : "+l"(x) : "r"((int)(bits >> 23) - e0));
+          sums.v[3 * k + q][t] += ((long long)x ^ neg) - neg;
+        }
       }
     }
     if (!valid) added[0] = added[1] = added[2] = 0;
-    commit_all(sums, a.Uw, added, corner0, c1x, c1y, c1z, eb, 150 + kWeightBits);
+    commit_all(sums, a.Uw, added, corner0, c1x, c1y, c1z, eb, 150);
     if (!valid) continue;
     a.db[p] = db;
     a.ab[p] = ab_sum;

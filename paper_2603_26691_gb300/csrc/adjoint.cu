@@ -197,15 +197,17 @@ __global__ void __launch_bounds__(kAdjThreads) adjoint_step_kernel(const AdjArgs
 //   * the interpolation and its derivatives by the position run on integers (fix_gather.cuh);
 //   * what the diameter decides is computed once per particle, and the adjoints of position, velocity and
 //     diameter stay in registers over the segment;
-//   * dL/dU: a particle's products of weight and adjoint velocity are integers too.  They are summed over the
-//     steps it stays in one stencil (64-bit sums in shared memory, in units of 2^-57 of the largest adjoint
-//     velocity they may hold: finer than the rounding of FP64 products of weights above 1/16) and each sum is
-//     added to the carry-save accumulator when the particle leaves the stencil or the segment ends: 24
-//     global commits of two or three 64-bit reductions per stencil instead of per step, which bound the sweep.
-// About 55 FP64 instructions are left per particle and step, against 349.  2e6 particles on 64^3, 40 steps: 20.7 ms
-// against 44.4 ms step by step.  Of these 15.7 ms are the sweep without the sums, at 12 warps per SM (168
-// registers; 16 warps with spills are no faster) waiting on its own instructions, 1.2 ms the sums and
-// 3.5 ms their commits.
+//   * dL/dU: a particle's products of weight and adjoint velocity are formed on integers too, each with a relative
+//     error below 2^-53 whatever the weight's size.  They are summed over the steps it stays in one stencil (96-bit
+//     sums in shared memory) and each sum is added to the carry-save accumulator when the particle leaves the stencil
+//     or the segment ends: 24 global commits of three or four 64-bit reductions per stencil instead of per step,
+//     which bound the sweep.  These sums are exact, and the diameter's run on over the segments, so the gradients do
+//     not depend on how the steps are cut into segments.
+// About 55 FP64 instructions are left per particle and step, against 349.  2e6 particles on 64^3, 40 steps: 23.0 ms
+// against 44.4 ms step by step; of these some 16 ms are the sweep without the sums, and the sums and their commits take
+// about as much as each other.  (With products and sums of 64 bits, which kept fewer bits of small weights than FP64
+// does, 20.6 ms.)  16 warps per SM at 128 registers: 12 at 168 take 0.9 ms more.  The loop over the components that adds
+// the products is not unrolled: the kernel is as large as the instruction cache likes (unrolled 24.1 ms).
 constexpr int kSegThreads = 128;
 // stencils in a warp up to which its lanes are summed before the commits at a segment's end (sorted particles,
 // 1e7 on 64^3: 22.9 ms with the line at 12 against 24.4 ms without sums across lanes; unsorted particles lie above
@@ -213,10 +215,30 @@ constexpr int kSegThreads = 128;
 constexpr int kSharedStencils = 12;
 
 // A thread's 24 running sums of products of corner weight k and adjoint velocity component q, integers in units
-// of 2^(eb[q] - bits), of the stencil with base cell c0 and steps sx, sy, sz to the next cells.
+// of 2^(eb[q] - bits), of the stencil with base cell c0 and steps sx, sy, sz to the next cells.  WIDE: of 96 bits.
+template <bool WIDE>
 struct StencilSums {
-  long long v[24][kSegThreads + 1];  // [3 k + q][thread]; padded: a commit reads columns
-  int e[3][kSegThreads];             // eb, read by the lanes that commit
+  unsigned long long v[24][kSegThreads + 1];  // [3 k + q][thread]; padded: a commit reads columns
+  int h[WIDE ? 24 : 1][kSegThreads + 1];      // bits 64 .. 95
+  int e[3][kSegThreads];                      // eb, read by the lanes that commit
+  // units that lanes may differ by to be summed first: their sums, aligned, have to fit 128 bits
+  static constexpr int kNear = WIDE ? 13 : 28;
+
+  __device__ __forceinline__ void clear(int t) {
+#pragma unroll
+    for (int i = 0; i < 24; ++i) {
+      v[i][t] = 0;
+      if (WIDE) h[i][t] = 0;
+    }
+  }
+  __device__ __forceinline__ __int128 take(int i, int t) {
+    const unsigned long long lo = v[i][t];
+    v[i][t] = 0;
+    if (!WIDE) return (long long)lo;
+    const long long hi = h[i][t];
+    h[i][t] = 0;
+    return (__int128)(((unsigned __int128)(unsigned long long)hi << 64) | lo);
+  }
 };
 
 // The sums of a lane's component q, and the stencil they belong to, for the commits below.
@@ -228,7 +250,8 @@ struct SumRef {
 // Adds component q's sums of the lanes `who` to dL/dU, all lanes of the warp together: four lanes' sums at a time,
 // one corner per lane.  (Few lanes leave their stencil in one step; each by itself would hold up the
 // others for its eight corners.)
-__device__ __noinline__ void commit_component(StencilSums& s, long long* __restrict__ Uw, unsigned who, int q, SumRef r,
+template <bool WIDE>
+__device__ __noinline__ void commit_component(StencilSums<WIDE>& s, long long* __restrict__ Uw, unsigned who, int q, SumRef r,
                                               int bits) {
   const int lane = threadIdx.x & 31, w0 = threadIdx.x & ~31, k = lane & 7;
   __syncwarp();
@@ -244,10 +267,13 @@ __device__ __noinline__ void commit_component(StencilSums& s, long long* __restr
               sy = __shfl_sync(0xffffffffu, r.sy, from), sz = __shfl_sync(0xffffffffu, r.sz, from),
               e = __shfl_sync(0xffffffffu, r.e, from);
     if (src >= 0) {
-      long long& v = s.v[3 * k + q][w0 + src];
+      const __int128 v = s.take(3 * k + q, w0 + src);
       const int c = c0 + ((k & 1) ? sx : 0) + ((k & 2) ? sy : 0) + ((k & 4) ? sz : 0);
-      wide_add_int(Uw + ((int64_t)c * 3 + q) * kWideWords, v, e - bits);
-      v = 0;
+      long long* w = Uw + ((int64_t)c * 3 + q) * kWideWords;
+      if (WIDE)
+        wide_add_int128(w, v, e - bits);
+      else
+        wide_add_int(w, (long long)v, e - bits);
     }
   }
   __syncwarp();
@@ -256,8 +282,10 @@ __device__ __noinline__ void commit_component(StencilSums& s, long long* __restr
 // The same for all lanes and components where many lanes share few stencils (sorted particles at the end of a
 // segment): the lanes of one stencil whose units are near enough are summed first.  The sums are exact, so
 // their order does not matter.
-__device__ __noinline__ void commit_shared(StencilSums& s, long long* __restrict__ Uw, unsigned who, int c0, int sx, int sy,
-                                           int sz, int e0, int e1, int e2, int bits) {
+template <bool WIDE>
+__device__ __noinline__ void commit_shared(StencilSums<WIDE>& s, long long* __restrict__ Uw, unsigned who, int c0, int sx,
+                                           int sy, int sz, int e0, int e1, int e2, int bits) {
+  constexpr int kNear = StencilSums<WIDE>::kNear;
   const int t = threadIdx.x, lane = t & 31, w0 = t & ~31;
   const bool need = (who >> lane) & 1u;
   s.e[0][t] = e0;
@@ -268,18 +296,17 @@ __device__ __noinline__ void commit_shared(StencilSums& s, long long* __restrict
     const int src = __ffs(who) - 1;
     const int b0 = __shfl_sync(0xffffffffu, c0, src), bx = __shfl_sync(0xffffffffu, sx, src),
               by = __shfl_sync(0xffffffffu, sy, src), bz = __shfl_sync(0xffffffffu, sz, src);
-    const bool same = need && ((who >> lane) & 1u) && c0 == b0 && abs(e0 - s.e[0][w0 + src]) <= 28 &&
-                      abs(e1 - s.e[1][w0 + src]) <= 28 && abs(e2 - s.e[2][w0 + src]) <= 28;
+    const bool same = need && ((who >> lane) & 1u) && c0 == b0 && abs(e0 - s.e[0][w0 + src]) <= kNear &&
+                      abs(e1 - s.e[1][w0 + src]) <= kNear && abs(e2 - s.e[2][w0 + src]) <= kNear;
     const unsigned grp = __ballot_sync(0xffffffffu, same);
     who &= ~grp;
     if (lane < 24) {
       const int k = lane / 3, q = lane - 3 * k;
-      const int low = s.e[q][w0 + src] - 28;
+      const int low = s.e[q][w0 + src] - kNear;
       __int128 sum = 0;
       for (unsigned g = grp; g; g &= g - 1u) {
         const int m = w0 + __ffs(g) - 1;
-        sum += (__int128)s.v[lane][m] << (s.e[q][m] - low);
-        s.v[lane][m] = 0;
+        sum += s.take(lane, m) << (s.e[q][m] - low);
       }
       const int c = b0 + ((k & 1) ? bx : 0) + ((k & 2) ? by : 0) + ((k & 4) ? bz : 0);
       wide_add_int128(Uw + ((int64_t)c * 3 + q) * kWideWords, sum, low - bits);
@@ -289,7 +316,8 @@ __device__ __noinline__ void commit_shared(StencilSums& s, long long* __restrict
 }
 
 // every lane's sums that hold anything (added), at the end of a segment
-__device__ __forceinline__ void commit_all(StencilSums& s, long long* __restrict__ Uw, const int (&added)[3], int c0,
+template <bool WIDE>
+__device__ __forceinline__ void commit_all(StencilSums<WIDE>& s, long long* __restrict__ Uw, const int (&added)[3], int c0,
                                            int sx, int sy, int sz, const int (&eb)[3], int bits) {
   const bool need = added[0] || added[1] || added[2];
   const unsigned who = __ballot_sync(0xffffffffu, need);
@@ -303,33 +331,134 @@ __device__ __forceinline__ void commit_all(StencilSums& s, long long* __restrict
   }
 }
 
-constexpr int kSumBits = 57;   // adjoint velocities below 2^eb are integers below 2^kSumBits in the sums
 constexpr int kSumSteps = 32;  // products one sum takes
+// Products are integers below 2^57 (FP64) or 2^24 (FP32), shifted up by 0 .. window, so kSumSteps of them fit 96 or 64
+// bits; a sum starts with `below` of the window below its first adjoint velocity's exponent (small weights, components
+// that cross zero).  (FP64's shifts stay below a word's 32.)
+template <bool WIDE>
+struct Window {
+  static constexpr int kWindow = WIDE ? 31 : 33, kBelow = WIDE ? 26 : 28;
+};
+
+// The trilinear weights with a relative error below 2^-58 each, whatever their size (the integers of fix::weights have 58
+// below the point): corner k = dx + 2 dy + 4 dz has the weight m[k] 2^(-46 - c[k]).
+// a b / 2^64, up to three units low (the product of the low halves is not formed)
+__device__ __forceinline__ unsigned long long mul_high(unsigned long long a, unsigned long long b) {
+  const uint32_t ah = (uint32_t)(a >> 32), al = (uint32_t)a, bh = (uint32_t)(b >> 32), bl = (uint32_t)b;
+  return (unsigned long long)ah * bh + __umulhi(ah, bl) + __umulhi(al, bh);
+}
+struct FloatWeights {
+  unsigned long long m[8];
+  int c[8];
+};
+// the largest c of a weight that is not zero
+__device__ __forceinline__ int smallest_weight(const int64_t (&f)[3]) {
+  int c = 0;
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    const int64_t m = min(f[q], fix::kOne - f[q]);
+    c += m > 0 ? __clzll(m) : 63 - fix::kFrac;
+  }
+  return c;
+}
+__device__ __forceinline__ void float_weights(const int64_t (&f)[3], FloatWeights& w) {
+  unsigned long long g[3][2];
+  int c[3][2];
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    const unsigned long long a = (unsigned long long)(fix::kOne - f[q]), b = (unsigned long long)f[q];  // a > 0
+    c[q][0] = __clzll((long long)a);
+    c[q][1] = b ? __clzll((long long)b) : 63 - fix::kFrac;  // a zero stays zero
+    g[q][0] = a << c[q][0];
+    g[q][1] = b << c[q][1];
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const unsigned long long xy = mul_high(g[0][k & 1], g[1][k >> 1]);
+    w.m[k] = mul_high(xy, g[2][0]);
+    w.m[4 + k] = mul_high(xy, g[2][1]);
+    w.c[k] = c[0][k & 1] + c[1][k >> 1] + c[2][0];
+    w.c[4 + k] = c[0][k & 1] + c[1][k >> 1] + c[2][1];
+  }
+}
+// |u| = m 2^(e - 1086), m at least 2^63, for u != 0
+__device__ __forceinline__ void float_value(double u, unsigned long long& m, int& e) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(u);
+  e = (int)((b >> 52) & 0x7ff);
+  m = (b << 11) | 0x8000000000000000ull;
+  if (__builtin_expect(e == 0, 0)) {  // subnormal
+    const int z = __clzll((long long)(b << 1 >> 1));
+    m = b << z;
+    e = 12 - z;
+  }
+}
+// their product: a whole number of at most 57 bits (53 at least), times 2^(e - c[k] - kProductBits), off by less than
+// 2^-53 of itself
+constexpr int kProductBits = 1061;
+__device__ __forceinline__ unsigned long long product(unsigned long long w, unsigned long long u) {
+  return (mul_high(w, u) + 64) >> 7;
+}
+
+// The products of the components `which` (a bit each), some of which a sum cannot hold (rare: weights below about
+// 2^-26), each straight to dL/dU.
+__device__ __noinline__ void commit_products(long long* __restrict__ Uw, unsigned which, SumRef r, int64_t f0, int64_t f1,
+                                             int64_t f2, double ub0, double ub1, double ub2) {
+  const int64_t f[3] = {f0, f1, f2};
+  FloatWeights w;
+  float_weights(f, w);
+#pragma unroll 1
+  for (; which; which &= which - 1) {
+    const int q = __ffs(which) - 1;
+    const double ub = q == 0 ? ub0 : q == 1 ? ub1 : ub2;
+    unsigned long long u;
+    int e;
+    float_value(ub, u, e);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int c = r.c0 + ((k & 1) ? r.sx : 0) + ((k & 2) ? r.sy : 0) + ((k & 4) ? r.sz : 0);
+      const long long p = (long long)product(w.m[k], u);
+      wide_add_int(Uw + ((int64_t)c * 3 + q) * kWideWords, ub < 0.0 ? -p : p, e - w.c[k] - kProductBits);
+    }
+  }
+}
+
+constexpr int kWeightOne = 3 * (63 - fix::kFrac);  // FloatWeights::c of a weight of one
+static_assert(Window<true>::kWindow + 57 + 5 < 96 && Window<true>::kWindow < 32, "kSumSteps products fit 96 bits");
+
+// the 96-bit sum (v, h) plus (x2, x1, x0), or minus it (neg: all ones)
+__device__ __forceinline__ void add96(unsigned long long& v, int& h, uint32_t x0, uint32_t x1, uint32_t x2, int neg) {
+  uint32_t s0 = (uint32_t)v, s1 = (uint32_t)(v >> 32), s2 = (uint32_t)h, carry;
+  asm("add.cc.u32 %3, %7, 1;\n\taddc.cc.u32 %0, %0, %4;\n\taddc.cc.u32 %1, %1, %5;\n\taddc.u32 %2, %2, %6;"
+      : "+r"(s0), "+r"(s1), "+r"(s2), "=&r"(carry)
+      : "r"(x0 ^ neg), "r"(x1 ^ neg), "r"(x2 ^ neg), "r"(neg));
+  v = ((unsigned long long)s1 << 32) | s0;
+  h = (int)s2;
+}
 
 struct SegArgs {
   const double* __restrict__ tape;  // [len][6][n]
   const double* __restrict__ d;
   double* __restrict__ xb[3];
   double* __restrict__ vb[3];
-  double* __restrict__ db;
+  double* __restrict__ ab;  // sums over the segments so far for dL/da and dL/dm; after the last one ab is dL/dd
+  double* __restrict__ mb;
   double* __restrict__ ab_part;
   const fix::FixCell* __restrict__ U;
   const double* __restrict__ lam;
   long long* __restrict__ Uw;
   int64_t n, ncell;
-  int nx, ny, nz, len;
+  int nx, ny, nz, len, last;
   fix::Scale scale;
   double dt, mcoef, g[3];
   double inv_ca, inv_alpha;
 };
 
-__global__ void __launch_bounds__(kSegThreads, 3) adjoint_segment_kernel(const SegArgs a) {
-  __shared__ StencilSums sums;
+__global__ void __launch_bounds__(kSegThreads, 4) adjoint_segment_kernel(const SegArgs a) {
+  __shared__ StencilSums<true> sums;
   const int n3[3] = {a.nx, a.ny, a.nz};
   const int t = threadIdx.x;
   double alphab_sum = 0.0;
-#pragma unroll
-  for (int i = 0; i < 24; ++i) sums.v[i][t] = 0;
+  sums.clear(t);
   for (int64_t wbase = blockIdx.x * (int64_t)blockDim.x + (t & ~31); wbase < a.n;
        wbase += (int64_t)gridDim.x * blockDim.x) {
     __syncwarp();
@@ -354,7 +483,7 @@ __global__ void __launch_bounds__(kSegThreads, 3) adjoint_segment_kernel(const S
       xb[q] = a.xb[q][p];
       vb[q] = a.vb[q][p];
     }
-    double ab_sum = 0.0, mb_sum = 0.0;
+    double ab_sum = a.ab[p], mb_sum = a.mb[p];
     int corner0 = -1, c1x = 0, c1y = 0, c1z = 0;  // the stencil of the sums: its base cell, steps to the next cells
     int eb[3] = {0, 0, 0}, added[3] = {0, 0, 0};
 #pragma unroll 1
@@ -409,20 +538,28 @@ __global__ void __launch_bounds__(kSegThreads, 3) adjoint_segment_kernel(const S
         fix::derivative<2>(u, st.f, g);
         xb[2] += (g[0] * ub[0] + g[1] * ub[1] + g[2] * ub[2]) * a.scale.inv_h[2];
       }
-      // dL/dU: the adjoint velocities as integers in the sums' units; sums that cannot take them, or belong to
-      // another stencil, are committed and started anew
+      // dL/dU: sums of another stencil, or whose unit does not suit the products (too large, or too small as the adjoint
+      // velocity decays within a cell: 24.9 against 31.9 ms with such products committed by themselves), are committed
+      // and started anew; lone: components with a product that a new sum cannot hold either, summed: those with any for
+      // the sums
       const bool moved = base != corner0;
+      const int cmax = smallest_weight(st.f);
+      unsigned lone = 0, summed = 0;
 #pragma unroll
       for (int q = 0; q < 3; ++q) {
-        const int eu = (int)(((unsigned long long)__double_as_longlong(ub[q]) >> 52) & 0x7ff) - 1022;  // |ub| < 2^eu
-        const bool full = valid && added[q] && (moved || added[q] >= kSumSteps || eu > eb[q]);
+        const unsigned long long b = (unsigned long long)__double_as_longlong(ub[q]);
+        const int e = (int)((b >> 52) & 0x7ff), fresh = e - kWeightOne - Window<true>::kBelow;
+        const bool some = valid && (b << 1) != 0;
+        const bool suits = !some || (e - kWeightOne - eb[q] <= Window<true>::kWindow && (e - cmax >= eb[q] || fresh >= eb[q]));
+        const bool full = valid && added[q] && (moved || added[q] >= kSumSteps || !suits);
         const unsigned who = __ballot_sync(0xffffffffu, full);
-        if (who) commit_component(sums, a.Uw, who, q, SumRef{corner0, c1x, c1y, c1z, eb[q]}, kSumBits);
-        if (full || added[q] == 0) {
-          added[q] = 0;
-          eb[q] = eu + 1;
+        if (who) commit_component(sums, a.Uw, who, q, SumRef{corner0, c1x, c1y, c1z, eb[q]}, kProductBits);
+        if (full) added[q] = 0;
+        if (some) {
+          if (added[q] == 0) eb[q] = fresh;
+          ++added[q];
+          (e != 0 && e - cmax >= eb[q] ? summed : lone) |= 1u << q;
         }
-        ++added[q];
       }
       if (moved) {
         corner0 = base;
@@ -430,27 +567,39 @@ __global__ void __launch_bounds__(kSegThreads, 3) adjoint_segment_kernel(const S
         c1y = a.nx * (st.i1[1] - st.i0[1]);
         c1z = a.nx * a.ny * (st.i1[2] - st.i0[2]);
       }
-#pragma unroll
+      if (__any_sync(0xffffffffu, lone != 0u))
+        commit_products(a.Uw, lone, SumRef{corner0, c1x, c1y, c1z, 0}, st.f[0], st.f[1], st.f[2], ub[0], ub[1], ub[2]);
+      __syncwarp();
+      FloatWeights w;
+      float_weights(st.f, w);
+#pragma unroll 1
       for (int q = 0; q < 3; ++q) {
-        const unsigned long long b = (unsigned long long)__double_as_longlong(ub[q]);
-        // the significand, at 2^63 for |ub| in [2^(eu-1), 2^eu), down to units of 2^(eb - kSumBits)
-        const int sh = eb[q] - ((int)((b >> 52) & 0x7ff) - 1022) + 64 - kSumBits;
-        unsigned long long mag = ((b << 11) | 0x8000000000000000ull);
-        mag = ((b << 1) == 0 || sh > 63 || !valid) ? 0ull : (mag >> sh) + ((mag >> (sh - 1)) & 1ull);
-        const int64_t ui = (b >> 63) ? -(int64_t)mag : (int64_t)mag;
-        const int uh = (int)(ui >> 29), ul = (int)(ui & ((1 << 29) - 1));
+        const double ubq = q == 0 ? ub[0] : q == 1 ? ub[1] : ub[2];
+        const int ebq = q == 0 ? eb[0] : q == 1 ? eb[1] : eb[2];
+        const unsigned long long b = (unsigned long long)__double_as_longlong(ubq);
+        const int e = (int)((b >> 52) & 0x7ff);
+        const unsigned long long u = (summed >> q) & 1u ? (b << 11) | 0x8000000000000000ull : 0ull;
+        const int neg = (int)((long long)b >> 63), up = e - ebq;
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
-          const int wh = (int)(W[k] >> 29), wl = (int)(W[k] & ((1 << 29) - 1));
-          sums.v[3 * k + q][t] += (int64_t)uh * wh + (((int64_t)uh * wl + (int64_t)ul * wh) >> 29);
+          const unsigned long long p = product(w.m[k], u);
+          const uint32_t p0 = (uint32_t)p, p1 = (uint32_t)(p >> 32);
+          const int sh = up - w.c[k];  // 0 .. kWindow where the product is not zero
+          add96(sums.v[3 * k + q][t], sums.h[3 * k + q][t], p0 << (sh & 31), __funnelshift_l(p0, p1, sh),
+                __funnelshift_l(p1, 0u, sh), neg);
         }
       }
     }
     if (!valid) added[0] = added[1] = added[2] = 0;
-    commit_all(sums, a.Uw, added, corner0, c1x, c1y, c1z, eb, kSumBits);
+    commit_all(sums, a.Uw, added, corner0, c1x, c1y, c1z, eb, kProductBits);
     if (!valid) continue;
-    alphab_sum += ab_sum * ra * a.inv_alpha;
-    a.db[p] += ab_sum * (-2.0 * ra * inv_d) + mb_sum * (3.0 * m * inv_d);
+    if (a.last) {
+      alphab_sum += ab_sum * ra * a.inv_alpha;
+      a.ab[p] = ab_sum * (-2.0 * ra * inv_d) + mb_sum * (3.0 * m * inv_d);
+    } else {
+      a.ab[p] = ab_sum;
+      a.mb[p] = mb_sum;
+    }
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
       a.xb[q][p] = xb[q];
@@ -504,10 +653,6 @@ struct AdjMixedArgs {
   float dt, cadt, inv_ca, mcoef, g[3], gdt[3];
 };
 
-// Products of biased exponents eb .. eb + kWindow are integers below 2^57 in the sums, so that kSumSteps of them fit 64
-// bits; a sum starts with kBelow of them below its first adjoint velocity's (small weights, components that cross zero).
-constexpr int kWindow = 33, kBelow = 28;
-
 // the weight of corner k = dx + 2 dy + 4 dz
 __device__ __forceinline__ float corner_weight(const float (&f)[3], int k) {
   return (k & 1 ? f[0] : 1.0f - f[0]) * (k & 2 ? f[1] : 1.0f - f[1]) * (k & 4 ? f[2] : 1.0f - f[2]);
@@ -532,12 +677,11 @@ __device__ __noinline__ void commit_products(long long* __restrict__ Uw, unsigne
 }
 
 __global__ void __launch_bounds__(kSegThreads, 4) adjoint_segment_mixed_kernel(const AdjMixedArgs a) {
-  __shared__ StencilSums sums;
+  __shared__ StencilSums<false> sums;
   const int n3[3] = {a.nx, a.ny, a.nz};
   const int row = a.nx + 2 * kFluidPad, slab = row * (a.ny + 2 * kFluidPad);
   const int t = threadIdx.x;
-#pragma unroll
-  for (int i = 0; i < 24; ++i) sums.v[i][t] = 0;
+  sums.clear(t);
   for (int64_t wbase = blockIdx.x * (int64_t)blockDim.x + (t & ~31); wbase < a.n;
        wbase += (int64_t)gridDim.x * blockDim.x) {
     __syncwarp();
@@ -640,12 +784,12 @@ __global__ void __launch_bounds__(kSegThreads, 4) adjoint_segment_mixed_kernel(c
 #pragma unroll
       for (int q = 0; q < 3; ++q) {
         const int eu = max((int)((__float_as_uint(ub[q]) >> 23) & 0xffu), 1);
-        const bool full = valid && added[q] && (moved || added[q] >= kSumSteps || eu - eb[q] > kWindow);
+        const bool full = valid && added[q] && (moved || added[q] >= kSumSteps || eu - eb[q] > Window<false>::kWindow);
         const unsigned who = __ballot_sync(0xffffffffu, full);
         if (who) commit_component(sums, a.Uw, who, q, SumRef{corner0, c1x, c1y, c1z, eb[q]}, 150);
         if (full || added[q] == 0) {
           added[q] = 0;
-          eb[q] = max(eu - kBelow, 1);
+          eb[q] = max(eu - Window<false>::kBelow, 1);
         }
         ++added[q];
       }
@@ -800,7 +944,9 @@ cudaError_t launch_adjoint_segment(st_ctx* h, const AdjointStepArgs& s, int len)
     a.g[q] = h->g[q];
   }
   a.scale = fix::make_scale(h->geo.inv_h);
-  a.db = s.db;
+  a.ab = s.db;
+  a.mb = s.mb;
+  a.last = s.last;
   a.ab_part = s.ab_part;
   a.U = (const fix::FixCell*)h->fluid_fix.p;
   a.lam = s.lam;

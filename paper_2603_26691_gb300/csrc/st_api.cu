@@ -1062,7 +1062,7 @@ st_status st_adjoint_backward(st_handle h, const double* lam, int lam_on_device,
     for (Buf* b : {&blam, &work, &tape, &adj, &abp, &Uw, &tmp}) dev_free(h, *b);
   };
   st_status s = dev_alloc(h, tape, (size_t)std::min(C, nsteps) * 6 * n * sizeof(double));
-  if (s == ST_OK) s = dev_alloc(h, adj, (size_t)7 * n * sizeof(double));
+  if (s == ST_OK) s = dev_alloc(h, adj, (size_t)(fixed_step_supported(h) ? 8 : 7) * n * sizeof(double));
   if (s == ST_OK) s = dev_alloc(h, abp, (size_t)kAdjBlocks * sizeof(double));
   if (s == ST_OK) s = dev_alloc(h, Uw, (size_t)nc * 3 * kWideWords * sizeof(long long));
   if (s == ST_OK && !lam_on_device) s = dev_alloc(h, blam, (size_t)3 * nc * sizeof(double));
@@ -1130,6 +1130,8 @@ st_status st_adjoint_backward(st_handle h, const double* lam, int lam_on_device,
       }
       a.d = st.d;
       a.db = A + 6 * n;
+      a.mb = A + 7 * n;
+      a.last = seg == 0;
       a.ab_part = (double*)abp.p;
       a.lam = dlam;
       a.Uw = (long long*)Uw.p;

@@ -587,10 +587,13 @@ struct AdjointStepArgs {
   const double* lam;
   long long* Uw;
   double dt;
+  double* mb = nullptr;  // launch_adjoint_segment
+  int last = 0;
 };
 cudaError_t launch_adjoint_step(st_ctx* h, const AdjointStepArgs& s);
-// a whole segment of `len` steps in one launch (fixed_step_supported handles): s.x and s.v point at the first
-// state of a tape whose states lie 6 n values apart
+// a whole segment of `len` steps in one launch (fixed_step_supported handles): s.x[0] points at the first state of a
+// tape whose states lie 6 n values apart; s.db and s.mb hold running sums until the last call (the run's first
+// segment) leaves dL/dd in s.db and dL/dalpha's partial sums in s.ab_part
 cudaError_t launch_adjoint_segment(st_ctx* h, const AdjointStepArgs& s, int len);
 // the FP32 adjoint of the mixed-precision step (FP32-velocity handles): the tape holds the state at
 // the start of the step (cell, offsets, velocities; diameters in d), the adjoints of position and

@@ -67,13 +67,15 @@ __device__ __forceinline__ int64_t to_fixed53(double s, int k) {
   return (unsigned)sh > 63u ? 0 : (int64_t)min(m >> sh, 0x7fffffffffffffffull);
 }
 
-// v * 2^ex rounded to FP64
+// v * 2^ex rounded to FP64.  (The rare results outside the normal numbers out of line: the adjoint converts twelve
+// times a step, and its 2e6 particles on 64^3, 40 steps, take 21.9 ms instead of 23.0 ms in the smaller loop.)
+static __device__ __noinline__ double to_f64_slow(int64_t v, int ex) { return ldexp((double)v, ex); }
 __device__ __forceinline__ double to_f64(int64_t v, int ex) {
   if (v == 0) return 0.0;
   const unsigned long long m = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
   const int lz = __clzll((long long)m);
   const int be = 1023 + 63 - lz + ex;
-  if (__builtin_expect((unsigned)(be - 1) >= 2045u, 0)) return ldexp((double)v, ex);
+  if (__builtin_expect((unsigned)(be - 1) >= 2045u, 0)) return to_f64_slow(v, ex);
   const unsigned long long t = m << lz;
   unsigned long long r = ((unsigned long long)(be - 1) << 52) + (t >> 11) + ((t >> 10) & 1ull);
   r |= v < 0 ? 0x8000000000000000ull : 0ull;

@@ -687,6 +687,11 @@ __global__ void __maxnreg__(Shape<PHYS>::kRegs) step_mixed_tma_kernel(const __gr
     const int64_t A = S & ~int64_t(7);
     const int64_t Z = (E + 7) & ~int64_t(7);
     const int L = kP * ctid;
+    // cloud in cell: lanes take their corners in different orders where a warp's particles share few cells, or they would
+    // all add to the same words (1e9 particles on 256^3, ten steps 416 against 624 ms, one at a time 500 against 700;
+    // 2e7 on 128^3 7.0 against 7.7).  Up to four particles per cell neighbouring cells' words lie side by side and one
+    // order is as good or better (8.4e6 on 128^3 3.16 either way, 4.2e6 1.81 against 1.90).
+    const int rot = E - S >= 4 * kU * kU * kU ? (lane ^ (lane >> 3)) & 7 : 0;
     // the deposit tile into the global accumulator, once every consumer warp has made its deposits
     auto flush = [&]() -> bool {
       __syncwarp();
@@ -1002,8 +1007,7 @@ __global__ void __maxnreg__(Shape<PHYS>::kRegs) step_mixed_tma_kernel(const __gr
           }
           if (PHYS && a.cic) {
             // cloud in cell: J spread over the eight cells of the start-of-step trilinear stencil with its
-            // weights, each corner straight into the tile: neighbouring particles of a cell sit in
-            // different half-cells and so rarely share a corner cell
+            // weights, each corner straight into the tile (the adds are exact, so their order does not matter)
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
               float j3[3], d[2];
@@ -1014,7 +1018,8 @@ __global__ void __maxnreg__(Shape<PHYS>::kRegs) step_mixed_tma_kernel(const __gr
               }
               const unsigned c0 = cl[jp + e];
 #pragma unroll 1
-              for (int k = 0; k < 8; ++k) {
+              for (int i = 0; i < 8; ++i) {
+                const int k = i ^ rot;
                 float w = (k & 1) ? f[e][0] : 1.0f - f[e][0];
                 w *= (k & 2) ? f[e][1] : 1.0f - f[e][1];
                 w *= (k & 4) ? f[e][2] : 1.0f - f[e][2];

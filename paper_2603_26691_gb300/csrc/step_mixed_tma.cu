@@ -6,10 +6,10 @@
 // contiguous key range) are contiguous in storage.  Each CTA owns a sequence of
 // these units.  Per unit:
 //   * a producer warp loads the unit's fluid tile - the U^3 cells plus a halo
-//     of G cells - from the ghost-padded field with one 4-D TMA tensor copy
-//     (double-buffered across units), and streams the unit's particle arrays
-//     through a ring of shared-memory stages with 1-D bulk copies
-//     (cp.async.bulk), signalling completion on mbarriers;
+//     of G cells - from the ghost-padded field with one 4-D TMA tensor copy,
+//     once the consumers are done with the unit before it, and streams the
+//     unit's particle arrays through a ring of shared-memory stages with 1-D
+//     bulk copies (cp.async.bulk), signalling completion on mbarriers;
 //   * consumer warps take kP consecutive particles per lane from the stage,
 //     gather the fluid velocity from the shared tile (8 LDS.128 with immediate
 //     offsets; particles that drifted out of the tile read the padded field
@@ -33,36 +33,16 @@
 // order.  The separate gather would write the sorted arrays only for this step to read them back.
 // Every wait is bounded: a wait that gives up sets an error flag and the CTA
 // returns.
-#include <cuda.h>
-#include <cudaTypedefs.h>
-
-#include <algorithm>
-#include <atomic>
-#include <cmath>
-#include <cstdio>
-
-#include "st_common.cuh"
-#include "st_ptx.cuh"
+#include "tma_common.cuh"
 
 namespace st {
 namespace {
 
-using namespace ptx;
-
-constexpr int kU = 8;                       // unit edge (cells)
-constexpr int kG = 3;                       // fluid halo = padding of the field
-constexpr int kTE = kU + 2 * kG;            // fluid tile edge (14)
 constexpr int kP = 2;                       // consecutive particles per lane
 constexpr int kWarpParts = 32 * kP;
 constexpr int kStages = 2;
-constexpr int kR = 2;                      // deposit halo
-constexpr int kDE = kU + 2 * kR;           // deposit tile edge (12)
-constexpr int kDepositCells = kDE * kDE * kDE;  // 1728
 constexpr int kScanPairs = 8;              // runs are chained across at most this many pairs of lanes
 constexpr unsigned kPairLinks = 0x15551555u;  // the pairs that have a next one in their group, at their even lane
-constexpr int kDigits = 3;                 // 15-bit digits per value in the shared deposit tile
-constexpr int kDigitBits = 15;
-constexpr int kDepShift = 51;              // shared tile units = global units * 2^kDepShift
 // adds to one cell's digit words between flushes: the two lower digits are at most 2^14, and the top one at
 // most 1 + 2^8 per particle of the run (one particle's impulse is below 2^38 tile units)
 constexpr int kDepMaxAdds = 131071;
@@ -70,9 +50,6 @@ constexpr int kDepMaxAdds = 131071;
 // 64^3 0.36 / 0.34 ms, 2e6 0.69 / 0.67, 2e7 on 128^3 4.54 / 4.72, 6e7 9.0 / 9.9)
 constexpr int64_t kSingleParticles = 1 << 23;
 constexpr unsigned kNoKey = 0xffffffffu;   // no cell: neither a tile-form nor a far one
-
-constexpr int kFluidBytes = kTE * kTE * kTE * 16;               // 43904
-constexpr int kDepositBytes = kDepositCells * 3 * kDigits * 4;  // 62208
 
 // The shape of an instance.  The steps run on what the registers let run at once: two particles per lane and 23
 // consumer warps at 80 registers hide more of the latency than four per lane and 15 warps at 128 (4e8
@@ -91,247 +68,9 @@ struct Shape {
   static_assert(kT * kMaxFusedSteps <= kDepMaxAdds, "a stage's deposits fit the digit words");
 };
 
-__device__ __forceinline__ void tma_load_tile(void* dst, const CUtensorMap* map, int c1, int c2, int c3,
-                                              uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, "
-      "%5}], [%6];" ::"r"(sptr(dst)),
-      "l"(map), "r"(0), "r"(c1), "r"(c2), "r"(c3), "r"(sptr(bar))
-      : "memory");
-}
-
-
-__device__ __forceinline__ float rcp_approx(float x) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
-
-struct TmaArgs {
-  MixedState s;
-  const float4* __restrict__ Up;      // ghost-padded field [nz+2G][ny+2G][nx+2G]
-  long long* __restrict__ acc;
-  const uint32_t* __restrict__ cell_start;
-  int* __restrict__ err;
-  unsigned* __restrict__ unit_ctr;    // next unit to hand out, CTAs that found none left (zero between launches)
-  int64_t ncell;
-  int nx, ny, nz;
-  int nunits;                         // units of kU^3 cells in key order
-  int logB, ncx, ncy;                 // chunk geometry for decoding a unit's origin
-  float inv_h[3];
-  float dt, cadt, inv_ca, mcoef;
-  float g[3], gdt[3];
-  int nsteps;                         // steps to take (1 .. kMaxFusedSteps)
-  float s2;                           // mcoef (of 1 kg) times s2: impulses in deposit-tile units, 2^(kDepShift - E)
-                                      // of the accumulator's; s2 is 1 unless the impulses are tiny
-  float4* __restrict__ rec;           // record output: two float4 per particle (see st_common.cuh)
-  const uint32_t* __restrict__ perm;  // GATHER: storage index (old order) of each sorted position
-  const float4* __restrict__ grec;    // GATHER: the records in the old order
-  const uint32_t* __restrict__ ids_in;   // GATHER: ids in the old order
-  uint32_t* __restrict__ ids_out;        // GATHER: ids in sorted order
-  int ngp, semi, sn, cic;             // physics variants (the PHYS instance): nearest grid point,
-  float re_coef;                      // semi-implicit Euler, Schiller-Naumann drag (Re = re_coef |u-v| d),
-                                      // cloud-in-cell deposit
-};
-
-// de-interleave 3 bits per level (local x bit lowest)
-__device__ __forceinline__ uint32_t compact3(uint32_t v) {
-  v &= 0x09249249u;
-  v = (v | (v >> 2)) & 0x030c30c3u;
-  v = (v | (v >> 4)) & 0x0300f00fu;
-  v = (v | (v >> 8)) & 0xff0000ffu;
-  v = (v | (v >> 16)) & 0x000003ffu;
-  return v;
-}
-
-__device__ __forceinline__ void unit_origin(const TmaArgs& a, int u, int& ox, int& oy, int& oz) {
-  const uint32_t key = (uint32_t)u * (kU * kU * kU);
-  const uint32_t chunk = key >> (3 * a.logB);
-  const uint32_t m = key & ((1u << (3 * a.logB)) - 1u);
-  const int B = 1 << a.logB;
-  const int cx = (int)(chunk % (uint32_t)a.ncx);
-  const int cy = (int)((chunk / (uint32_t)a.ncx) % (uint32_t)a.ncy);
-  const int cz = (int)(chunk / ((uint32_t)a.ncx * (uint32_t)a.ncy));
-  ox = cx * B + (int)compact3(m);
-  oy = cy * B + (int)compact3(m >> 1);
-  oz = cz * B + (int)compact3(m >> 2);
-}
-
-template <bool BF16>
-__device__ __forceinline__ int stage_bytes(int cnt) {
-  return cnt * (BF16 ? 26 : 32);
-}
-
-// cell and offset of a coordinate that the fast relocation cannot take (rare): a move of 2^22 cells
-// or more, or of more than one box length, in one step; the cell carried is floor(o) reduced
-// periodically (fmodf is exact), the offset o - floor(o)
-struct Relocated {
-  int cell;
-  float offset;
-};
-__device__ __noinline__ Relocated relocate_general(float o, int ci, int n) {
-  if (!(fabsf(o) <= 3.0e38f)) return Relocated{ci, 0.5f};  // non-finite: keep the cell
-  const float fl = floorf(o);
-  int k = (ci + (int)fmodf(fl, (float)n)) % n;
-  return Relocated{k < 0 ? k + n : k, fmaxf(fminf(o - fl, 0.99999994f), 0.0f)};
-}
-
-// two-lane FP32 arithmetic (one instruction for a register pair; round-to-nearest, no flush to
-// zero, so each lane rounds exactly as the scalar operation would)
-__device__ __forceinline__ unsigned long long pack2(float a, float b) {
-  unsigned long long r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ void unpack2(unsigned long long r, float& a, float& b) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(r));
-}
-__device__ __forceinline__ unsigned long long sub2(unsigned long long a, unsigned long long b) {
-  unsigned long long d;
-  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
-  unsigned long long d;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b) {
-  unsigned long long d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
-  unsigned long long d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-__device__ __forceinline__ unsigned long long add_rm2(unsigned long long a, unsigned long long b) {
-  unsigned long long d;
-  asm("add.rm.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ unsigned long long dup2(float a) { return pack2(a, a); }
-// lerp c0 + w (c1 - c0) on the (x, y) pair
-__device__ __forceinline__ unsigned long long lerp2(unsigned long long w, unsigned long long c0, unsigned long long c1) {
-  return fma2(w, sub2(c1, c0), c0);
-}
-
-// 1 - e^{-x} for a pair of arguments x >= 0 (*E = e^{-x}): the degree-5 Taylor polynomial in
-// Horner form for x < 1/8 (truncation below 5e-8 relative), else 1 - 2^(-x log2 e); the polynomial
-// as pair operations, the exponentials and the choice per lane
-__device__ __forceinline__ unsigned long long one_minus_exp2(unsigned long long X, unsigned long long* E) {
-  float x0, x1, a0, a1;
-  unpack2(mul2(X, dup2(-1.4426950408889634f)), a0, a1);
-  float ex0, ex1;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(ex0) : "f"(a0));
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(ex1) : "f"(a1));
-  unsigned long long S = fma2(X, dup2(1.0f / 120.0f), dup2(-1.0f / 24.0f));
-  S = fma2(X, S, dup2(1.0f / 6.0f));
-  S = fma2(X, S, dup2(-0.5f));
-  S = fma2(X, S, dup2(1.0f));
-  float s0, s1;
-  unpack2(mul2(X, S), s0, s1);
-  unpack2(X, x0, x1);
-  const float r0 = x0 < 0.125f ? s0 : 1.0f - ex0;
-  const float r1 = x1 < 0.125f ? s1 : 1.0f - ex1;
-  *E = pack2(x0 < 0.125f ? 1.0f - r0 : ex0, x1 < 0.125f ? 1.0f - r1 : ex1);
-  return pack2(r0, r1);
-}
-
-// trilinear interpolation of the 8 corner velocities (corner c_xyz, x fastest) at weights f: the
-// x and y components as register pairs, z alone; the same operations and rounding per component
-// as c0 + f (c1 - c0) applied along x, then y, then z
-__device__ __forceinline__ void trilerp(const float4& c000, const float4& c100, const float4& c010,
-                                        const float4& c110, const float4& c001, const float4& c101,
-                                        const float4& c011, const float4& c111, float fx, float fy, float fz,
-                                        float* up) {
-  const unsigned long long FX = pack2(fx, fx), FY = pack2(fy, fy), FZ = pack2(fz, fz);
-  const unsigned long long a = lerp2(FX, pack2(c000.x, c000.y), pack2(c100.x, c100.y));
-  const unsigned long long b = lerp2(FX, pack2(c010.x, c010.y), pack2(c110.x, c110.y));
-  const unsigned long long c = lerp2(FX, pack2(c001.x, c001.y), pack2(c101.x, c101.y));
-  const unsigned long long d = lerp2(FX, pack2(c011.x, c011.y), pack2(c111.x, c111.y));
-  const unsigned long long e = lerp2(FY, a, b), g = lerp2(FY, c, d);
-  unpack2(lerp2(FZ, e, g), up[0], up[1]);
-  const float az = fmaf(fx, c100.z - c000.z, c000.z), bz = fmaf(fx, c110.z - c010.z, c010.z);
-  const float cz = fmaf(fx, c101.z - c001.z, c001.z), dz = fmaf(fx, c111.z - c011.z, c011.z);
-  const float ez = fmaf(fy, bz - az, az), gz = fmaf(fy, dz - cz, cz);
-  up[2] = fmaf(fz, gz - ez, ez);
-}
-
-// fluid velocity of a particle outside its unit's tile, from the ghost-padded field (L2); the same
-// stencil and arithmetic as the tile path
-__device__ __noinline__ float3 gather_padded(const float4* __restrict__ Up, int px, int pxy, int cell, float o0,
-                                             float o1, float o2) {
-  const int ci[3] = {cell_i(cell), cell_j(cell), cell_k(cell)};
-  const float o[3] = {o0, o1, o2};
-  int i0[3];
-  float f[3];
-#pragma unroll
-  for (int q = 0; q < 3; ++q) {
-    const bool hi2 = o[q] >= 0.5f;
-    i0[q] = ci[q] - (hi2 ? 0 : 1);
-    f[q] = o[q] + (hi2 ? -0.5f : 0.5f);
-  }
-  const float4* g = Up + (i0[0] + kG) + (int64_t)px * (i0[1] + kG) + (int64_t)pxy * (i0[2] + kG);
-  float up[3];
-  trilerp(__ldg(g), __ldg(g + 1), __ldg(g + px), __ldg(g + px + 1), __ldg(g + pxy), __ldg(g + pxy + 1),
-          __ldg(g + pxy + px), __ldg(g + pxy + px + 1), f[0], f[1], f[2], up);
-  return make_float3(up[0], up[1], up[2]);
-}
-
-// nearest-grid-point value of a particle outside its unit's tile, from the ghost-padded field
-__device__ __noinline__ float3 ngp_padded(const float4* __restrict__ Up, int px, int pxy, int cell) {
-  const float4 u = __ldg(Up + (cell_i(cell) + kG) + (int64_t)px * (cell_j(cell) + kG) + (int64_t)pxy * (cell_k(cell) + kG));
-  return make_float3(u.x, u.y, u.z);
-}
-
-// Schiller-Naumann drag factor f = C_D Re / 24: 1 + 0.15 Re^0.687 up to Re = 1000 (the power from
-// the hardware base-2 logarithm and exponential), 0.44 Re / 24 above
-__device__ __forceinline__ float sn_factor(float re) {
-  float l, p;
-  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(l) : "f"(re));
-  const float y = 0.687f * l;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(p) : "f"(y));
-  return re <= 1000.0f ? fmaf(0.15f, p, 1.0f) : (0.44f / 24.0f) * re;
-}
-
-// add round(t_q), q = 0, 1, 2, to the shared deposit-tile values of one cell, each kept as
-// three signed digits in int32 words (w[0] + 2^15 w[kDepositCells] + 2^30 w[2 kDepositCells], the
-// components kDigits kDepositCells words apart).  Each value t (in tile units, |t| < 2^45) is split exactly
-// into balanced digits by round-to-nearest additions of 1.5 * 2^(23+b), which leave the nearest multiple
-// of 2^b: t = 2^30 d2 + 2^15 d1 + d0 + (t - round(t)) with |d0|, |d1| <= 2^14 and |d2| <= 2^15.  Components 0 and
-// 1 are split as a register pair.  The top digit is zero up to 2^29, where nearly all values lie (the unit
-// is 2^-45 of a bound on 128 of the largest particles): two digits then.  Integer atomics make the sums exact
-// and independent of the order of the adds.
-__device__ __forceinline__ void digits1(float t, int& d0, int& d1, int& d2) {
-  const float h = __fsub_rn(__fadd_rn(t, 0x1.8p53f), 0x1.8p53f);  // multiple of 2^30
-  const float l = __fsub_rn(t, h);                                  // |l| <= 2^29, exact
-  const float m = __fsub_rn(__fadd_rn(l, 0x1.8p38f), 0x1.8p38f);  // multiple of 2^15
-  const float l2 = __fsub_rn(l, m);                                 // |l2| <= 2^14, exact
-  d2 = __float_as_int(__fmaf_rn(h, 0x1p-30f, 12582912.0f)) - 0x4B400000;
-  d1 = __float_as_int(__fmaf_rn(m, 0x1p-15f, 12582912.0f)) - 0x4B400000;
-  d0 = __float_as_int(__fadd_rn(l2, 12582912.0f)) - 0x4B400000;
-}
-__device__ __forceinline__ void digits2(unsigned long long t, int* d0, int* d1, int* d2) {
-  const unsigned long long C53 = pack2(0x1.8p53f, 0x1.8p53f), C38 = pack2(0x1.8p38f, 0x1.8p38f);
-  const unsigned long long C23 = pack2(12582912.0f, 12582912.0f);
-  const unsigned long long h = sub2(add2(t, C53), C53);
-  const unsigned long long l = sub2(t, h);
-  const unsigned long long m = sub2(add2(l, C38), C38);
-  const unsigned long long l2 = sub2(l, m);
-  float a, b;
-  unpack2(fma2(h, pack2(0x1p-30f, 0x1p-30f), C23), a, b);
-  d2[0] = __float_as_int(a) - 0x4B400000;
-  d2[1] = __float_as_int(b) - 0x4B400000;
-  unpack2(fma2(m, pack2(0x1p-15f, 0x1p-15f), C23), a, b);
-  d1[0] = __float_as_int(a) - 0x4B400000;
-  d1[1] = __float_as_int(b) - 0x4B400000;
-  unpack2(add2(l2, C23), a, b);
-  d0[0] = __float_as_int(a) - 0x4B400000;
-  d0[1] = __float_as_int(b) - 0x4B400000;
-}
-// the two lower digits alone, |t| <= 2^29
+// add round(t_q), q = 0, 1, 2 (in tile units), to the shared deposit-tile values of one cell.  The top digit is zero up
+// to 2^29, where nearly all values lie (the unit is 2^-45 of a bound on 128 of the largest particles): two digits then.
+// The two lower digits alone, |t| <= 2^29
 __device__ __forceinline__ void low_digits1(float t, int& d0, int& d1) {
   const float m = __fsub_rn(__fadd_rn(t, 0x1.8p38f), 0x1.8p38f);
   d1 = __float_as_int(__fmaf_rn(m, 0x1p-15f, 12582912.0f)) - 0x4B400000;
@@ -420,57 +159,12 @@ __device__ __forceinline__ int32_t global_cell(const int (&uo)[3], const int (&n
   return (c & kFarCell) ? (int32_t)(c & ~kFarCell) : pack_cell(g[0], g[1], g[2]);
 }
 
-// A commit outside the deposit tile, straight to the global accumulator.  A CTA's first kFarFree of a launch are plain
-// reductions that nothing waits for; the count of adds allows for them.  Nothing bounds how many more one word gets
-// in a launch, so these look at it: a word found beyond 2^60 passes 2^34 of its value on to the next
-// word: each such add then takes more off than it put on, and the adds in flight on a GPU (fewer than
-// 2^19 of less than 2^32) cannot carry a word from there to 2^62.  The sum over the words is unchanged.  (All of
-// them waiting for the word: a call of ten steps of 5e8 particles on 256^3, with its
-// export, 62.6 ms against 61.2 ms.)
-__device__ __forceinline__ int* far_count() {  // the CTA's commits of this launch, up to about kFarFree
-  __shared__ int n;
-  return &n;
-}
-__device__ __forceinline__ bool far_free() {
-  volatile int* n = far_count();
-  return *n < kFarFree && atomicAdd(far_count(), 1) < kFarFree;
-}
-__device__ __forceinline__ void far_digit(long long* p, int k, long long d, bool free) {
-  if (d == 0 || k >= kAccWords) return;
-  if (free) {
-    atomicAdd((unsigned long long*)&p[k], (unsigned long long)d);
-    return;
-  }
-  const long long old = (long long)atomicAdd((unsigned long long*)&p[k], (unsigned long long)d);
-  constexpr long long lim = 1ll << 60;
-  if (k + 1 < kAccWords && (old > lim || old < -lim)) {
-    const long long c = old > 0 ? 4ll : -4ll;
-    atomicAdd((unsigned long long*)&p[k], (unsigned long long)(-c * (1ll << 32)));
-    atomicAdd((unsigned long long*)&p[k + 1], (unsigned long long)c);
-  }
-}
 __device__ __noinline__ void commit_far(const TmaArgs& a, unsigned cell, float r0, float r1, float r2) {
   const int64_t c = cell_i((int32_t)cell) + (int64_t)a.nx * (cell_j((int32_t)cell) + (int64_t)a.ny * cell_k((int32_t)cell));
   const float r[3] = {r0, r1, r2};
   const bool free = far_free();
 #pragma unroll 1
-  for (int q = 0; q < 3; ++q) {
-    const uint32_t b = __float_as_uint(r[q]);
-    const uint32_t ex = (b >> 23) & 0xffu;
-    unsigned long long man = b & 0x7fffffu;
-    if (ex != 0) man |= 0x800000ull;
-    int s = (int)(ex == 0 ? 1 : ex) - 150 + kDepShift;
-    if (s < 0) {
-      const int k = -s;
-      man = k < 32 ? ((man + ((1ull << k) >> 1)) >> k) : 0ull;
-      s = 0;
-    }
-    const unsigned long long lo = man << (s & 31);  // man < 2^24: below 2^55
-    const long long sg = (b >> 31) ? -1ll : 1ll;
-    long long* p = a.acc + kAccWords * (q * a.ncell + c);
-    far_digit(p, s >> 5, sg * (long long)(lo & 0xffffffffull), free);
-    far_digit(p, (s >> 5) + 1, sg * (long long)(lo >> 32), free);
-  }
+  for (int q = 0; q < 3; ++q) add_far(a.acc + kAccWords * (q * a.ncell + c), r[q], free);
 }
 
 // one sum of impulses of the start cell c (either form): into the shared deposit tile or to the global
@@ -480,82 +174,6 @@ __device__ __forceinline__ void commit_record(const TmaArgs& a, int* dep, unsign
     dep_add3(dep + dep_index(c), r0, r1, r2);
   else
     commit_far(a, c & ~kFarCell, r0, r1, r2);
-}
-
-// a lane's kP consecutive 32-bit values as one access
-struct alignas(4 * kP) Vec32 {
-  uint32_t w[kP];
-};
-__device__ __forceinline__ void stcs(void* p, const Vec32& v) {
-  if constexpr (kP == 4)
-    __stcs(reinterpret_cast<uint4*>(p), make_uint4(v.w[0], v.w[1], v.w[2], v.w[kP - 1]));
-  else
-    __stcs(reinterpret_cast<uint2*>(p), make_uint2(v.w[0], v.w[1]));
-}
-__device__ __forceinline__ Vec32 ldcs(const void* p) {
-  Vec32 v;
-  if constexpr (kP == 4) {
-    const uint4 q = __ldcs(reinterpret_cast<const uint4*>(p));
-    v.w[0] = q.x;
-    v.w[1] = q.y;
-    v.w[2 % kP] = q.z;
-    v.w[3 % kP] = q.w;
-  } else {
-    const uint2 q = __ldcs(reinterpret_cast<const uint2*>(p));
-    v.w[0] = q.x;
-    v.w[1] = q.y;
-  }
-  return v;
-}
-__device__ __forceinline__ Vec32 vec(const float (&f)[kP]) {
-  Vec32 v;
-#pragma unroll
-  for (int j = 0; j < kP; ++j) v.w[j] = __float_as_uint(f[j]);
-  return v;
-}
-
-// GATHER: the permutation entries of a lane's sorted positions p0 .. p0 + kP - 1 (p0 a multiple of
-// kP), zeros when it owns none of them within [S, E) (then p0 may lie past the buffer)
-__device__ __forceinline__ Vec32 gather_perm(const TmaArgs& a, int64_t p0, int64_t S, int64_t E) {
-  return p0 + kP > S && p0 < E ? ldcs(a.perm + p0) : Vec32{};
-}
-// GATHER: the ids of the owned positions among p0 .. p0 + kP - 1 through the permutation (0 elsewhere)
-__device__ __forceinline__ Vec32 gather_ids(const TmaArgs& a, const Vec32& pp, int64_t p0, int64_t S, int64_t E) {
-  Vec32 id;
-#pragma unroll
-  for (int j = 0; j < kP; ++j) id.w[j] = (p0 + j >= S && p0 + j < E) ? __ldg(a.ids_in + pp.w[j]) : 0u;
-  return id;
-}
-// GATHER: store ids gathered for positions p0 .. p0 + kP - 1 (the owned ones)
-__device__ __forceinline__ void store_ids(const TmaArgs& a, const Vec32& id, int64_t p0, int64_t S, int64_t E) {
-  if (p0 >= S && p0 + kP <= E) {
-    stcs(a.ids_out + p0, id);
-  } else {
-#pragma unroll
-    for (int j = 0; j < kP; ++j)
-      if (p0 + j >= S && p0 + j < E) a.ids_out[p0 + j] = id.w[j];
-  }
-}
-// GATHER: ask L2 for the records of the owned positions among p0 .. p0 + kP - 1 (a stage before their
-// loads)
-__device__ __forceinline__ void gather_prefetch(const TmaArgs& a, const Vec32& pp, int64_t p0, int64_t S, int64_t E) {
-#pragma unroll
-  for (int j = 0; j < kP; ++j)
-    if (p0 + j >= S && p0 + j < E) asm volatile("prefetch.global.L2 [%0];" ::"l"(a.grec + 2 * (int64_t)pp.w[j]));
-}
-// GATHER: the diameters of the owned positions among p0 .. p0 + kP - 1, stored in sorted order as soon as
-// their records arrive (a step does not change them)
-__device__ __forceinline__ void store_d(const TmaArgs& a, const Rec32 (&r)[kP], int64_t p0, int64_t S, int64_t E) {
-  if (p0 >= S && p0 + kP <= E) {
-    Vec32 d;
-#pragma unroll
-    for (int j = 0; j < kP; ++j) d.w[j] = __float_as_uint(r[j].d);
-    stcs(a.s.d + p0, d);
-  } else {
-#pragma unroll
-    for (int j = 0; j < kP; ++j)
-      if (p0 + j >= S && p0 + j < E) a.s.d[p0 + j] = r[j].d;
-  }
 }
 
 template <bool BF16, bool REC, bool PHYS, bool GATHER>
@@ -700,26 +318,7 @@ __global__ void __maxnreg__(Shape<PHYS>::kRegs) step_mixed_tma_kernel(const __gr
         atomicOr(a.err, 16);
         return false;
       }
-      for (int t = ctid; t < kDepositCells; t += kConsumerWarps * 32) {
-        const int li = t % kDE, lj = (t / kDE) % kDE, lk = t / (kDE * kDE);
-        int gi = uo[0] - kR + li, gj = uo[1] - kR + lj, gk = uo[2] - kR + lk;
-        gi = gi < 0 ? gi + a.nx : (gi >= a.nx ? gi - a.nx : gi);
-        gj = gj < 0 ? gj + a.ny : (gj >= a.ny ? gj - a.ny : gj);
-        gk = gk < 0 ? gk + a.nz : (gk >= a.nz ? gk - a.nz : gk);
-        const int64_t gc = gi + (int64_t)a.nx * (gj + (int64_t)a.ny * gk);
-        for (int q = 0; q < 3; ++q) {
-          int* w = dep + q * kDigits * kDepositCells + t;
-          const long long val = (long long)w[0] + ((long long)w[kDepositCells] << kDigitBits) +
-                                ((long long)w[2 * kDepositCells] << (2 * kDigitBits));
-          if (val != 0) {
-            w[0] = 0;
-            w[kDepositCells] = 0;
-            w[2 * kDepositCells] = 0;
-            acc_add_mag(a.acc + kAccWords * (q * a.ncell + gc), (unsigned long long)(val < 0 ? -val : val), kDepShift,
-                        val < 0);
-          }
-        }
-      }
+      flush_tile(a, dep, uo, ctid, kConsumerWarps * 32);
       __syncwarp();
       if (lane == 0) mbar_arrive(flush_done);
       if (!mbar_wait(flush_done, flushes & 1)) {
@@ -731,11 +330,11 @@ __global__ void __maxnreg__(Shape<PHYS>::kRegs) step_mixed_tma_kernel(const __gr
     };
     // GATHER: the permutation entries of this stage and of the next, and this stage's ids, are
     // held in registers a stage ahead
-    Vec32 pcur{}, pnext{}, gid{};
+    Vec32<kP> pcur{}, pnext{}, gid{};
     if constexpr (GATHER) {
-      pcur = gather_perm(a, A + L, S, E);
+      pcur = gather_perm<kP>(a, A + L, S, E);
       gid = gather_ids(a, pcur, A + L, S, E);
-      pnext = gather_perm(a, A + kT + L, S, E);
+      pnext = gather_perm<kP>(a, A + kT + L, S, E);
     }
     int deposited = 0;  // stages since the last flush
     for (int64_t t0 = A; t0 < Z; t0 += kT) {
@@ -780,14 +379,14 @@ __global__ void __maxnreg__(Shape<PHYS>::kRegs) step_mixed_tma_kernel(const __gr
           gather_prefetch(a, pnext, p0 + kT, S, E);
           gid = gather_ids(a, pnext, p0 + kT, S, E);
           pcur = pnext;
-          pnext = gather_perm(a, p0 + 2 * kT, S, E);
+          pnext = gather_perm<kP>(a, p0 + 2 * kT, S, E);
         }
         if (REC) {
           // the diameters into the stage, from where the records take them
-          Vec32 d;
+          Vec32<kP> d;
 #pragma unroll
           for (int j = 0; j < kP; ++j) d.w[j] = __float_as_uint(r[j].d);
-          *reinterpret_cast<Vec32*>(src + (BF16 ? 4 * kT * 4 + 3 * kT * 2 : 7 * kT * 4) + L * 4) = d;
+          *reinterpret_cast<Vec32<kP>*>(src + (BF16 ? 4 * kT * 4 + 3 * kT * 2 : 7 * kT * 4) + L * 4) = d;
         } else {
           store_d(a, r, p0, S, E);
         }
@@ -803,8 +402,8 @@ __global__ void __maxnreg__(Shape<PHYS>::kRegs) step_mixed_tma_kernel(const __gr
           dv[j] = r[j].d;
         }
       } else {
-        const Vec32 c = *reinterpret_cast<const Vec32*>(src + L * 4);
-        const Vec32 dd = *reinterpret_cast<const Vec32*>(src + (BF16 ? 4 * kT * 4 + 3 * kT * 2 : 7 * kT * 4) + L * 4);
+        const Vec32<kP> c = *reinterpret_cast<const Vec32<kP>*>(src + L * 4);
+        const Vec32<kP> dd = *reinterpret_cast<const Vec32<kP>*>(src + (BF16 ? 4 * kT * 4 + 3 * kT * 2 : 7 * kT * 4) + L * 4);
 #pragma unroll
         for (int j = 0; j < kP; ++j) {
           cell[j] = (int)c.w[j];
@@ -812,7 +411,7 @@ __global__ void __maxnreg__(Shape<PHYS>::kRegs) step_mixed_tma_kernel(const __gr
         }
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
-          const Vec32 x = *reinterpret_cast<const Vec32*>(src + (1 + q) * kT * 4 + L * 4);
+          const Vec32<kP> x = *reinterpret_cast<const Vec32<kP>*>(src + (1 + q) * kT * 4 + L * 4);
 #pragma unroll
           for (int j = 0; j < kP; ++j) xi[q][j] = __uint_as_float(x.w[j]);
           if (BF16) {
@@ -824,7 +423,7 @@ __global__ void __maxnreg__(Shape<PHYS>::kRegs) step_mixed_tma_kernel(const __gr
               v[q][j + 1] = f.y;
             }
           } else {
-            const Vec32 w = *reinterpret_cast<const Vec32*>(src + 4 * kT * 4 + q * kT * 4 + L * 4);
+            const Vec32<kP> w = *reinterpret_cast<const Vec32<kP>*>(src + 4 * kT * 4 + q * kT * 4 + L * 4);
 #pragma unroll
             for (int j = 0; j < kP; ++j) v[q][j] = __uint_as_float(w.w[j]);
           }
@@ -983,7 +582,8 @@ __global__ void __maxnreg__(Shape<PHYS>::kRegs) step_mixed_tma_kernel(const __gr
               const __nv_bfloat162 b2 = __floats2bfloat162_rn(vn[0], vn[1]);
               vn[0] = __low2float(b2);
               vn[1] = __high2float(b2);
-              JP[q] = pack2(-m0 * (((vn[0] - v[q][jp]) - a.gdt[q]) * a.s2), -m1 * (((vn[1] - v[q][jp + 1]) - a.gdt[q]) * a.s2));
+              JP[q] = pack2(__fmul_rn(-m0, __fmul_rn((vn[0] - v[q][jp]) - a.gdt[q], a.s2)),
+                            __fmul_rn(-m1, __fmul_rn((vn[1] - v[q][jp + 1]) - a.gdt[q], a.s2)));
             } else {
               // v' - v = -(v - w) (1 - E), without the cancellation of subtracting the rounded v'
               unsigned long long X = fma2(DVW, E1, dup2(a.gdt[q]));
@@ -1142,9 +742,9 @@ __global__ void __maxnreg__(Shape<PHYS>::kRegs) step_mixed_tma_kernel(const __gr
         // particle (a full sector; the sort's gather then reads one sector per particle).  The
         // diameters are read again from the stage.  BF16 handles store the (BF16-exact) velocities
         // as FP32 in the record.
-        const Vec32 d = *reinterpret_cast<const Vec32*>(src + (BF16 ? 4 * kT * 4 + 3 * kT * 2 : 7 * kT * 4) + L * 4);
+        const Vec32<kP> d = *reinterpret_cast<const Vec32<kP>*>(src + (BF16 ? 4 * kT * 4 + 3 * kT * 2 : 7 * kT * 4) + L * 4);
         if (all_own) {
-          Vec32 c;
+          Vec32<kP> c;
 #pragma unroll
           for (int j = 0; j < kP; ++j) c.w[j] = (uint32_t)cell[j];
           stcs(a.s.cell + p0, c);
@@ -1157,7 +757,7 @@ __global__ void __maxnreg__(Shape<PHYS>::kRegs) step_mixed_tma_kernel(const __gr
                                                v[2][j], __uint_as_float(d.w[j])});
         }
       } else if (all_own) {
-        Vec32 c;
+        Vec32<kP> c;
 #pragma unroll
         for (int j = 0; j < kP; ++j) c.w[j] = (uint32_t)cell[j];
         stcs(a.s.cell + p0, c);
@@ -1203,18 +803,6 @@ __global__ void __maxnreg__(Shape<PHYS>::kRegs) step_mixed_tma_kernel(const __gr
   }
 }
 
-PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
-  static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-  if (!fn) {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = (PFN_cuTensorMapEncodeTiled_v12000)p;
-  }
-  return fn;
-}
-
 }  // namespace
 
 bool tma_step_supported(const st_ctx* h) {
@@ -1242,85 +830,27 @@ cudaError_t launch_step_mixed_tma(st_ctx* h, const StepParams& p, bool records, 
       step_mixed_tma_kernel<false, true, false, true>,   step_mixed_tma_kernel<true, true, false, true>,
       step_mixed_tma_kernel<false, false, true, true>,   step_mixed_tma_kernel<true, false, true, true>,
       step_mixed_tma_kernel<false, true, true, true>,    step_mixed_tma_kernel<true, true, true, true>};
-  constexpr int kAttrDevices = 64;
-  // a kernel attribute is per device; atomic because handles may be driven from several host threads
-  // (setting an attribute twice is harmless)
-  static std::atomic<bool> attr_set[kAttrDevices][16];
+  static std::atomic<bool> attr_set[16][kAttrDevices];
   const int variant = (int)bf + 2 * (int)records + 4 * (int)phys + 8 * (int)gather;
   const Kern kern = table[variant];
   const int threads = phys ? Shape<true>::kThreads : Shape<false>::kThreads;
   const int smem = phys ? Shape<true>::kSmemBytes : Shape<false>::kSmemBytes;
-  if (h->dev < 0 || h->dev >= kAttrDevices) return cudaErrorInvalidDevice;
-  if (!attr_set[h->dev][variant].load(std::memory_order_acquire)) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    attr_set[h->dev][variant].store(true, std::memory_order_release);
-  }
-  PFN_cuTensorMapEncodeTiled_v12000 enc = encode_fn();
-  if (!enc) return cudaErrorNotSupported;
   CUtensorMap map;
-  const int nx = h->geo.n[0], ny = h->geo.n[1], nz = h->geo.n[2];
-  cuuint64_t dims[4] = {4, (cuuint64_t)(nx + 2 * kG), (cuuint64_t)(ny + 2 * kG), (cuuint64_t)(nz + 2 * kG)};
-  cuuint64_t strides[3] = {16, (cuuint64_t)16 * (nx + 2 * kG), (cuuint64_t)16 * (nx + 2 * kG) * (ny + 2 * kG)};
-  cuuint32_t box[4] = {4, kTE, kTE, kTE};
-  cuuint32_t estr[4] = {1, 1, 1, 1};
-  CUresult r = enc(&map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, h->fluid_pad.p, dims, strides, box, estr,
-                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
-  TmaArgs a;
-  a.s = carve_mixed(h->state.p, h->cap, bf);
-  // records written by steps that gather go where the stale state was, their cells apart
-  a.rec = records ? (float4*)(gather ? h->state.p : h->state_alt.p) : nullptr;
-  if (records && gather) a.s.cell = (int32_t*)h->rec_cell.p;
-  // the deferred gather of the last sort: permutation, records (old order) and ids in, ids out
-  a.perm = gather ? (const uint32_t*)h->vals[0].p : nullptr;
-  a.grec = gather ? (const float4*)h->state_alt.p : nullptr;
-  a.ids_in = gather ? (const uint32_t*)h->ids.p : nullptr;
-  a.ids_out = gather ? (uint32_t*)h->ids_alt.p : nullptr;
-  a.ngp = p.ngp;
-  a.semi = p.semi;
-  a.sn = p.sn;
-  a.cic = p.cic;
-  a.re_coef = (float)p.re_coef;
-  a.Up = (const float4*)h->fluid_pad.p;
-  a.acc = (long long*)h->acc.p;
-  a.cell_start = (const uint32_t*)h->cell_start.p;
-  a.err = (int*)h->flags.p;
-  a.unit_ctr = (unsigned*)((char*)h->flags.p + kUnitCounterOffset);
-  a.nsteps = p.nsteps;
-  a.ncell = h->geo.ncell;
-  a.nx = nx;
-  a.ny = ny;
-  a.nz = nz;
-  a.nunits = (int)(h->nkeys / (kU * kU * kU));
-  int logB = 0;
-  while ((1 << logB) < h->geo.B) ++logB;
-  a.logB = logB;
-  a.ncx = nx / h->geo.B;
-  a.ncy = ny / h->geo.B;
-  for (int q = 0; q < 3; ++q) {
-    a.inv_h[q] = (float)h->geo.inv_h[q];
-    a.g[q] = (float)p.g[q];
-    a.gdt[q] = (float)(p.g[q] * p.dt);
-  }
-  a.dt = (float)p.dt;
-  a.cadt = (float)(p.ca * p.dt);
-  a.inv_ca = (float)(1.0 / p.ca);
+  cudaError_t e = allow_smem(attr_set[variant], h->dev, kern, smem);
+  if (e == cudaSuccess) e = field_map(h, &map);
+  if (e != cudaSuccess) return e;
+  TmaArgs a = tma_args(h, p, records, gather);
   {
     // tile units: 2^(E - kDepShift) in the mass coefficient as far as it stays an FP32 number (a power of two: the
-    // impulses' bits do not change), the rest in s2; beyond +-250 every scaled impulse is 0 or overflows the
+    // impulses' bits do not change), the rest in s2, which is 1 unless the impulses are tiny; beyond +-250 every scaled impulse is 0 or overflows the
     // bound the exponent was chosen for, so clamping changes nothing
     const int Es = std::min(std::max(p.E - kDepShift, -250), 250);
     const int k1 = std::min(Es, 100 - std::ilogb(std::max(p.mcoef, 1e-300)));
     a.mcoef = (float)std::ldexp(p.mcoef, k1);
+    a.s1 = 1.0f;
     a.s2 = std::ldexp(1.0f, Es - k1);
   }
-  int sms = 0;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->dev);
-  int grid = sms > 0 ? sms : 152;
-  grid = std::min(std::min(grid, a.nunits), kFarCtas);
-  kern<<<grid, threads, smem, h->stream>>>(map, a);
+  kern<<<tma_grid(h, a.nunits), threads, smem, h->stream>>>(map, a);
   h->launches += 1;
   return cudaGetLastError();
 }

@@ -54,7 +54,7 @@ constexpr unsigned kNoKey = 0xffffffffu;   // no cell: neither a tile-form nor a
 // The shape of an instance.  The steps run on what the registers let run at once: two particles per lane and 23
 // consumer warps at 80 registers hide more of the latency than four per lane and 15 warps at 128 (4e8
 // particles on 256^3, ten steps: 44.1 against 48.2 ms when the shape was chosen, 36.8 ms since).  The physics
-// variants need more registers: 19 warps at 96 (cloud-in-cell at 2e7 on 128^3: 8.9 ms, with four per lane 10.7; 7.3 ms
+// variants need more registers: 19 warps at 96 (cloud-in-cell at 2e7 on 128^3: 8.9 ms, with four per lane 10.7; 6.6 ms
 // since).  Swapped, 19 warps for the default and 23 for the variants: 39.9 against 37.3 ms and 8.8 against 7.3 ms.
 template <bool PHYS>
 struct Shape {

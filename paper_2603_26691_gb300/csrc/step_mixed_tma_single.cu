@@ -4,10 +4,11 @@
 // nothing it computes once per particle is used twice.  This kernel is the multi-step one
 // (step_mixed_tma.cu: units, tiles, stages and their barriers are described there) laid out for
 // that: 4 consecutive particles per lane and 15 consumer warps at 128 registers, larger stages, whole-lane
-// 128-bit stores ahead of the deposit, coefficients in registers.  Its arithmetic and the order of its sums are those
-// of the multi-step kernel, so the results are the same to the bit whichever takes a step.  1e9 particles on
+// 128-bit stores ahead of the deposit, coefficients in registers.  What the two share is in tma_common.cuh; the step's
+// arithmetic and the order of its sums are those of the multi-step kernel too, so the results are the same to the bit
+// whichever takes a step.  1e9 particles on
 // 256^3: 12.5 ms a step against 14.9 ms there; 6e7 on 128^3 9.0 against 9.9 ms for ten, the paper's physics 9.8
-// against 11.6 ms.  The cloud-in-cell deposit, bound by its adds, is faster there (10.4 against 13.6 ms at 2e7).
+// against 11.6 ms.  The cloud-in-cell deposit, bound by its adds, is faster there (9.6 against 13.6 ms at 2e7).
 // A unit of more particles than the tile's digit words take (the multi-step kernel flushes the tile in between) sends
 // its sums to the global accumulator.
 // The first step after a sort may also do that sort's payload gather (the GATHER instance): the sort

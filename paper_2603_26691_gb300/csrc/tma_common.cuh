@@ -68,9 +68,9 @@ struct TmaArgs {
   const float4* __restrict__ grec;    // GATHER: the records in the old order
   const uint32_t* __restrict__ ids_in;   // GATHER: ids in the old order
   uint32_t* __restrict__ ids_out;        // GATHER: ids in sorted order
-  int ngp, semi, sn, cic;             // physics variants (the PHYS instance): nearest grid point,
-  float re_coef;                      // semi-implicit Euler, Schiller-Naumann drag (Re = re_coef |u-v| d),
-                                      // cloud-in-cell deposit
+  int ngp, semi, sn, cic;             // physics variants (the PHYS instances): nearest grid point, semi-implicit Euler,
+  float re_coef;                      // Schiller-Naumann drag (Re = re_coef |u-v| d), cloud-in-cell deposit (the
+                                      // multi-step kernel's alone)
 };
 
 // de-interleave 3 bits per level (local x bit lowest)

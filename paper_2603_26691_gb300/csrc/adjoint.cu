@@ -203,11 +203,12 @@ __global__ void __launch_bounds__(kAdjThreads) adjoint_step_kernel(const AdjArgs
 //     or the segment ends: 24 global commits of three or four 64-bit reductions per stencil instead of per step,
 //     which bound the sweep.  These sums are exact, and the diameter's run on over the segments, so the gradients do
 //     not depend on how the steps are cut into segments.
-// About 55 FP64 instructions are left per particle and step, against 349.  2e6 particles on 64^3, 40 steps: 23.0 ms
-// against 44.4 ms step by step; of these some 16 ms are the sweep without the sums, and the sums and their commits take
-// about as much as each other.  (With products and sums of 64 bits, which kept fewer bits of small weights than FP64
-// does, 20.6 ms.)  16 warps per SM at 128 registers: 12 at 168 take 0.9 ms more.  The loop over the components that adds
-// the products is not unrolled: the kernel is as large as the instruction cache likes (unrolled 24.1 ms).
+// 69 FP64 instructions (109 operations) are left per particle and step in segments of 20, what is done once per segment
+// included, against 349 operations.  2e6 particles on 64^3, 40 steps: 21.9 ms against 44.4 ms step by step; of these some
+// 16 ms are the sweep without the sums, and the sums and their commits take about as much as each other.  (With products
+// and sums of 64 bits, which kept fewer bits of small weights than FP64 does, 20.6 ms.)  16 warps per SM at 128
+// registers: 12 at 168 take 0.9 ms more.  The loop over the components that adds the products is not unrolled: the kernel
+// is as large as the instruction cache likes (1.1 ms more unrolled).
 constexpr int kSegThreads = 128;
 // stencils in a warp up to which its lanes are summed before the commits at a segment's end (sorted particles,
 // 1e7 on 64^3: 22.9 ms with the line at 12 against 24.4 ms without sums across lanes; unsorted particles lie above

@@ -285,7 +285,7 @@ st_status st_couple_run(st_handle h, int nintervals, double dt) {
     double* slot = (double*)h->src_hist[h->couple_done % 4].p;
     ST_TRY(cuda_check(h, launch_acc_to_f64(h, slot, h->acc_E), "archive source"));
     ST_CUDA(h, cudaMemsetAsync(h->acc.p, 0, h->acc.bytes, h->stream));
-    ST_CUDA(h, reset_acc_counter(h));
+    ST_CUDA(h, reset_acc_counter(h, false));
     h->acc_empty = true;
     h->acc_load = 0.0;
     // the next interval runs in the new field (its max |u|, read back, sets the next exponent; the

@@ -556,7 +556,8 @@ static double deposits_per_cell(const st_ctx* h) {
 // Choose the fixed-point exponent so that a committed run at its bound maps to
 // at most 2^96 and the accumulated integer stays below 2^125.
 // For a launch of nsteps steps; digits: what it can add to one word (far: see launch_acc_maybe_normalize).
-static st_status prepare_accumulator(st_handle h, double dt, int nsteps, double digits, bool far, int* E_out) {
+static st_status prepare_accumulator(st_handle h, double dt, int nsteps, double digits, bool far, bool capturing,
+                                     int* E_out) {
   const double pi = 3.14159265358979323846;
   double gn = std::sqrt(h->g[0] * h->g[0] + h->g[1] * h->g[1] + h->g[2] * h->g[2]);
   double tau_max = h->rho_p * h->dmax * h->dmax / (18.0 * h->mu);
@@ -569,7 +570,7 @@ static st_status prepare_accumulator(st_handle h, double dt, int nsteps, double 
   if (!h->acc_empty && E < h->acc_E) {
     cudaError_t e = launch_rescale_acc(h, h->acc_E - E);
     ST_TRY(cuda_check(h, e, "rescale accumulator"));
-    ST_TRY(cuda_check(h, reset_acc_counter(h), "reset accumulator counter"));
+    ST_TRY(cuda_check(h, reset_acc_counter(h, capturing), "reset accumulator counter"));
     h->acc_load = std::ldexp(h->acc_load, E - h->acc_E);
   }
   if (h->acc_empty || E < h->acc_E) h->acc_E = E;
@@ -580,7 +581,7 @@ static st_status prepare_accumulator(st_handle h, double dt, int nsteps, double 
   while (h->acc_load + add > 0x1p125) {
     cudaError_t e = launch_rescale_acc(h, 1);
     ST_TRY(cuda_check(h, e, "rescale accumulator"));
-    ST_TRY(cuda_check(h, reset_acc_counter(h), "reset accumulator counter"));
+    ST_TRY(cuda_check(h, reset_acc_counter(h, capturing), "reset accumulator counter"));
     h->acc_E -= 1;
     E = h->acc_E;
     h->acc_load *= 0.5;
@@ -588,7 +589,7 @@ static st_status prepare_accumulator(st_handle h, double dt, int nsteps, double 
   }
   h->acc_load += add;
   h->acc_empty = false;
-  ST_TRY(cuda_check(h, launch_acc_maybe_normalize(h, digits, far), "normalise accumulator"));
+  ST_TRY(cuda_check(h, launch_acc_maybe_normalize(h, digits, far, capturing), "normalise accumulator"));
   *E_out = E;
   return ST_OK;
 }
@@ -642,7 +643,7 @@ st_status run_steps(st_ctx* h, int nsteps, double dt) {
                                tma ? 8.0 * ((double)h->np * m / 65536.0 + 2.0) +
                                          std::min(deposits_per_cell(h) * (double)h->np * m, (double)kFarFree * kFarCtas)
                                    : deposits_per_cell(h) * (double)h->np * m + 8.0,
-                               tma, &E));
+                               tma, capturing, &E));
     StepParams p;
     p.dt = dt;
     p.nsteps = m;
@@ -702,7 +703,7 @@ st_status st_get_sources(st_handle h, double* out, int reset, int on_device) {
   cudaError_t e = launch_acc_to_f64(h, dst, h->acc_E);
   if (e == cudaSuccess && !on_device) e = cudaMemcpyAsync(out, dst, bytes, cudaMemcpyDeviceToHost, h->stream);
   if (e == cudaSuccess && reset) e = cudaMemsetAsync(h->acc.p, 0, h->acc.bytes, h->stream);
-  if (e == cudaSuccess && reset) e = reset_acc_counter(h);
+  if (e == cudaSuccess && reset) e = reset_acc_counter(h, false);
   // the error flags' read waits for all of it
   const st_status fs = e == cudaSuccess ? check_flags(h) : ST_OK;
   dev_free(h, tmp);
@@ -994,7 +995,7 @@ st_status st_adjoint_forward(st_handle h, int nsteps, double dt, int checkpoint_
   F64State s = carve_f64(h->state.p, h->cap);
   double* ck = (double*)h->ckpt.p;
   // checkpoints written by the step kernel, several steps per launch (not by the general FP64 kernel)
-  const bool tape = mixed || fixed_step_supported(h);
+  const bool tape = mixed || fixed_step_supported(h), capturing = stream_capturing(h);
   for (int step = 0; step < nsteps;) {
     int m = 1;
     if (tape)
@@ -1010,7 +1011,7 @@ st_status st_adjoint_forward(st_handle h, int nsteps, double dt, int checkpoint_
       ST_TRY(cuda_check(h, e, "checkpoint"));
     }
     int E = 0;
-    ST_TRY(prepare_accumulator(h, dt, m, deposits_per_cell(h) * (double)h->np * m + 8.0, false, &E));
+    ST_TRY(prepare_accumulator(h, dt, m, deposits_per_cell(h) * (double)h->np * m + 8.0, false, capturing, &E));
     StepParams p;
     p.dt = dt;
     p.nsteps = m;

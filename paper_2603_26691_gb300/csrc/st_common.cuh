@@ -638,14 +638,15 @@ constexpr int kFarFree = 1 << 16, kFarCtas = 256;
 cudaError_t launch_step_mixed_tma(st_ctx* h, const StepParams& p, bool records, bool gather);  // step_mixed_tma.cu
 cudaError_t launch_step_mixed_tma_single(st_ctx* h, const StepParams& p, bool records, bool gather);  // step_mixed_tma_single.cu
 cudaError_t launch_rescale_acc(st_ctx* h, int shift);
-cudaError_t launch_normalize_acc(st_ctx* h);
+cudaError_t launch_normalize_acc(st_ctx* h);  // not under capture: its caller waits for the device
 // the particle steps of st_step (sort when due, accumulator bookkeeping, step kernel)
 st_status run_steps(st_ctx* h, int nsteps, double dt);
 // the carries propagated before a launch that could overflow a word (`add`: the digits it adds to one at most;
 // far: the sorted-step kernel, whose commits outside its tiles keep themselves below 2^60 and are not counted); the
 // rule and who keeps the count: acc_count.h
-cudaError_t launch_acc_maybe_normalize(st_ctx* h, double add, bool far);
-cudaError_t reset_acc_counter(st_ctx* h);
+// (capturing: the launches go into a graph; asked for once a call)
+cudaError_t launch_acc_maybe_normalize(st_ctx* h, double add, bool far, bool capturing);
+cudaError_t reset_acc_counter(st_ctx* h, bool capturing);
 bool stream_capturing(const st_ctx* h);   // the handle's stream is being captured into a graph
 constexpr size_t kAccCountOffset = 64;     // bytes into the flags buffer: AccDeviceCount
 constexpr size_t kFarFlagOffset = 84;      // int: the neighbourhood sort found a particle it cannot place

@@ -196,7 +196,8 @@ __global__ void __launch_bounds__(256) step_f64_kernel(const F64Args a) {
 //     the steps a particle stays in a cell and then over the warp's lanes of equal cell: exact, so the
 //     sources do not depend on the storage order or on how steps are split over launches.
 // 21 to 24 FP64 instructions are left per particle and step (2 to 3 per axis for the position and cell, 5 for the
-// motion and the impulse), against 190.  3e7 particles on 128^3, ten steps: 17.7 ms against 84.7 ms.
+// motion and the impulse; 59 in a launch of a single step, with what the diameter decides), against 134.  3e7 particles
+// on 128^3, ten steps: 17.7 ms against 84.7 ms.
 struct FixArgs {
   const double* in[6];              // position and velocity before the steps
   F64State s;                       // after them (the same arrays, or others); diameters

@@ -577,7 +577,7 @@ cudaError_t launch_normalize_acc(st_ctx* h) {
   normalize_kernel<<<grid_for(m), kThreads, 0, h->stream>>>((long long*)h->acc.p, m, nullptr);
   h->launches += 1;
   cudaError_t e = cudaGetLastError();
-  return e == cudaSuccess ? reset_acc_counter(h) : e;
+  return e == cudaSuccess ? reset_acc_counter(h, false) : e;
 }
 
 __global__ void acc_decide_kernel(AccDeviceCount* __restrict__ c, double base, double add) { acc_decide(*c, base, add); }
@@ -594,8 +594,8 @@ bool stream_capturing(const st_ctx* h) {
 
 static AccDeviceCount* device_count(st_ctx* h) { return (AccDeviceCount*)((char*)h->flags.p + kAccCountOffset); }
 
-cudaError_t launch_acc_maybe_normalize(st_ctx* h, double add, bool far) {
-  const AccCount::Action act = h->acc_count.launch(add, far, stream_capturing(h));
+cudaError_t launch_acc_maybe_normalize(st_ctx* h, double add, bool far, bool capturing) {
+  const AccCount::Action act = h->acc_count.launch(add, far, capturing);
   if (act == AccCount::kNothing) return cudaSuccess;
   const int* flag = nullptr;
   if (act == AccCount::kAskDevice) {
@@ -609,8 +609,8 @@ cudaError_t launch_acc_maybe_normalize(st_ctx* h, double add, bool far) {
   return cudaGetLastError();
 }
 
-cudaError_t reset_acc_counter(st_ctx* h) {
-  if (!h->acc_count.cleared(stream_capturing(h))) return cudaSuccess;
+cudaError_t reset_acc_counter(st_ctx* h, bool capturing) {
+  if (!h->acc_count.cleared(capturing)) return cudaSuccess;
   acc_cleared_kernel<<<1, 1, 0, h->stream>>>(device_count(h));
   h->launches += 1;
   return cudaGetLastError();

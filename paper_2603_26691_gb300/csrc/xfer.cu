@@ -145,7 +145,7 @@ st_status st_get_sources_async(st_handle h, double* out, int reset) {
   cudaError_t e = cudaStreamWaitEvent(h->stream, x->out_done[b], 0);
   if (e == cudaSuccess) e = launch_acc_to_f64(h, (double*)x->sstage[b].p, h->acc_E);
   if (e == cudaSuccess && reset) e = cudaMemsetAsync(h->acc.p, 0, h->acc.bytes, h->stream);
-  if (e == cudaSuccess && reset) e = reset_acc_counter(h);
+  if (e == cudaSuccess && reset) e = reset_acc_counter(h, stream_capturing(h));
   if (e == cudaSuccess) e = cudaEventRecord(x->ready[b], h->stream);
   // the download stream: the copy to the host
   if (e == cudaSuccess) e = cudaStreamWaitEvent(x->down, x->ready[b], 0);

@@ -35,18 +35,44 @@ METRIC = "particle-steps/s at 1e9 particles, % HBM roofline; mixed vs FP64 at fi
 UNIT = "particle-steps/s"
 # algorithmic bytes per particle-step of the step kernel (read + write of the particle state)
 STEP_BYTES = {"mixed_f32": 32 + 28, "mixed_bf16": 26 + 22, "fp64": 56 + 48}
+CSRC = os.path.join(ROOT, "paper_2603_26691_gb300", "csrc")
+
+
+def _source_hash(*files):
+    """SHA-256 over a kernel's source files: what was counted by ncu holds for this source alone."""
+    import hashlib
+
+    h = hashlib.sha256()
+    for name in files:
+        with open(os.path.join(CSRC, name), "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()
+
+
+# The kernels that the workloads time, and the source files their counters are keyed by.  Steps are taken one
+# at a time: a launch of one step of many particles has a kernel of its own.
+SINGLE_STEP = ("step_mixed_tma_single_kernel", "step_mixed_tma_single.cu", "tma_common.cuh")
+FEW_PARTICLES_STEP = ("step_mixed_tma_kernel", "step_mixed_tma.cu", "tma_common.cuh")
+SINGLE_STEP_PARTICLES = 1 << 23  # from this many particles on
+FP64_STEP = ("step_f64_fixed_kernel", "step_f64.cu", "fix_gather.cuh")
+ADJOINT = ("adjoint_segment_kernel", "adjoint.cu", "fix_gather.cuh")
+
+
+def _measured(table, kernel, *more):
+    """A counter of a kernel (name, source files ...), None once its source has changed."""
+    return table.get((_source_hash(*kernel[1:]), kernel[0], *more))
+
+
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per particle and launch of the sorted-step
-# kernel at the workload's density, keyed by the SHA-256 of the kernel's source file; a kernel whose
+# kernel at the workload's density, keyed by its source; a kernel whose
 # source has changed since has no measured traffic (null).  Counter captures run on small cases only
 # (a few GB on the device), so the figure is derived from two of them at 24 and 60 particles per cell
 # (128^3 / 5.0e7 and 64^3 / 1.6e7 particles): per particle the traffic is the state's bytes plus
 # per-unit costs (fluid tile, deposit-tile flush) divided by the density, and a small capture misses
 # the dirty lines still in L2 when the kernel ends.  Fitted: reads 32 + 120 / rho B, writes
 # 28 + 99 / rho B with ~60 MB left in L2; at the 1e9 workload's 59.6 particles per cell, 63.7 B.
-STEP_SOURCE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "paper_2603_26691_gb300", "csrc",
-                           "step_mixed_tma.cu")
 MEASURED_TRAFFIC = {
-    ("cc6fd6e7278a727c5c1b8648edf045fc9ea4547380736fa09847ca45e4fe51f8", "fourier256_mixed_1e9"): 63.7,
+    ("853407b0111e00bc100c6df9c21b21015257a11564f258da530f052adf7b4803", "step_mixed_tma_single_kernel", "fourier256_mixed_1e9"): 63.7,
 }
 
 
@@ -245,19 +271,17 @@ def timed_steps(sim, steps, dt, reorder_every, step_index0):
     return ev
 
 
-# FP64 operations per particle of one adjoint step launch (adjoint_step_kernel) and of one FP64
-# step launch, from ncu instruction counters (2 x DFMA + DADD + DMUL, thread instructions) on the
-# adjoint workload; keyed by the SHA-256 of the kernel source, absent (null) once it changes
+# FP64 operations per particle and step of the adjoint sweep and of FP64 steps taken one at a time, from ncu instruction
+# counters (2 x DFMA + DADD + DMUL, thread instructions) on the adjoint workload's and the FP64 run's particles; keyed
+# by the kernel's source, absent (null) once it changes.  Both kernels interpolate on integers, so the share of the FP64
+# rate is what is left of their FP64 work.
 MEASURED_FP64_OPS = {
-    # ncu instruction counters: 116 DFMA + 46.8 DADD + 70 DMUL per particle; FP64 pipe 79 % busy
-    # (the cell-deposit instance adjoint_step_kernel<false>)
-    ("745faef8cafcc409ab81adaf96843ca26e35db7c534e64437178455cdd04f368", "adjoint_step_kernel"): 348.8,
-    # step_f64_kernel: 56 DFMA + 59 DADD + 19 DMUL per particle (2e6 particles on 128^3)
-    ("8fc2e56686bddc20dfeca2e836f247c15b1f3655db751a7a9f10af9a572c8820", "step_f64_kernel"): 190.0,
+    ("cc842a956fe4aff8fd4e6f00bf6226a8a77543c73b943ee4255d09cbd7a6cd58", "adjoint_segment_kernel"): 108.8,  # segments of 20 steps: 39.4 DFMA + 10.3 DADD + 19.7 DMUL
+    ("308b8018d5472e24cb3e38a460f45cc4a4bdc0c4c6f6b085124c51f6514581eb", "step_f64_fixed_kernel"): 91.0,  # 32 DFMA + 10 DADD + 17 DMUL
 }
-MEASURED_FP64_PIPE = {("745faef8cafcc409ab81adaf96843ca26e35db7c534e64437178455cdd04f368", "adjoint_step_kernel"): 0.794,
-                      ("8fc2e56686bddc20dfeca2e836f247c15b1f3655db751a7a9f10af9a572c8820", "step_f64_kernel"): 0.858}
-F64_SOURCE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "paper_2603_26691_gb300", "csrc", "step_f64.cu")
+# sm__pipe_fp64_cycles_active over the same launches
+MEASURED_FP64_PIPE = {("cc842a956fe4aff8fd4e6f00bf6226a8a77543c73b943ee4255d09cbd7a6cd58", "adjoint_segment_kernel"): 0.426,
+                      ("308b8018d5472e24cb3e38a460f45cc4a4bdc0c4c6f6b085124c51f6514581eb", "step_f64_fixed_kernel"): 0.726}
 
 
 def fp64_peak(sim):
@@ -270,18 +294,14 @@ def fp64_peak(sim):
 
 def fp64_step_roofline(n, ms, peak=None, peak_kind=None):
     """The FP64 step kernel against the FP64 rate (its operation count from ncu, by source)."""
-    import hashlib
-
-    with open(F64_SOURCE, "rb") as f:
-        key = (hashlib.sha256(f.read()).hexdigest(), "step_f64_kernel")
-    ops = MEASURED_FP64_OPS.get(key)
+    ops = _measured(MEASURED_FP64_OPS, FP64_STEP)
     ach = ops * n / (ms * 1e-3) / 1e9 if ops else None
     peak = peak or FP64_NOMINAL_GFLOPS
     return {"bound": "alu", "unit": "GFLOP/s (FP64)", "fp64_ops_per_particle": ops, "achieved": ach,
             "peak": peak, "peak_kind": peak_kind or "nominal GB300 dense FP64",
-            "frac": ach / peak if ach else None, "fp64_pipe_busy_ncu": MEASURED_FP64_PIPE.get(key)}
-ADJOINT_SOURCE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "paper_2603_26691_gb300", "csrc",
-                              "adjoint.cu")
+            "frac": ach / peak if ach else None, "fp64_pipe_busy_ncu": _measured(MEASURED_FP64_PIPE, FP64_STEP)}
+
+
 FP64_NOMINAL_GFLOPS = 1250.0  # GB300 dense FP64, the nominal figure (no measured FP64 peak on this pool)
 
 
@@ -289,8 +309,6 @@ def run_adjoint(args, workload):
     """The adjoint workload: FP64 forward with checkpoints, then the backward sweep (recomputation of
     each segment and the adjoint step), for a loss on the time-summed source field.  One JSON line:
     forward+backward particle-steps/s, with the library's kernel timers."""
-    import hashlib
-
     import torch
 
     ws, rank, local = _dist()
@@ -335,18 +353,16 @@ def run_adjoint(args, workload):
     value = n * steps / (total_ms * 1e-3)
     adj_ms, adj_n = tm["adjoint"]
     stp_ms, stp_n = tm["step"]
-    with open(ADJOINT_SOURCE, "rb") as f:
-        src_hash = hashlib.sha256(f.read()).hexdigest()
-    ops = MEASURED_FP64_OPS.get((src_hash, "adjoint_step_kernel"))
+    ops = _measured(MEASURED_FP64_OPS, ADJOINT)
     adj_avg = adj_ms / max(adj_n, 1)
     achieved = ops * n / (adj_avg * 1e-3) / 1e9 if ops else None
     p64, p64_kind = fp64_peak(sim)
-    roofline = {"bound": "alu", "kernel": "adjoint_step_kernel", "unit": "GFLOP/s (FP64)", "peak": p64,
+    roofline = {"bound": "alu", "kernel": ADJOINT[0], "unit": "GFLOP/s (FP64)", "peak": p64,
                 "peak_kind": p64_kind, "achieved": achieved,
                 "frac": achieved / p64 if achieved else None, "traffic": None,
-                "fp64_ops_per_particle": ops, "launches": adj_n, "ms_per_launch": adj_avg,
-                "fp64_pipe_busy_ncu": MEASURED_FP64_PIPE.get((src_hash, "adjoint_step_kernel")),
-                "step_f64_kernel": {"launches": stp_n, "ms_per_launch": stp_ms / max(stp_n, 1)}}
+                "fp64_ops_per_particle": ops, "steps": adj_n, "ms_per_step": adj_avg,
+                "fp64_pipe_busy_ncu": _measured(MEASURED_FP64_PIPE, ADJOINT),
+                FP64_STEP[0]: {"steps": stp_n, "ms_per_step": stp_ms / max(stp_n, 1)}}
     # end to end through the public API with host buffers: lam from host memory, the gradients to host
     lam_h = lam.cpu().numpy()
     torch.cuda.synchronize()
@@ -375,8 +391,8 @@ def run_adjoint(args, workload):
     ids64 = sim.particles(host=False)[3].long()
     cf_ms, cb_ms = c0e.elapsed_time(c1e), c1e.elapsed_time(c2e)
     cic = {"forward_ms": cf_ms, "backward_ms": cb_ms, "particle_steps_per_s": n * steps / ((cf_ms + cb_ms) * 1e-3),
-           "adjoint_kernel_ms_per_launch": tmc["adjoint"][0] / max(tmc["adjoint"][1], 1),
-           "step_kernel_ms_per_launch": tmc["step"][0] / max(tmc["step"][1], 1)}
+           "adjoint_kernel_ms_per_step": tmc["adjoint"][0] / max(tmc["adjoint"][1], 1),
+           "step_kernel_ms_per_step": tmc["step"][0] / max(tmc["step"][1], 1)}
     sim.close()
     # the same workload on a mixed FP32-velocity handle: the FP32 adjoint (general mixed step forward,
     # FP32 reverse step), its gradients compared with the FP64 run's
@@ -410,8 +426,8 @@ def run_adjoint(args, workload):
     gd32_id[ids32] = gd32
     ff_ms, fb_ms = f0e.elapsed_time(f1e), f1e.elapsed_time(f2e)
     fp32 = {"forward_ms": ff_ms, "backward_ms": fb_ms, "particle_steps_per_s": n * steps / ((ff_ms + fb_ms) * 1e-3),
-            "adjoint_kernel_ms_per_launch": tmf["adjoint"][0] / max(tmf["adjoint"][1], 1),
-            "step_kernel_ms_per_launch": tmf["step"][0] / max(tmf["step"][1], 1),
+            "adjoint_kernel_ms_per_step": tmf["adjoint"][0] / max(tmf["adjoint"][1], 1),
+            "step_kernel_ms_per_step": tmf["step"][0] / max(tmf["step"][1], 1),
             "grad_alpha_rel_diff_to_fp64": abs(ga32 - ga) / abs(ga),
             "grad_U_rel_l2_diff_to_fp64": float((torch.linalg.vector_norm(gU32 - gU) / torch.linalg.vector_norm(gU)).item()),
             "grad_d_rel_l2_diff_to_fp64": float((torch.linalg.vector_norm(gd32_id - gd_id) / torch.linalg.vector_norm(gd)).item()),
@@ -769,14 +785,12 @@ def main():
     bytes_per_launch = STEP_BYTES[precision] * n
     achieved = bytes_per_launch / (step_avg * 1e-3) / 1e9
     traffic = None
+    kernel = FP64_STEP if precision == "fp64" else SINGLE_STEP if n >= SINGLE_STEP_PARTICLES else FEW_PARTICLES_STEP
     if precision != "fp64":
-        import hashlib
-
-        with open(STEP_SOURCE, "rb") as f:
-            m = MEASURED_TRAFFIC.get((hashlib.sha256(f.read()).hexdigest(), workload.name))
+        m = _measured(MEASURED_TRAFFIC, kernel, workload.name)
         if m is not None:
             traffic = m * n
-    kname = "step_f64_kernel" if precision == "fp64" else "step_mixed_tma_kernel (plain instance)"
+    kname = kernel[0] if precision == "fp64" else kernel[0] + " (plain instance)"
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                 "traffic": traffic,
                 # the same kernel's measured DRAM bytes (ncu, this source) at the measured rate
@@ -798,7 +812,7 @@ def main():
                                     if gat_ms else None}}
 
     if precision == "fp64":  # the FP64 step is bound by FP64 arithmetic, not by HBM
-        roofline = dict(fp64_step_roofline(n, step_avg, *fp64_peak(sim)), kernel="step_f64_kernel", launches=len(step_ms),
+        roofline = dict(fp64_step_roofline(n, step_avg, *fp64_peak(sim)), kernel=FP64_STEP[0], launches=len(step_ms),
                         step_kernel_ms=step_avg, hbm_frac_of_algorithmic=achieved / peak)
 
     # per-chunk bounding boxes of the sorted state (on demand: one read of cells and offsets)
@@ -925,7 +939,8 @@ def main():
             ms = sum(e1.elapsed_time(e2) for (e0, e1, e2, _) in ev) / len(ev)
             variants[name] = {"physics": ph, "step_kernel_ms": ms, "particle_steps_per_s": n / (ms * 1e-3),
                               "hbm_frac_of_algorithmic": STEP_BYTES[precision] * n / (ms * 1e-3) / 1e9 / peak,
-                              "kernel": "step_mixed_tma_kernel (physics instance)"}
+                              "kernel": (SINGLE_STEP if n >= SINGLE_STEP_PARTICLES and ph.get("deposit") != "cic"
+                                         else FEW_PARTICLES_STEP)[0] + " (physics instance)"}
         sim.set_physics()
     sim.close()
     del sim

@@ -525,9 +525,10 @@ st_status st_num_particles(st_handle h, int64_t* n) {
   return ST_OK;
 }
 
-static st_status reorder(st_handle h) {
+static st_status reorder(st_handle h, bool gather_now) {
   timer_begin(h, ST_TIMER_SORT, h->stream);
-  const st_status ss = sort_particles(h);
+  st_status ss = sort_particles(h);
+  if (ss == ST_OK && gather_now) ss = materialize_state(h);
   timer_end(h, ST_TIMER_SORT, h->stream);
   ST_TRY(ss);
   h->adj_ready = false;
@@ -538,10 +539,9 @@ static st_status reorder(st_handle h) {
 
 st_status st_reorder(st_handle h) {
   ST_TRY(check_handle(h));
-  ST_TRY(reorder(h));
   // the physics variants' steps after a sort that was asked for can be captured and replayed: the sort gathers at once
   // (in the step loop the step that gathers follows in the same call)
-  return default_physics(h) ? ST_OK : materialize_state(h);
+  return reorder(h, !default_physics(h));
 }
 
 // Contributions one particle can make to one cell in one step: one, except that the cloud-in-cell
@@ -609,7 +609,7 @@ st_status run_steps(st_ctx* h, int nsteps, double dt) {
   const bool capturing = stream_capturing(h);
   for (int s = 0; s < nsteps;) {
     if (h->np == 0) break;
-    if (h->reorder_every > 0 && (!h->sorted || h->steps_since_sort >= h->reorder_every)) ST_TRY(reorder(h));
+    if (h->reorder_every > 0 && (!h->sorted || h->steps_since_sort >= h->reorder_every)) ST_TRY(reorder(h, false));
     const bool tma = !h->micro_on && h->prec != ST_FP64 && h->sorted && tma_step_supported(h);
     // the field is frozen and particles do not act on each other, so a launch takes several steps where
     // its kernel can, up to the next sort
